@@ -440,7 +440,6 @@ __device__ __forceinline__ void pencil_group(const pencil_args &A, int64_t grp, 
     constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
     constexpr int NC = ws_consumers<N, EB>();
     static_assert(!WS || GM == GM_L2G, "the staged pipeline reads x through l2g");
-    static_assert(GM != GM_L2G_CG || std::is_same<T, S>::value, "the fused path is FP32 or FP64");
     static_assert(!(FL && (SP || WS || GM != GM_L2G)), "the element-major store is a plain-kernel mode");
     constexpr bool kReloadIds = GM != GM_SCAT && !KEEP_IDS && !FL && reload_ids<N>();
     using P = pad<N>;
@@ -482,8 +481,6 @@ __device__ __forceinline__ void pencil_group(const pencil_args &A, int64_t grp, 
                     if (g >= 0) v = __ldg(x + g);
                     else if (g < -1) v = __ldg(A.halo + (-2 - g));
                     U[P::at(p0, p1, k)] = to_c(v);
-                } else if constexpr (GM == GM_L2G_CG) {
-                    U[P::at(p0, p1, k)] = g >= 0 ? to_c(__ldcg(x + g)) : T(0);
                 } else {
                     U[P::at(p0, p1, k)] = g >= 0 ? to_c(__ldg(x + g)) : T(0);
                 }
@@ -723,6 +720,298 @@ __device__ __forceinline__ void pencil_element3(const pencil_args &A, int64_t e,
     __syncthreads();  // the buffers are reused by the next element
 }
 
+// ------------------------------------------------------------ split element
+// One element over the C thread blocks of a cluster (C = 1, 2, 4, ...): block
+// c owns the slabs k and N - k of the pairs k = c, c + C, ... (and, for odd n,
+// the middle slab goes to block half % C). Each block gathers the whole u; the
+// r- and s-lines of a slab, its metric step and its epilogue need that slab
+// only, and the t-lines are cut by output: a block forms the outputs of its
+// own slabs (a pair (k, N - k) is what one row of the even-odd split gives).
+// The one exchange is v_t, which every block stores into its peers' shared
+// memory. For a mesh with fewer elements than the GPU has room for, where one
+// element's own chain of loads and FP64 operations sets the time (12 K FP64
+// operations at N = 7, 5.7 us on one SM), this spreads it over C SMs, and its
+// 2 n ns + n^2 line tasks (ns slabs) over as many threads. Same arithmetic per
+// node as pencil_group, value for value.
+template <int N>
+struct split {
+    static constexpr int n = N + 1, n2 = n * n, n3 = n2 * n, half = n / 2;
+    static constexpr bool odd = (n & 1) != 0;
+    static constexpr int MAXT = 3 * n2 <= 256 ? (3 * n2 + 31) / 32 * 32 : 256;
+    // most slabs a block of a cluster of C owns
+    static __host__ __device__ constexpr int slabs(int C) { return 2 * ((half + C - 1) / C) + (odd ? 1 : 0); }
+    static __host__ __device__ constexpr size_t smem(int C) { return sizeof(T) * 2 * (size_t)(pad<N>::size + slabs(C) * pad<N>::ss); }
+    static int threads(int C)
+    {
+        const int t = (2 * slabs(C) * n + n2 + 31) / 32 * 32;
+        return t < MAXT ? t : MAXT;
+    }
+};
+
+// Time of one element's FP64 or double-float operations on one SM, in
+// microseconds: about 6 n + 15 operations per node (even-odd split), 4140 FP64
+// operations per microsecond and SM, double-float about 2.5 times as fast
+// (its N = 7 operator takes 4.4 ms where FP64 takes 12.2).
+template <int N>
+constexpr double element_us()
+{
+    return (N + 1.0) * (N + 1) * (N + 1) * (6.0 * (N + 1) + 15.0) /
+           (std::is_same<T, double>::value ? 4140.0 : 10000.0);
+}
+
+// Blocks per element, E elements on 152 SMs: the power of two for which the
+// largest block's share of the element plus 1.5 us per doubling (the exchange,
+// the shorter loops) is least, while every block has an SM of its own.
+// Measured, FP64 A x in us with C = 1 / 2 / 4: N = 7 and 27 elements 16.6 /
+// 12.8 / 13.2, 64 elements 17.1 / 13.3 / 14.5; N = 3, 27: 8.6 / 9.9 / 9.9;
+// N = 15, 27: 98 / 57 / 36; two blocks per SM gain nothing (N = 9, 125
+// elements: 30.0 / 31.2 / 43.6).
+template <int N>
+inline int cluster_blocks(int64_t E)
+{
+    int best = 1;
+    double cost = element_us<N>();
+    for (int C = 2; C <= 4 && E * C <= 152 && C <= split<N>::half; C *= 2) {
+        const double c = element_us<N>() * split<N>::slabs(C) / (N + 1) + 1.5 * (C == 2 ? 1 : 2);
+        if (c < cost) {
+            cost = c;
+            best = C;
+        }
+    }
+    return best;
+}
+
+// Blocks per element of the split kernel in place of the base block shape
+// (EB = 256 / n^2 elements a block), 0 for the base shape. FP64: when one
+// block per element (or a cluster) leaves the busiest SM at most 3/4 of the
+// base shape's elements, and at most 8 (more small blocks than that cost
+// more than they spread: N = 3, 1728 elements 18.7 -> 21.2 us). Measured, us
+// per A x, base -> split: N = 3, 64 elements 17.2 -> 10.3; N = 5, 125: 25.5 ->
+// 14.6; N = 7, 64: 35.5 -> 13.3, 343: 35.8 -> 31.1; N = 9, 27: 41.6 -> 19.0;
+// N = 15, 64: 90 -> 57. FP32 keeps the base shape (its arithmetic is a small
+// part of the time: N = 7, 64 elements 8.2 us either way, larger meshes lose).
+// Double-float: the same rule (N = 7, 64 elements 18.4 -> 12.5), and from N =
+// 11 on at every size: its 256 threads a block whatever n^2 is, without the
+// node ids, leave registers and shared memory for more warps than the base
+// shape (us on 24^3 elements, base -> split: N = 11 1535 -> 1186, 12 2555 ->
+// 1515, 13 2853 -> 2252, 14 3269 -> 2975; N = 15 6986 -> 4861 with one block
+// per element, one an SM for its shared memory, 3660 with two).
+template <int N>
+inline int split_blocks(int64_t E)
+{
+    if (std::is_same<T, float>::value || N == 1) return 0;
+    constexpr int n2 = (N + 1) * (N + 1), EB = n2 >= 256 ? 1 : 256 / n2;
+    const int C = cluster_blocks<N>(E);
+    if (C > 1) return C;
+    const int64_t q0 = ((E + EB - 1) / EB + 151) / 152 * EB, q = (E + 151) / 152;
+    if (4 * q <= 3 * q0 && q <= 8) return 1;
+    return !std::is_same<T, S>::value && N >= 11 ? (N == 15 ? 2 : 1) : 0;
+}
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// Address of this block's shared-memory object in block `rank` of the cluster.
+template <typename V>
+__device__ __forceinline__ V *peer(V *p, int rank)
+{
+    uint64_t a;
+    asm volatile("mapa.u64 %0, %1, %2;" : "=l"(a) : "l"(reinterpret_cast<uint64_t>(p)), "r"(rank));
+    return reinterpret_cast<V *>(a);
+}
+
+// line_st with the even-odd split, for the outputs of the pairs i = c, c + C,
+// ... (and the middle one) only.
+template <int N, bool TR, class F>
+__device__ __forceinline__ void line_part(T (&in)[N + 1], int c, int C, F &&store)
+{
+    constexpr int n = N + 1, o = off(N), h = hh(N), oh = offh(N), half = n / 2;
+    constexpr bool odd = (n & 1) != 0;
+    const T *M = TR ? c_Dt : c_D;
+    const T *Ec = TR ? c_Et : c_E;
+    const T *Oc = TR ? c_Ot : c_O;
+#pragma unroll
+    for (int m = 0; m < half; m++) {
+        const T u = in[m], v = in[N - m];
+        in[m] = u + v;
+        in[N - m] = u - v;
+    }
+    for (int i = c; i < half; i += C) {
+        T P = Ec[oh + i * h] * in[0];
+        T Q = Oc[oh + i * h] * in[N];
+#pragma unroll
+        for (int m = 1; m < half; m++) {
+            P = fma(Ec[oh + i * h + m], in[m], P);
+            Q = fma(Oc[oh + i * h + m], in[N - m], Q);
+        }
+        if constexpr (odd) P = fma(Ec[oh + i * h + half], in[half], P);
+        store(i, P + Q);
+        store(N - i, Q - P);
+    }
+    if constexpr (odd) {
+        if (c == half % C) {
+            T Q = M[o + half * n] * in[N];
+#pragma unroll
+            for (int m = 1; m < half; m++) Q = fma(M[o + half * n + m], in[N - m], Q);
+            store(half, Q);
+        }
+    }
+}
+
+// Element e by the C blocks of this cluster, this one being block c; sm holds
+// split<N>::smem(C) bytes. load(q, g) gives node q's value of u from its DOF
+// id g >= 0, id(q) the id itself. stop (null: never) points to one flag per
+// block of the cluster in shared memory, which the callers set in every peer
+// before the call: if one is set, all blocks of the cluster return false
+// after their first cluster barrier, nothing stored in a peer since. Every
+// thread of every block must call it.
+template <int N, class FI, class FL>
+__device__ __forceinline__ bool pencil_split(const pencil_args &A, int64_t e, int c, int C, T *sm,
+                                             hbacc::dot_acc<S> &acc, FI &&id, FL &&load, const int *stop = nullptr)
+{
+    using L = split<N>;
+    using P = pad<N>;
+    constexpr int n = L::n, n2 = L::n2, n3 = L::n3, half = L::half, rs = P::rs, ss = P::ss;
+    constexpr int NS = surf_count<N>();
+    constexpr int PRE = 2;  // nodes whose factors a thread loads before the contractions
+    const S *__restrict__ geo = A.geo + e * 7 * n3;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int np = c < half ? (half - c + C - 1) / C : 0;
+    const int ns = 2 * np + ((L::odd && c == half % C) ? 1 : 0);
+    auto slab = [&](int q) {  // the q-th slab of this block
+        const int p = c + C * (q >> 1);
+        return q < 2 * np ? ((q & 1) ? N - p : p) : half;
+    };
+    T *U = sm, *B3 = U + P::size, *B1 = B3 + P::size, *B2 = B1 + L::slabs(C) * ss;
+#pragma unroll 4
+    for (int q = tid; q < n3; q += nt) {
+        const int g = id(q);
+        U[(q / n2) * ss + (q / n) % n * rs + q % n] = g >= 0 ? to_c(load(q, g)) : T(0);
+    }
+    S G[PRE][6];
+#pragma unroll
+    for (int t = 0; t < PRE; t++) {
+        const int w = tid + t * nt;
+        if (w < ns * n2) {
+            const S *g = geo + slab(w / n2) * 7 * n2 + w % n2;
+#pragma unroll
+            for (int f = 0; f < 6; f++) G[t][f] = __ldcs(g + f * n2);
+        }
+    }
+    cluster_arrive();  // (waited for before the first store to a peer)
+    __syncthreads();
+    // lines: 2 ns n along r and s in the own slabs, then n^2 along t
+    const int nl = ns * n;
+    for (int w = tid; w < 2 * nl + n2; w += nt) {
+        T in[n];
+        if (w < 2 * nl) {
+            const bool s = w >= nl;
+            const int wl = s ? w - nl : w, q = wl / n, b = wl - q * n;
+            const int at = s ? b : b * rs, step = s ? rs : 1;
+            const T *src = U + slab(q) * ss + at;
+            T *dst = (s ? B2 : B1) + q * ss + at;
+#pragma unroll
+            for (int m = 0; m < n; m++) in[m] = src[m * step];
+            line_st<N, false, true>(in, [&](int m, T v) { dst[m * step] = v; });
+        } else {
+            const int b = w - 2 * nl, at = b / n * rs + b % n;
+#pragma unroll
+            for (int m = 0; m < n; m++) in[m] = U[m * ss + at];
+            line_part<N, false>(in, c, C, [&](int m, T v) { B3[m * ss + at] = v; });
+        }
+    }
+    __syncthreads();
+    cluster_wait();
+    if (stop) {
+        int any = 0;
+        for (int r = 0; r < C; r++) any |= stop[r];
+        if (any) return false;
+    }
+    auto metric = [&](int w, const S (&g)[6]) {
+        const int q = w / n2, a = w - q * n2, at = a / n * rs + a % n, own = q * ss + at, full = slab(q) * ss + at;
+        const T grr = to_c(g[0]), grs = to_c(g[1]), grt = to_c(g[2]), gss = to_c(g[3]), gst = to_c(g[4]),
+                gtt = to_c(g[5]);
+        const T ur = B1[own], us = B2[own], ut = B3[full];
+        B1[own] = fma(grt, ut, fma(grs, us, grr * ur));
+        B2[own] = fma(gst, ut, fma(gss, us, grs * ur));
+        const T vt = fma(gtt, ut, fma(gst, us, grt * ur));
+        B3[full] = vt;
+        for (int r = 1; r < C; r++) *peer(B3 + full, c + r < C ? c + r : c + r - C) = vt;
+    };
+#pragma unroll
+    for (int t = 0; t < PRE; t++)
+        if (tid + t * nt < ns * n2) metric(tid + t * nt, G[t]);
+    for (int w = tid + PRE * nt; w < ns * n2; w += nt) {
+        const S *g = geo + slab(w / n2) * 7 * n2 + w % n2;
+        S f[6];
+#pragma unroll
+        for (int q = 0; q < 6; q++) f[q] = __ldcs(g + q * n2);
+        metric(w, f);
+    }
+    cluster_arrive();
+    __syncthreads();
+    // D^T in place along the lines (each is read whole before it is written)
+    for (int w = tid; w < 2 * nl; w += nt) {
+        const bool s = w >= nl;
+        const int wl = s ? w - nl : w, q = wl / n, b = wl - q * n, step = s ? rs : 1;
+        T *dst = (s ? B2 : B1) + q * ss + (s ? b : b * rs);
+        T in[n];
+#pragma unroll
+        for (int m = 0; m < n; m++) in[m] = dst[m * step];
+        line_st<N, true, true>(in, [&](int m, T v) { dst[m * step] = v; });
+    }
+    cluster_wait();  // the peers' v_t is here
+    // the threads past the r- and s-lines first: the t-lines go to them
+    for (int w = (tid + nt - 2 * nl % nt) % nt; w < n2; w += nt) {
+        const int at = w / n * rs + w % n;
+        T in[n];
+#pragma unroll
+        for (int m = 0; m < n; m++) in[m] = B3[m * ss + at];
+        line_part<N, true>(in, c, C, [&](int m, T v) { B3[m * ss + at] = v; });
+    }
+    __syncthreads();
+    S *ys = A.ysurf + e * NS;
+    for (int w = tid; w < ns * n2; w += nt) {
+        const int q = w / n2, a = w - q * n2, k = slab(q), j = a / n, i = a - j * n;
+        const int own = q * ss + j * rs + i, full = k * ss + j * rs + i;
+        const T yc = B1[own] + B2[own] + B3[full];
+        if (k == 0) {
+            ys[a] = to_s(yc);
+        } else if (k == N) {
+            ys[n2 + a] = to_s(yc);
+        } else if (i == 0 || i == N || j == 0 || j == N) {
+            ys[2 * n2 + (k - 1) * 4 * N + ring_index<N>(i, j)] = to_s(yc);
+        } else {
+            const int gk = id(k * n2 + a);
+            const S xv = std::is_same<T, S>::value ? to_s(U[full]) : __ldg(A.x + gk);
+            const S jw = A.screen ? __ldg(geo + (k * 7 + 6) * n2 + a) : S(1);
+            S y = to_s(yc);
+            y += A.lambda * (jw * xv);
+            A.y[gk] = y;
+            acc.add(xv, y);
+        }
+    }
+    __syncthreads();  // the buffers are reused by the next element
+    return true;
+}
+
+// Grid: E * C blocks in clusters of C.
+template <int N>
+__global__ void __launch_bounds__(split<N>::MAXT) ax_split_kernel(const pencil_args A, int C)
+{
+    if (A.run && *A.run == 0) return;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    hbacc::dot_acc<S> acc;
+    const int64_t e = blockIdx.x / C;
+    const int32_t *__restrict__ lg = A.l2g + e * split<N>::n3;
+    const S *__restrict__ x = A.x;
+    pencil_split<N>(A, e, blockIdx.x % C, C, reinterpret_cast<T *>(smem_raw), acc,
+                    [&](int q) { return __ldg(lg + q); }, [&](int, int g) { return __ldg(x + g); });
+    if (A.partials) {
+        const double v = hbacc::block_sum(acc.value());
+        if (threadIdx.x == 0) A.partials[blockIdx.x] = v;
+    }
+}
+
 // ------------------------------------------------------------ WS kernel
 // Shared memory of a WS block: the four element buffers (T), then from
 // 128-byte boundaries the staged factors (S) and node map of one group.
@@ -828,7 +1117,7 @@ hb_status launch(const pencil_args &A, int eb_mode, cudaStream_t s, int64_t *nbl
     constexpr int n = N + 1, n2 = n * n;
     constexpr int EB1 = n2 >= 256 ? 1 : 256 / n2;
     if (A.E <= 0) return HB_OK;
-    static int attr_set[9][32] = {{0}};
+    static int attr_set[10][32] = {{0}};
     int dev = 0;
     HB_TRY_CUDA(cudaGetDevice(&dev));
     const bool sp = (eb_mode & 8) != 0;   // CSR-position surface store
@@ -903,6 +1192,32 @@ hb_status launch(const pencil_args &A, int eb_mode, cudaStream_t s, int64_t *nbl
             }
         }
 #endif
+        if constexpr (EO) {
+            const int C = which == 0 ? split_blocks<N>(A.E) : 0;
+            if (C > 0) {
+                auto kern = ax_split_kernel<N>;
+                if (dev >= 0 && dev < 32 && !attr_set[9][dev]) {
+                    HB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     (int)split<N>::smem(1)));
+                    attr_set[9][dev] = 1;
+                }
+                if (nblocks_out) *nblocks_out = A.E * C;
+                cudaLaunchConfig_t cfg = {};
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeClusterDimension;
+                at[0].val.clusterDim.x = C;
+                at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+                cfg.gridDim = dim3((unsigned)(A.E * C));
+                cfg.blockDim = dim3((unsigned)split<N>::threads(C));
+                cfg.dynamicSmemBytes = split<N>::smem(C);
+                cfg.stream = s;
+                cfg.attrs = at;
+                cfg.numAttrs = C > 1 ? 1 : 0;
+                hb_prof_scope prof("ax_local", s);
+                HB_TRY_CUDA(cudaLaunchKernelEx(&cfg, kern, A, C));
+                return HB_OK;
+            }
+        }
         return go(ax_pencil_kernel<N, EO, EB1>, EB1);
     }
 }

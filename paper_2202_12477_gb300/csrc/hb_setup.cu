@@ -871,9 +871,9 @@ extern "C" hb_status hb_mesh_create(const hb_mesh_desc *d, void *stream, hb_mesh
     {
         hb_status sst = build_surface_csr(m, s);
         if (sst != HB_OK) { hb_mesh_destroy(m); return sst; }
-        // one partial per element-kernel block (at most one block per element)
-        // one partial per element-kernel block: at most one block per element
-        m->n_ax_partials = E + 1;
+        // one partial per element-kernel block: at most two per element, or
+        // as many as there are SMs (a small mesh split over more)
+        m->n_ax_partials = 2 * E + 152;
         cudaError_t ae = hb_dev_alloc((void **)&m->ax_partials, sizeof(double) * m->n_ax_partials, s);
         if (ae != cudaSuccess) {
             hb_set_error("ax partials: %s", cudaGetErrorString(ae));

@@ -1,0 +1,46 @@
+"""The element kernel that spreads one element over a cluster of blocks (small
+FP64 and double-float meshes, double-float from N = 11 on): value for value
+the result of the other pencil variants, on one, two and four blocks per
+element, even and odd lines."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+from paper_2202_12477_gb300 import hb, inputs  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    hb.lib()
+
+
+# four blocks per element (few elements, high degree), two, one, the base shape
+@pytest.mark.parametrize("dims,N", [((1, 1, 1), 2), ((2, 1, 1), 15), ((3, 2, 1), 14), ((2, 2, 2), 11), ((5, 2, 4), 9),
+                                    ((4, 4, 4), 8), ((19, 2, 2), 7), ((7, 11, 1), 7), ((3, 3, 3), 3), ((5, 5, 5), 4),
+                                    ((6, 7, 8), 6), ((10, 9, 8), 5), ((8, 19, 1), 10), ((6, 5, 6), 13), ((3, 7, 8), 15),
+                                    ((7, 7, 7), 12)])
+@pytest.mark.parametrize("prec", [hb.HB_F64, hb.HB_F64X])
+def test_split_equals_other_variants(dims, N, prec):
+    m = hb.Mesh(*dims, N, perturb=0.15, seed=N, faces=0x15, fp32=False)
+    x = torch.from_numpy(inputs.random_vector(m.n_global, seed=N + 1)).cuda()
+    for screen, lam in [(0, 0.1), (1, 0.6)]:
+        y = {}
+        for v in (3, 67):
+            hb.hb_set_kernel_variant(m.handle, prec, v)
+            y[v] = m.apply_A(x, lam=lam, screen=screen, prec=prec).cpu().numpy()
+        assert np.array_equal(y[3], y[67])
+    # the partials of x.y (every block of a cluster has one) through CG: the
+    # same iterates as with the other variant, to the rounding of the sums
+    b = m.rhs(kind=0, seed=3)
+    hb.lib().hb_set_cg_fused(m.handle, 1)
+    xs = {}
+    for v in (3, 67):
+        hb.hb_set_kernel_variant(m.handle, prec, v)
+        xs[v] = m.cg(b, lam=0.5, max_it=12, prec=prec)[0].cpu().numpy()
+    assert np.linalg.norm(xs[3] - xs[67]) <= 1e-12 * np.linalg.norm(xs[67])
+    m.close()
