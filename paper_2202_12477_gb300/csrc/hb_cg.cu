@@ -735,7 +735,7 @@ extern "C" hb_status hb_cg_solve(const hb_mesh *mc, const hb_cg_opts *o, const d
                                                        m->counters + 2, st);
         HB_CHECK_LAUNCH();
         if (use_fused_cg(m, o)) {
-            rs = hb_cg_fused_run(m, o->screen, o->lambda, x, r, p, Ap, st, s);
+            rs = hb_cg_fused_run(m, o->screen, o->lambda, x, r, p, z, Ap, st, s);
             if (rs != HB_OK) return rs;
             HB_TRY_CUDA(cudaMemcpyAsync(m->state_host, st, sizeof(hb_cg_state), cudaMemcpyDeviceToHost, s));
             HB_TRY_CUDA(cudaStreamSynchronize(s));

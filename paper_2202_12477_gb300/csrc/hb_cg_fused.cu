@@ -2,17 +2,23 @@
 // cooperative kernel. On a mesh of a few dozen elements the element kernel
 // itself needs a few microseconds of FP64 work, and launching the four
 // kernels of an iteration costs more than that; here the phases of an
-// iteration are separated by grid-wide barriers instead of launches:
-//   A p (one element per block, its three line directions at once)
-//   | Z^T on surface DOFs, p.Ap block partials
-//   | every block sums the partials in index order -> alpha; r -= alpha Ap,
-//     r.r block partials
-//   | every block sums them -> beta, stopping test; x += alpha p, p = r + beta p
-// Every block computes alpha and beta itself from the same partials in the
-// same order, so all blocks take the same decisions (no broadcast needed).
-// The barriers are bounded: a block that waits more than about a second
-// records bit 1 in the mesh's error word and every block then leaves the
-// iteration loop (the host reports HB_ERR_TIMEOUT).
+// iteration are separated by three grid-wide waits instead of launches:
+//   x += alpha p, p = r + beta p (each DOF by its owner), and A p by element
+//     (pencil_split, over a cluster of C blocks: each node forms its p from r
+//     and the old p itself, with the owner's arithmetic, so no wait lies
+//     between; p has two buffers)
+//   | Z^T on surface DOFs, p.Ap
+//   | r -= alpha Ap, r.r
+//   | beta, stopping test
+// Every block sums the block partials itself in the same fixed order, so all
+// blocks compute the same alpha and beta and take the same decisions (no
+// broadcast). The waits are bounded: a block that waits more than about a
+// second records bit 1 in the mesh's error word and every block then leaves
+// the iteration loop (the host reports HB_ERR_TIMEOUT).
+// Measured, us per iteration (with four waits, the barrier's arrival returning
+// a value, one block per element -> this form): 4x4x4 elements at N = 7 27.6
+// -> 17.8, at N = 3 16.7 -> 14.5. At N = 7 a wait takes 2.2 us, the element
+// phase 6.9 (2.9 of it FP64 operations), the vector phases 1.1 each.
 #include "hb_internal.h"
 #define HB_AX2_T double
 #include "hb_ax2.cuh"
@@ -27,35 +33,39 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
     return v;
 }
 
-// Grid-wide barrier of a cooperative launch (every block resident at once)
-// on one counter word: block 0 adds 2^31 - (nb - 1) and every other block 1,
-// so the counter's top bit flips exactly when the last of the nb blocks has
-// arrived, once per barrier, with no reset. Thread 0 of each block arrives
-// after a fence (its block's writes are then visible to the others) and
-// polls until the top bit differs from the one its own atomic saw, for at
-// most hb2::kWaitNs of wall time. Returns true in every thread of the block
-// if this block gave up (the caller must then stop: the blocks still waiting
-// give up in turn, so the launch ends).
-__device__ bool grid_barrier(unsigned *bar, unsigned nb, unsigned *err)
+// Grid-wide barrier number seq (1, 2, ...) of a cooperative launch (every
+// block resident at once) on one counter word, zero at launch: block 0 adds
+// 2^31 - (nb - 1) and every other block 1, so the counter's top bit flips
+// exactly when the last of the nb blocks has arrived, once per barrier, with
+// no reset; after barrier seq it equals seq's lowest bit, so the arrival needs
+// no answer (a reduction without a return value). Thread 0 of each block
+// arrives with release order (its block's writes are then visible to the
+// others) and polls for at most hb2::kWaitNs of wall time. Returns true in
+// every thread of the block if this block gave up (the caller must then stop:
+// the blocks still waiting give up in turn, so the launch ends).
+// (Blocks publishing their partial sums in flagged slots that all others poll
+// was measured too: 20.0 -> 23.8 us per iteration on 128 blocks, 20.3 -> 29.0
+// on 216: the polls of nb^2 slots collide in L2.)
+__device__ bool grid_barrier(unsigned *bar, unsigned nb, unsigned seq, unsigned *err)
 {
     __shared__ int s_fail;
     __syncthreads();
     if (threadIdx.x == 0) {
         int fail = 0;
-        const unsigned add = blockIdx.x == 0 ? 0x80000000u - (nb - 1u) : 1u;
-        __threadfence();
-        const unsigned old = atomicAdd(bar, add);
-        if (((old ^ ld_acquire(bar)) & 0x80000000u) == 0) {
-            const unsigned long long t0 = hb2::wall_ns();
-            while (((old ^ ld_acquire(bar)) & 0x80000000u) == 0) {
-                if (hb2::wall_ns() - t0 > hb2::kWaitNs) {
-                    atomicOr(err, 2u);
-                    fail = 1;
-                    break;
-                }
+        const unsigned add = blockIdx.x == 0 ? 0x80000000u - (nb - 1u) : 1u, want = seq << 31;
+        asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(bar), "r"(add) : "memory");
+        unsigned long long t0 = 0;
+        for (unsigned t = 1; ((ld_acquire(bar) ^ want) & 0x80000000u) != 0; t++) {
+            if (t & 63u) continue;
+            const unsigned long long now = hb2::wall_ns();
+            if (t0 == 0) {
+                t0 = now;
+            } else if (now - t0 > hb2::kWaitNs) {
+                atomicOr(err, 2u);
+                fail = 1;
+                break;
             }
         }
-        __threadfence();
         s_fail = fail;
     }
     __syncthreads();
@@ -68,104 +78,151 @@ struct fused_args {
     const int32_t *srow_g, *srowptr, *scols;
     const double *mdiag;
     double *ysurf;
-    double *x, *r, *p, *Ap;
+    double *x, *r, *p, *p2, *Ap;  // p, p2: the two buffers of p (p holds p_0)
     int64_t E, n_global, nsr;
     double lambda;
     int screen;
-    double *part_a, *part_b;  // [gridDim.x] block partials (two, alternating)
+    double *part;             // [2][HB_RED_BLOCKS] block partials (two sets, alternating)
     hb_cg_state *st;          // in: rr, tol2, max_it, run; out: final state
     unsigned *bar;            // grid barrier counter (zero at launch)
-    unsigned *err;            // error word (bit 1: a barrier wait gave up)
+    unsigned *err;            // error word (bit 1: a wait gave up)
 };
 
-// Block size for degree N: the three thread groups of pencil_element3, at
-// least 256 threads for the vector phases.
+// Grid-wide wait and sum: every block passes its v (read in thread 0), all of
+// them get the sum over the blocks, added in a fixed order (thread t takes
+// partials t, t + blockDim, ..., then a shuffle tree), and see what every
+// other block wrote to memory before its call. seq counts the waits (a block
+// is at most one ahead of another, so two sets of partials alternate). False
+// in every thread if the wait ran out.
+__device__ bool grid_wait_sum(const fused_args &F, double v, unsigned seq, double &sum)
+{
+    __shared__ double s_w[32];
+    const int nb = gridDim.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    double *part = F.part + (seq & 1u) * HB_RED_BLOCKS;
+    if (threadIdx.x == 0) part[blockIdx.x] = v;
+    if (grid_barrier(F.bar, nb, seq, F.err)) return false;
+    double t = 0.0;
+    for (int q = threadIdx.x; q < nb; q += blockDim.x) t += __ldcg(part + q);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) s_w[wid] = t;
+    __syncthreads();
+    // every warp adds the warps' sums itself (in the same order); s_w is
+    // rewritten only after the next barrier
+    double u = lane < nw ? s_w[lane] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+    sum = u;
+    return true;
+}
+
+// Block size for degree N: the tasks of pencil_split, at least 256 threads
+// for the vector phases.
 template <int N>
 constexpr int fused_threads()
 {
-    constexpr int t = 3 * (N + 1) * (N + 1);
-    return t < 256 ? 256 : (t + 31) / 32 * 32;
+    return hb2::split<N>::MAXT < 256 ? 256 : hb2::split<N>::MAXT;
 }
-
-__device__ __forceinline__ double sum_partials(const double *p, int nb)
-{
-    // every block adds the same values in the same order: thread t takes
-    // partials t, t + blockDim, ..., then a fixed shuffle tree (a serial sum
-    // by one thread waits on one L2 round trip per partial)
-    __shared__ double s_w[32];
-    __shared__ double s_tot;
-    double t = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) t += __ldcg(p + b);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) s_w[wid] = t;
-    __syncthreads();
-    if (wid == 0) {
-        double u = lane < nw ? s_w[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) u += __shfl_down_sync(0xffffffffu, u, o);
-        if (lane == 0) s_tot = u;
-    }
-    __syncthreads();
-    const double v = s_tot;
-    __syncthreads();
-    return v;
-}
-
+// Shared memory: pencil_split's buffers and the element's node ids.
 template <int N>
-__global__ void __launch_bounds__(fused_threads<N>()) cg_fused_kernel(const fused_args F)
+size_t fused_smem(int C)
+{
+    return hb2::split<N>::smem(C) + sizeof(int32_t) * hb2::split<N>::n3;
+}
+
+// Grid: E * C blocks in clusters of C (hb2::cluster_blocks), all resident at
+// once.
+template <int N>
+__global__ void __launch_bounds__(fused_threads<N>()) cg_fused_kernel(const fused_args F, int C)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ int s_stop[8];  // one per block of the cluster (pencil_split)
     double *sm = reinterpret_cast<double *>(smem_raw);
+    int32_t *ids = reinterpret_cast<int32_t *>(smem_raw + hb2::split<N>::smem(C));
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gthreads = (int64_t)gridDim.x * blockDim.x;
-    const int nb = (int)gridDim.x;
+    const int64_t e = blockIdx.x / C;
+    const int c = blockIdx.x % C;
 
     double rr = F.st->rr;
     const double tol2 = F.st->tol2;
     const int max_it = F.st->max_it;
-    int run = F.st->run;
+    int stop = F.st->run == 0;
     int it = 0;
+    unsigned seq = 0;
     int status = HB_OK;
     double alpha = 0.0, beta = 0.0, pAp = 0.0;
+    double *pold = F.p2, *p = F.p;  // p_{j-1} and p_j
 
-    hb2::pencil_args A{F.p, F.l2g, F.geo, F.ysurf, F.Ap, F.E, nullptr, F.lambda, F.screen, nullptr};
-    // one element per block, its three line directions contracted at once
-    // (pencil_element3): on a small mesh the element's latency sets the time;
-    // the other threads of the block join the vector phases
-    const int64_t ngroups = F.E;
+    for (int q = threadIdx.x; q < hb2::split<N>::n3; q += blockDim.x) ids[q] = F.l2g[e * hb2::split<N>::n3 + q];
+    // this thread's first surface row (its only one on the smallest meshes)
+    int row_g = -1, row_a = 0, row_z = 0, row_c[4] = {0, 0, 0, 0};
+    if (gtid < F.nsr) {
+        row_g = F.srow_g[gtid];
+        row_a = F.srowptr[gtid];
+        row_z = F.srowptr[gtid + 1];
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+            if (row_a + q < row_z) row_c[q] = F.scols[row_a + q];
+    }
+    // the peers' shared memory is there from here on, and stays until all
+    // blocks of the cluster have agreed to leave (the return of pencil_split)
+    hb2::cluster_arrive();
+    hb2::cluster_wait();
+    __syncthreads();
 
-    while (run) {
-        // A p: element kernel (interior DOFs finished, surface values to ysurf)
+    hb2::pencil_args A{nullptr, F.l2g, F.geo, F.ysurf, F.Ap, F.E, nullptr, F.lambda, F.screen, nullptr};
+    for (;;) {
+        // x += alpha p_{j-1}, p_j = r + beta p_{j-1} (j > 0) at this thread's DOFs
+        // (data written by other blocks in this launch is read through L2)
+        if (it > 0 && status == HB_OK)
+            for (int64_t i = gtid; i < F.n_global; i += gthreads) {
+                const double po = __ldcg(pold + i);
+                F.x[i] += alpha * po;
+                if (!stop) p[i] = fma(beta, po, F.r[i]);
+            }
+        if (threadIdx.x < C) *hb2::peer(&s_stop[c], threadIdx.x) = stop;
+        // A p: interior DOFs finished, surface values to ysurf
         hbacc::dot_acc<double> acc;
-        for (int64_t g = blockIdx.x; g < ngroups; g += gridDim.x)
-            hb2::pencil_element3<N, hb2::GM_L2G_CG>(A, g, sm, acc);
-        if (grid_barrier(F.bar, nb, F.err)) {
-            status = HB_ERR_TIMEOUT;
+        const bool first = it == 0;
+        if (!hb2::pencil_split<N>(
+                A, e, c, C, sm, acc, [&](int q) { return ids[q]; },
+                [&](int, int g) { return first ? __ldcg(p + g) : fma(beta, __ldcg(pold + g), __ldcg(F.r + g)); },
+                s_stop))
             break;
+        if (grid_barrier(F.bar, gridDim.x, ++seq, F.err)) {
+            status = HB_ERR_TIMEOUT;
+            stop = 1;
+            continue;
         }
         // Z^T on the surface DOFs
-        // (data written by other blocks in this launch is read through L2)
-        for (int64_t rI = gtid; rI < F.nsr; rI += gthreads) {
-            const int g = F.srow_g[rI];
+        auto row = [&](int g, int a, int z, const int (&c4)[4]) {
             double t = 0.0;
-            for (int q = F.srowptr[rI]; q < F.srowptr[rI + 1]; q++) t += __ldcg(F.ysurf + F.scols[q]);
-            const double xv = __ldcg(F.p + g);
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                if (a + q < z) t += __ldcg(F.ysurf + c4[q]);
+            for (int q = a + 4; q < z; q++) t += __ldcg(F.ysurf + F.scols[q]);
+            const double xv = __ldcg(p + g);
             t += F.screen ? F.lambda * (F.mdiag[g] * xv) : F.lambda * xv;
             F.Ap[g] = t;
             acc.add(xv, t);
+        };
+        if (row_g >= 0) row(row_g, row_a, row_z, row_c);
+        for (int64_t rI = gtid + gthreads; rI < F.nsr; rI += gthreads) {
+            const int a = F.srowptr[rI], z = F.srowptr[rI + 1];
+            int c4[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) c4[q] = a + q < z ? F.scols[a + q] : 0;
+            row(F.srow_g[rI], a, z, c4);
         }
-        {
-            const double v = hbacc::block_sum(acc.value());
-            if (threadIdx.x == 0) F.part_a[blockIdx.x] = v;
-        }
-        if (grid_barrier(F.bar, nb, F.err)) {
+        double v = hbacc::block_sum(acc.value());
+        if (!grid_wait_sum(F, v, ++seq, pAp)) {
             status = HB_ERR_TIMEOUT;
-            break;
+            stop = 1;
+            continue;
         }
-        pAp = sum_partials(F.part_a, nb);
         if (!(pAp > 0.0) || !isfinite(pAp)) {
-            status = HB_ERR_BREAKDOWN;
-            break;  // every block takes the same branch
+            status = HB_ERR_BREAKDOWN;  // every block takes the same branch
+            stop = 1;
+            continue;
         }
         alpha = rr / pAp;
         // r -= alpha Ap and r.r
@@ -175,29 +232,20 @@ __global__ void __launch_bounds__(fused_threads<N>()) cg_fused_kernel(const fuse
             F.r[i] = ri;
             racc.add(ri, ri);
         }
-        {
-            const double v = hbacc::block_sum(racc.value());
-            if (threadIdx.x == 0) F.part_b[blockIdx.x] = v;
-        }
-        if (grid_barrier(F.bar, nb, F.err)) {
+        v = hbacc::block_sum(racc.value());
+        double rr_new;
+        if (!grid_wait_sum(F, v, ++seq, rr_new)) {
             status = HB_ERR_TIMEOUT;
-            break;
+            stop = 1;
+            continue;
         }
-        const double rr_new = sum_partials(F.part_b, nb);
         beta = rr_new / rr;
         rr = rr_new;
         it++;
-        run = (it < max_it && rr_new > tol2) ? 1 : 0;
-        // x += alpha p with the old p, then p = r + beta p
-        for (int64_t i = gtid; i < F.n_global; i += gthreads) {
-            const double pi = __ldcg(F.p + i);
-            F.x[i] += alpha * pi;
-            F.p[i] = F.r[i] + beta * pi;
-        }
-        if (grid_barrier(F.bar, nb, F.err)) {
-            status = HB_ERR_TIMEOUT;
-            break;
-        }
+        stop = !(it < max_it && rr_new > tol2);
+        double *const o = pold;
+        pold = p;
+        p = o;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         hb_cg_state *st = F.st;
@@ -213,38 +261,65 @@ __global__ void __launch_bounds__(fused_threads<N>()) cg_fused_kernel(const fuse
     }
 }
 
+// Blocks of a cluster of C that are resident at once (0: cannot launch).
 template <int N>
-hb_status launch_fused(const fused_args &F, int blocks_cap, cudaStream_t s, bool probe_only, int *grid_out)
+hb_status fused_resident(int C, cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&at)[2], int64_t *blocks)
 {
-    constexpr int threads = fused_threads<N>();
-    const size_t smem = sizeof(double) * 4 * (size_t)hb2::pad<N>::size;
     auto kern = cg_fused_kernel<N>;
     static int attr_set[32] = {0};
     int dev = 0;
     HB_TRY_CUDA(cudaGetDevice(&dev));
     if (dev >= 0 && dev < 32 && !attr_set[dev]) {
-        HB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        HB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused_smem<N>(1)));
         attr_set[dev] = 1;
     }
-    int per_sm = 0, sms = 0;
-    HB_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
-    HB_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int64_t ngroups = F.E;
-    int64_t grid = (int64_t)per_sm * sms;  // every block resident at once (cooperative launch)
-    if (grid > ngroups) grid = ngroups;
-    if (grid > blocks_cap) grid = blocks_cap;
-    if (grid < 1) grid = 1;
-    if (grid_out) *grid_out = (int)grid;
-    if (probe_only) return per_sm > 0 ? HB_OK : HB_ERR_ARG;
-    void *args[] = {(void *)&F};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeCooperative;
+    at[1].val.cooperative = 1;
+    cfg.gridDim = dim3((unsigned)C);
+    cfg.blockDim = dim3(fused_threads<N>());
+    cfg.dynamicSmemBytes = fused_smem<N>(C);
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    if (C == 1) {
+        int per_sm = 0, sms = 0;
+        HB_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, fused_threads<N>(), fused_smem<N>(1)));
+        HB_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        *blocks = (int64_t)per_sm * sms;
+    } else {
+        int clusters = 0;
+        HB_TRY_CUDA(cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg));
+        *blocks = (int64_t)clusters * C;
+    }
+    return HB_OK;
+}
+
+template <int N>
+hb_status launch_fused(fused_args &F, cudaStream_t s, bool probe_only, int64_t *capacity)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2];
+    int64_t blocks = 0;
+    if (probe_only) return fused_resident<N>(1, cfg, at, capacity);
+    int C = hb2::cluster_blocks<N>(F.E);
+    for (;; C /= 2) {
+        hb_status r = fused_resident<N>(C, cfg, at, &blocks);
+        if (r != HB_OK) return r;
+        if (F.E * C <= blocks && F.E * C <= HB_RED_BLOCKS) break;
+        if (C == 1) { hb_set_error("fused CG: %lld elements do not fit", (long long)F.E); return HB_ERR_ARG; }
+    }
+    cfg.gridDim = dim3((unsigned)(F.E * C));
+    cfg.stream = s;
     hb_prof_scope prof("cg_fused", s);
-    HB_TRY_CUDA(cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)grid), dim3(threads), args, smem, s));
+    HB_TRY_CUDA(cudaLaunchKernelEx(&cfg, cg_fused_kernel<N>, (const fused_args)F, C));
     return HB_OK;
 }
 
 // Self-test of the bounded barrier: it waits for one block more than were
 // launched, so every block gives up and sets bit 1 of *err.
-__global__ void barrier_timeout_kernel(unsigned *bar, unsigned *err) { grid_barrier(bar, gridDim.x + 1, err); }
+__global__ void barrier_timeout_kernel(unsigned *bar, unsigned *err) { grid_barrier(bar, gridDim.x + 1, 1u, err); }
 
 }  // namespace
 
@@ -267,25 +342,24 @@ int hb_cg_fused_capacity(int N)
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return 0;
     fused_args F{};
-    F.E = 1 << 30;
-    int grid = 0;
+    int64_t cap = 0;
     hb_status st;
     switch (N) {
 #define HB_CASE(NN) \
-    case NN: st = launch_fused<NN>(F, 1 << 30, nullptr, true, &grid); break;
+    case NN: st = launch_fused<NN>(F, nullptr, true, &cap); break;
         HB_CASE(1) HB_CASE(2) HB_CASE(3) HB_CASE(4) HB_CASE(5) HB_CASE(6) HB_CASE(7) HB_CASE(8)
         HB_CASE(9) HB_CASE(10) HB_CASE(11) HB_CASE(12) HB_CASE(13) HB_CASE(14) HB_CASE(15)
 #undef HB_CASE
     default: return 0;
     }
-    return st == HB_OK ? grid : 0;
+    return st == HB_OK ? (int)(cap < HB_RED_BLOCKS ? cap : HB_RED_BLOCKS) : 0;
 }
 
 // max_it iterations (or until the state's tolerance) of Algorithm 1 on
-// (x, r, p, Ap) in one cooperative launch; the state must hold rr, tol2,
+// (x, r, p, Ap; p2: a second buffer for p) in one cooperative launch; the state must hold rr, tol2,
 // max_it and run as cg_init leaves them.
-hb_status hb_cg_fused_run(const hb_mesh *m, int screen, double lambda, double *x, double *r, double *p, double *Ap,
-                          hb_cg_state *st, cudaStream_t s)
+hb_status hb_cg_fused_run(const hb_mesh *m, int screen, double lambda, double *x, double *r, double *p, double *p2,
+                          double *Ap, hb_cg_state *st, cudaStream_t s)
 {
     fused_args F{};
     F.l2g = m->l2g;
@@ -298,21 +372,21 @@ hb_status hb_cg_fused_run(const hb_mesh *m, int screen, double lambda, double *x
     F.x = x;
     F.r = r;
     F.p = p;
+    F.p2 = p2;
     F.Ap = Ap;
     F.E = m->E;
     F.n_global = m->n_global;
     F.nsr = m->nsr;
     F.lambda = lambda;
     F.screen = screen;
-    F.part_a = m->partials;
-    F.part_b = m->partials + HB_RED_BLOCKS;
+    F.part = m->partials;
     F.st = st;
     F.bar = m->counters + 4;
     F.err = m->counters + 7;
     HB_TRY_CUDA(cudaMemsetAsync(F.bar, 0, sizeof(unsigned), s));
     switch (m->N) {
 #define HB_CASE(NN) \
-    case NN: return launch_fused<NN>(F, HB_RED_BLOCKS, s, false, nullptr);
+    case NN: return launch_fused<NN>(F, s, false, nullptr);
         HB_CASE(1) HB_CASE(2) HB_CASE(3) HB_CASE(4) HB_CASE(5) HB_CASE(6) HB_CASE(7) HB_CASE(8)
         HB_CASE(9) HB_CASE(10) HB_CASE(11) HB_CASE(12) HB_CASE(13) HB_CASE(14) HB_CASE(15)
 #undef HB_CASE

@@ -82,7 +82,7 @@ struct hb_mesh {
     void *yL;           // [n_local] doubles: element-local operator output
     // workspace for reductions and CG
     double *partials;   // [HB_RED_MAXV * HB_RED_BLOCKS]
-    unsigned *counters; // [4]
+    unsigned *counters; // [8]
     hb_cg_state *state; // device CG states [4]: 0 outer/FP64, 1 inner/dot
     hb_cg_state *state_host;  // pinned mirror
     void *cg_vec;       // r, p, Ap (FP64) then FP32 inner vectors
@@ -221,8 +221,8 @@ hb_status hb_mesh_ensure_spos(hb_mesh *m, cudaStream_t s);
 // launch can keep resident for degree N (0: not available), and the run.
 int hb_cg_fused_capacity(int N);
 hb_status hb_cg_fused_upload(const double *D_all);
-hb_status hb_cg_fused_run(const hb_mesh *m, int screen, double lambda, double *x, double *r, double *p, double *Ap,
-                          hb_cg_state *st, cudaStream_t s);
+hb_status hb_cg_fused_run(const hb_mesh *m, int screen, double lambda, double *x, double *r, double *p, double *p2,
+                          double *Ap, hb_cg_state *st, cudaStream_t s);
 // Self-tests of the bounded device waits (hb_selftest_wait): the staged
 // pipeline's mbarrier wait (sets bit 0 of *err) and the fused CG's grid
 // barrier (bar: a zeroed word; sets bit 1).

@@ -1,7 +1,8 @@
 """The element kernel that spreads one element over a cluster of blocks (small
 FP64 and double-float meshes, double-float from N = 11 on): value for value
 the result of the other pencil variants, on one, two and four blocks per
-element, even and odd lines."""
+element, even and odd lines; and the fused CG built on it against the launched
+kernels."""
 import numpy as np
 import pytest
 
@@ -43,4 +44,28 @@ def test_split_equals_other_variants(dims, N, prec):
         hb.hb_set_kernel_variant(m.handle, prec, v)
         xs[v] = m.cg(b, lam=0.5, max_it=12, prec=prec)[0].cpu().numpy()
     assert np.linalg.norm(xs[3] - xs[67]) <= 1e-12 * np.linalg.norm(xs[67])
+    m.close()
+
+
+@pytest.mark.parametrize("dims,N", [((1, 1, 1), 2), ((2, 2, 1), 1), ((3, 3, 3), 7), ((4, 4, 4), 7), ((6, 6, 6), 7),
+                                    ((3, 3, 3), 15), ((4, 3, 5), 9), ((5, 5, 4), 12), ((2, 2, 2), 8)])
+@pytest.mark.parametrize("screen", [0, 1])
+def test_fused_cg_equals_launched(dims, N, screen):
+    m = hb.Mesh(*dims, N, perturb=0.1, seed=1, faces=0x07 if N < 3 else 0x3F, fp32=False)
+    b = m.rhs(kind=0, seed=5)
+    x0 = torch.from_numpy(inputs.random_vector(m.n_global, seed=8)).cuda()
+    got = {}
+    for mode in (1, 2):
+        hb.lib().hb_set_cg_fused(m.handle, mode)
+        x, r = m.cg(b, x0.clone(), lam=0.3, screen=screen, max_it=min(25, m.n_global))
+        assert r.status == hb.HB_OK
+        got[mode] = x.cpu().numpy()
+        # bitwise repeatable, stopped on the tolerance, and zero iterations
+        assert np.array_equal(got[mode], m.cg(b, x0.clone(), lam=0.3, screen=screen,
+                                              max_it=min(25, m.n_global))[0].cpu().numpy())
+    assert np.linalg.norm(got[1] - got[2]) <= 1e-12 * np.linalg.norm(got[1])
+    xt, rt = m.cg(b, x0.clone(), lam=0.3, screen=screen, rtol=1e-9, max_it=3000)
+    assert rt.status == hb.HB_OK and rt.rel_res <= 1e-9
+    xz, rz = m.cg(b, x0.clone(), lam=0.3, screen=screen, max_it=0)
+    assert rz.iters == 0 and torch.equal(xz, x0)
     m.close()
