@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(HB_RED_THREADS)
     assemble_body<T, SCREEN, DOT>(yL, rowptr, cols, x, mdiag, lambda, y, ng, partials, counter, st);
 }
 
-template <typename T, int SCREEN, int DOT, bool CONTIG>
+template <typename T, int SCREEN, int DOT, bool CONTIG, bool WIDE>
 __global__ void __launch_bounds__(HB_RED_THREADS)
     assemble_surf_kernel(const T *__restrict__ ys, const int32_t *__restrict__ srow_g,
                          const int32_t *__restrict__ rowptr, const int32_t *__restrict__ cols,
@@ -47,17 +47,17 @@ __global__ void __launch_bounds__(HB_RED_THREADS)
                          int64_t nrows, const double *__restrict__ ax_partials, int64_t n_axp, double *partials,
                          unsigned *counter, hb_cg_state *st)
 {
-    assemble_surf_body<T, SCREEN, DOT, CONTIG>(ys, srow_g, rowptr, cols, x, mdiag, lambda, y, nrows, ax_partials,
-                                               n_axp, partials, counter, st);
+    assemble_surf_body<T, SCREEN, DOT, CONTIG, WIDE>(ys, srow_g, rowptr, cols, x, mdiag, lambda, y, nrows,
+                                                     ax_partials, n_axp, partials, counter, st);
 }
 
-template <typename T, int SCREEN, int DOT>
+template <typename T, int SCREEN, int DOT, int U>
 __global__ void __launch_bounds__(HB_RED_THREADS)
     assemble_grid_kernel(const T *__restrict__ yL, const lattice_t L, const T *__restrict__ x,
                          const T *__restrict__ mdiag, double lambda, T *__restrict__ y, double *partials,
                          unsigned *counter, hb_cg_state *st)
 {
-    assemble_grid_body<T, SCREEN, DOT>(yL, L, x, mdiag, lambda, y, partials, counter, st);
+    assemble_grid_body<T, SCREEN, DOT, U>(yL, L, x, mdiag, lambda, y, partials, counter, st);
 }
 
 template <typename T>
@@ -157,13 +157,22 @@ hb_status launch_assemble_surf(const hb_mesh *m, const T *ys, const T *x, T *y, 
     const int grid = red_grid(nr > 0 ? nr : 1);
     unsigned *ctr = m->counters + 0;
     hb_prof_scope prof("assemble", s);
-#define HB_ASM(SC, DM)                                                                                          \
-    (contig ? assemble_surf_kernel<T, SC, DM, true><<<grid, HB_RED_THREADS, 0, s>>>(                           \
-                  ys, m->srow_g, m->srowptr, nullptr, x, mdiag, lambda, y, nr, m->ax_partials, n_axp,          \
-                  m->partials, ctr, st)                                                                         \
-            : assemble_surf_kernel<T, SC, DM, false><<<grid, HB_RED_THREADS, 0, s>>>(                          \
-                  ys, m->srow_g, m->srowptr, m->scols, x, mdiag, lambda, y, nr, m->ax_partials, n_axp,         \
-                  m->partials, ctr, st))
+    // All copies of a row at once where the rows' reads come from DRAM; below,
+    // they hit L2 and the fewer registers of the narrow form (40 against 80)
+    // are worth more. us, narrow -> wide: FP32 A x, 1.8 M copies 12.1 -> 12.3,
+    // 3.0 M 19.1 -> 15.7, 14.7 M 98 -> 63, 74 M 583 -> 381; FP64 6.2 M 41 -> 42,
+    // 14.7 M 134 -> 90, 112 M 1176 -> 752. Inside CG (with the dot, more of the
+    // mesh in L2) a mixed iteration at 4.1 M copies 276 -> 278, at 7.1 M 386 ->
+    // 383, at 14.7 M 625 -> 590. FP64 contiguous runs never gain (455 -> 491).
+    const int64_t wide_from = dot_mode == HB_DOT_NONE && sizeof(T) == 4 ? 2000000 : 7000000;
+    const bool wide = m->nnz_s >= wide_from && !(contig && sizeof(T) == 8);
+    constexpr bool kWideContig = sizeof(T) == 4;
+#define HB_ASM3(SC, DM, CT, WD, COLS)                                                                         \
+    assemble_surf_kernel<T, SC, DM, CT, WD><<<grid, HB_RED_THREADS, 0, s>>>(                                   \
+        ys, m->srow_g, m->srowptr, COLS, x, mdiag, lambda, y, nr, m->ax_partials, n_axp, m->partials, ctr, st)
+#define HB_ASM(SC, DM)                                                                                        \
+    (contig ? (wide ? HB_ASM3(SC, DM, true, kWideContig, nullptr) : HB_ASM3(SC, DM, true, false, nullptr))     \
+            : (wide ? HB_ASM3(SC, DM, false, true, m->scols) : HB_ASM3(SC, DM, false, false, m->scols)))
     if (screen == 0) {
         if (dot_mode == HB_DOT_NONE) HB_ASM(0, HB_DOT_NONE);
         else if (dot_mode == HB_DOT_TO_TMP) HB_ASM(0, HB_DOT_TO_TMP);
@@ -173,6 +182,7 @@ hb_status launch_assemble_surf(const hb_mesh *m, const T *ys, const T *x, T *y, 
         else if (dot_mode == HB_DOT_TO_TMP) HB_ASM(1, HB_DOT_TO_TMP);
         else HB_ASM(1, HB_DOT_CG_PAP);
     }
+#undef HB_ASM3
 #undef HB_ASM
     HB_CHECK_LAUNCH();
     return HB_OK;
@@ -207,8 +217,14 @@ hb_status launch_assemble_grid(const hb_mesh *m, const T *yL, const T *x, T *y, 
     const int grid = red_grid(m->n_global);
     unsigned *ctr = m->counters + 0;
     hb_prof_scope prof("assemble", s);
-#define HB_ASM(SC, DM) \
-    assemble_grid_kernel<T, SC, DM><<<grid, HB_RED_THREADS, 0, s>>>(yL, L, x, mdiag, lambda, y, m->partials, ctr, st)
+    // points per lane: FP32 8 up to N = 7 (N = 3 388 us with 8, 494 with 4),
+    // then 4 (N = 11 338 with 4, 389 with 8); FP64 4 (N = 7 711, 774 with 8)
+    const bool wide = sizeof(T) == 4 && m->N <= 7;
+#define HB_ASM(SC, DM)                                                                                             \
+    (wide ? assemble_grid_kernel<T, SC, DM, sizeof(T) == 4 ? 8 : 4><<<grid, HB_RED_THREADS, 0, s>>>(               \
+                yL, L, x, mdiag, lambda, y, m->partials, ctr, st)                                                  \
+          : assemble_grid_kernel<T, SC, DM, 4><<<grid, HB_RED_THREADS, 0, s>>>(yL, L, x, mdiag, lambda, y,         \
+                                                                               m->partials, ctr, st))
     if (screen == 0) {
         if (dot_mode == HB_DOT_NONE) HB_ASM(0, HB_DOT_NONE);
         else if (dot_mode == HB_DOT_TO_TMP) HB_ASM(0, HB_DOT_TO_TMP);

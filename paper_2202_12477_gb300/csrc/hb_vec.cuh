@@ -140,7 +140,9 @@ __device__ __forceinline__ void assemble_body(const T *__restrict__ yL, const in
 // partials (interior DOFs) is reduced on the fixed grid.
 // CONTIG: the copies of row r are ys[rowptr[r] .. rowptr[r+1]) (the element
 // kernel wrote them at their CSR positions); cols is not read.
-template <typename T, int SCREEN, int DOT, bool CONTIG = false>
+// WIDE: all copies of a row at once, for meshes whose rows come from DRAM (the
+// same sums in the same order either way).
+template <typename T, int SCREEN, int DOT, bool CONTIG = false, bool WIDE = false>
 __device__ __forceinline__ void assemble_surf_body(const T *__restrict__ ys, const int32_t *__restrict__ srow_g,
                          const int32_t *__restrict__ rowptr, const int32_t *__restrict__ cols,
                          const T *__restrict__ x, const T *__restrict__ mdiag, double lambda, T *__restrict__ y,
@@ -150,46 +152,87 @@ __device__ __forceinline__ void assemble_surf_body(const T *__restrict__ ys, con
     if (DOT == HB_DOT_CG_PAP && st->run == 0) return;
     const T lam = (T)lambda;
     dot_acc<T> acc;
-    // four independent rows per pass keep several dependent load chains
-    // (row pointer -> column -> value) in flight per thread
-    constexpr int U4 = 4;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t r0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r0 < nrows; r0 += U4 * stride) {
-        int g[U4], a[U4], z[U4], c0[U4], c1[U4];
-        T xv[U4], s[U4];
+    if constexpr (!WIDE) {
+        // four independent rows per pass keep several dependent load chains
+        // (row pointer -> column -> value) in flight per thread
+        constexpr int U4 = 4;
+        for (int64_t r0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r0 < nrows; r0 += U4 * stride) {
+            int g[U4], a[U4], z[U4], c0[U4], c1[U4];
+            T xv[U4], s[U4];
 #pragma unroll
-        for (int u = 0; u < U4; u++) {
-            const int64_t r = r0 + u * stride;
-            const bool ok = r < nrows;
-            g[u] = ok ? __ldg(srow_g + r) : -1;
-            a[u] = ok ? __ldg(rowptr + r) : 0;
-            z[u] = ok ? __ldg(rowptr + r + 1) : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < U4; u++) {
-            if constexpr (CONTIG) {
-                c0[u] = a[u] < z[u] ? a[u] : -1;
-                c1[u] = a[u] + 1 < z[u] ? a[u] + 1 : -1;
-            } else {
-                c0[u] = a[u] < z[u] ? __ldcs(cols + a[u]) : -1;
-                c1[u] = a[u] + 1 < z[u] ? __ldcs(cols + a[u] + 1) : -1;
+            for (int u = 0; u < U4; u++) {
+                const int64_t r = r0 + u * stride;
+                const bool ok = r < nrows;
+                g[u] = ok ? __ldg(srow_g + r) : -1;
+                a[u] = ok ? __ldg(rowptr + r) : 0;
+                z[u] = ok ? __ldg(rowptr + r + 1) : 0;
             }
-            xv[u] = g[u] >= 0 ? x[g[u]] : T(0);
-        }
 #pragma unroll
-        for (int u = 0; u < U4; u++) {
-            T v0 = c0[u] >= 0 ? __ldcs(ys + c0[u]) : T(0);
-            T v1 = c1[u] >= 0 ? __ldcs(ys + c1[u]) : T(0);
-            s[u] = v0 + v1;
-        }
+            for (int u = 0; u < U4; u++) {
+                if constexpr (CONTIG) {
+                    c0[u] = a[u] < z[u] ? a[u] : -1;
+                    c1[u] = a[u] + 1 < z[u] ? a[u] + 1 : -1;
+                } else {
+                    c0[u] = a[u] < z[u] ? __ldcs(cols + a[u]) : -1;
+                    c1[u] = a[u] + 1 < z[u] ? __ldcs(cols + a[u] + 1) : -1;
+                }
+                xv[u] = g[u] >= 0 ? x[g[u]] : T(0);
+            }
 #pragma unroll
-        for (int u = 0; u < U4; u++) {
-            if (g[u] < 0) continue;
-            T t = s[u];
-            for (int p = a[u] + 2; p < z[u]; p++) t += __ldcs(ys + (CONTIG ? p : __ldcs(cols + p)));
-            t += SCREEN ? lam * (mdiag[g[u]] * xv[u]) : lam * xv[u];
-            y[g[u]] = t;
-            if (DOT) acc.add(xv[u], t);
+            for (int u = 0; u < U4; u++) {
+                T v0 = c0[u] >= 0 ? __ldcs(ys + c0[u]) : T(0);
+                T v1 = c1[u] >= 0 ? __ldcs(ys + c1[u]) : T(0);
+                s[u] = v0 + v1;
+            }
+#pragma unroll
+            for (int u = 0; u < U4; u++) {
+                if (g[u] < 0) continue;
+                T t = s[u];
+                for (int p = a[u] + 2; p < z[u]; p++) t += __ldcs(ys + (CONTIG ? p : __ldcs(cols + p)));
+                t += SCREEN ? lam * (mdiag[g[u]] * xv[u]) : lam * xv[u];
+                y[g[u]] = t;
+                if (DOT) acc.add(xv[u], t);
+            }
+        }
+    } else {
+        // UR independent rows per pass and all copies of each (at most 8 on a box
+        // of hexahedra) in flight per thread
+        constexpr int UR = sizeof(T) == 8 ? 2 : 4, W = 8;
+        for (int64_t r0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r0 < nrows; r0 += UR * stride) {
+            int g[UR], a[UR], z[UR], c[UR][W];
+            T xv[UR], v[UR][W];
+#pragma unroll
+            for (int u = 0; u < UR; u++) {
+                const int64_t r = r0 + u * stride;
+                const bool ok = r < nrows;
+                g[u] = ok ? __ldg(srow_g + r) : -1;
+                a[u] = ok ? __ldg(rowptr + r) : 0;
+                z[u] = ok ? __ldg(rowptr + r + 1) : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < UR; u++) {
+#pragma unroll
+                for (int w = 0; w < W; w++)
+                    c[u][w] = a[u] + w < z[u] ? (CONTIG ? a[u] + w : __ldcs(cols + a[u] + w)) : -1;
+                xv[u] = g[u] >= 0 ? x[g[u]] : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < UR; u++)
+#pragma unroll
+                for (int w = 0; w < W; w++) v[u][w] = c[u][w] >= 0 ? __ldcs(ys + c[u][w]) : T(0);
+#pragma unroll
+            for (int u = 0; u < UR; u++) {
+                if (g[u] < 0) continue;
+                T t = v[u][0] + v[u][1];
+#pragma unroll
+                for (int w = 2; w < W; w++)
+                    if (c[u][w] >= 0) t += v[u][w];
+                for (int p = a[u] + W; p < z[u]; p++) t += __ldcs(ys + (CONTIG ? p : __ldcs(cols + p)));
+                t += SCREEN ? lam * (mdiag[g[u]] * xv[u]) : lam * xv[u];
+                y[g[u]] = t;
+                if (DOT) acc.add(xv[u], t);
+            }
         }
     }
     if (DOT) {
@@ -246,7 +289,7 @@ __device__ __forceinline__ int lattice_axis(int I, int N, int Eax, int (&ec)[2],
 // (x_g | M_gg x_g). Lanes along I, so x, y and the runs of each element row
 // of yL are read and written coalesced. With a dot mode, x.y over all DOFs is
 // reduced on the fixed grid.
-template <typename T, int SCREEN, int DOT>
+template <typename T, int SCREEN, int DOT, int U>
 __device__ __forceinline__ void assemble_grid_body(const T *__restrict__ yL, const lattice_t L, const T *__restrict__ x,
                                                    const T *__restrict__ mdiag, double lambda, T *__restrict__ y,
                                                    double *partials, unsigned *counter, hb_cg_state *st)
@@ -260,34 +303,59 @@ __device__ __forceinline__ void assemble_grid_body(const T *__restrict__ yL, con
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t nrows = (int64_t)L.NYu * L.NZu;
-    // one warp per lattice row (J, K), lanes along I
+    // One warp per lattice row (J, K), lanes along I, U points per lane: the
+    // loads of up to 2 U copies are issued before the first is used.
+    // Measured at 1.28e8 local nodes, us, one load at a time -> this: FP32 N = 3
+    // 651 -> 392, N = 7 804 -> 302, N = 15 858 -> 306; FP64 N = 7 1013 -> 691,
+    // N = 15 1085 -> 703. Taking the copies as one stream along the lanes (a
+    // shuffle for the shared points) and more loads per lane were slower (FP64
+    // N = 7 815 and 774): what bounds it is the order in which the short runs
+    // of n values reach DRAM, 50 % of the copy rate at N = 7.
+    const unsigned magic = 0xFFFFFFFFu / (unsigned)L.N + 1u;  // I / N = hi(I * magic) for N > 1, I < 3e8 (I <= N Ex < 1.6e8: n_local < 2^31)
+    const int n3i = (int)n3;
     for (int64_t row = warp; row < nrows; row += nwarps) {
-        const int Ju = (int)(row % L.NYu), Ku = (int)(row / L.NYu);
+        const int Ku = (int)(row / L.NYu), Ju = (int)(row - (int64_t)Ku * L.NYu);
         int eyc[2], jc[2], ezc[2], kc[2];
         const int ny = lattice_axis(L.y0 + Ju, L.N, L.Ey, eyc, jc);
         const int nz = lattice_axis(L.z0 + Ku, L.N, L.Ez, ezc, kc);
         const T *__restrict__ xr = x + row * L.NXu;
         T *__restrict__ yr = y + row * L.NXu;
-        for (int Iu = lane; Iu < L.NXu; Iu += 32) {
-            int exc[2], ic[2];
-            const int nx = lattice_axis(L.x0 + Iu, L.N, L.Ex, exc, ic);
-            T t = T(0);
-            int cnt = 0;
-            for (int cz = 0; cz < nz; cz++)
-                for (int cy = 0; cy < ny; cy++) {
-                    const int64_t base = ((int64_t)eyc[cy] + (int64_t)L.Ey * ezc[cz]) * L.Ex;
-                    const int64_t off = ((int64_t)kc[cz] * n + jc[cy]) * n;
-                    for (int cx = 0; cx < nx; cx++) {
-                        const T v = __ldcs(yL + (base + exc[cx]) * n3 + off + ic[cx]);
-                        t = cnt == 0 ? v : t + v;
-                        cnt++;
-                    }
+        for (int i0 = lane; i0 < L.NXu; i0 += 32 * U) {
+            int lo[U], hi[U];  // offsets of the copies in this row of elements (-1: none), in element order
+            T t[U], xv[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int Iu = i0 + 32 * u, I = L.x0 + Iu;
+                const bool ok = Iu < L.NXu;
+                const int q = L.N == 1 ? I : (int)__umulhi((unsigned)I, magic), r = I - q * L.N;
+                lo[u] = ok && r == 0 && q > 0 ? (q - 1) * n3i + L.N : -1;
+                hi[u] = ok && q < L.Ex ? q * n3i + r : -1;
+                xv[u] = ok ? xr[Iu] : T(0);
+            }
+            for (int c = 0; c < nz * ny; c++) {
+                // (selects, not indexed arrays: those would live in local memory)
+                const bool hz = ny == 2 ? c >= 2 : c == 1, hy = ny == 2 && (c & 1);
+                const T *__restrict__ b = yL + ((int64_t)(hy ? eyc[1] : eyc[0]) + (int64_t)L.Ey * (hz ? ezc[1] : ezc[0])) * L.Ex * n3 +
+                                          ((int64_t)(hz ? kc[1] : kc[0]) * n + (hy ? jc[1] : jc[0])) * n;
+                T vl[U], vh[U];
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    vl[u] = lo[u] >= 0 ? __ldcs(b + lo[u]) : T(0);
+                    vh[u] = hi[u] >= 0 ? __ldcs(b + hi[u]) : T(0);
                 }
-            if (cnt == 1) t = t + T(0);
-            const T xv = xr[Iu];
-            t += SCREEN ? lam * (mdiag[row * L.NXu + Iu] * xv) : lam * xv;
-            yr[Iu] = t;
-            if (DOT) acc.add(xv, t);
+                // ascending element order: (c0 + c1) + c2 + ..., a lone copy plus zero
+#pragma unroll
+                for (int u = 0; u < U; u++) t[u] = c == 0 ? vl[u] + vh[u] : (t[u] + vl[u]) + vh[u];
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const int Iu = i0 + 32 * u;
+                if (Iu >= L.NXu) continue;
+                T v = t[u];
+                v += SCREEN ? lam * (mdiag[row * L.NXu + Iu] * xv[u]) : lam * xv[u];
+                yr[Iu] = v;
+                if (DOT) acc.add(xv[u], v);
+            }
         }
     }
     if (DOT) {
