@@ -482,12 +482,12 @@ double hb_u01(uint64_t seed, uint64_t stream, uint64_t idx);
  *                         per lattice row sums each DOF's copies in ascending
  *                         element order, as the CSR does, so y is bitwise the
  *                         same as with the other pencil variants.
- *   HB_VARIANT_TC         (alone or with CSR; HB_F64 at N = 7) the tensor-core element kernel:
+ *   HB_VARIANT_TC         (alone or with CSR; HB_F64 at N = 3, 7, 15) the tensor-core element kernel:
  *                         every derivative contraction (D and D^T along r, s, t) runs
  *                         on the tensor cores (tcgen05.mma, FP16 inputs, FP32
  *                         accumulators in tensor memory) exactly, on an
  *                         Ozaki-style split of the element's values and of D into
- *                         seven 8-bit digits on a per-element fixed-point grid
+ *                         8-bit digits (seven, eight for D) on a per-element fixed-point grid
  *                         (every product and partial sum an integer below 2^24);
  *                         the exact digit sums are combined in int64 and the
  *                         metric step runs in FP64. Error per contraction about
@@ -514,7 +514,7 @@ hb_status hb_get_kernel_variant(const hb_mesh *mesh, hb_precision prec, int *var
  * variant (0, PENCIL, PENCIL|EVEN_ODD, PENCIL|EB2, PENCIL|EVEN_ODD|EB2,
  * PENCIL|EVEN_ODD|ONE, PENCIL|EVEN_ODD|TMA, PENCIL|EVEN_ODD|WS, PENCIL|EVEN_ODD|CSR,
  * PENCIL|EVEN_ODD|ONE|CSR, PENCIL|EVEN_ODD|GRID, PENCIL|EVEN_ODD|ONE|GRID, and TC,
- * TC|CSR for HB_F64 at N = 7; for HB_F64X the six it takes) on `stream`, keeps the
+ * TC|CSR for HB_F64 at N = 3, 7, 15; for HB_F64X the six it takes) on `stream`, keeps the
  * fastest for `prec` (HB_F64, HB_F32 or HB_F64X) on this mesh and returns it in
  * *best_variant. ms_per_variant (may be NULL) has 512 slots
  * indexed by variant and receives the mean time of each. Allocates two scratch vectors for the

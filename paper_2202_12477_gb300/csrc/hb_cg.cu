@@ -370,8 +370,8 @@ extern "C" hb_status hb_set_kernel_variant(hb_mesh *m, hb_precision prec, int va
         hb_set_error("invalid kernel variant %d for precision %d", variant, (int)prec);
         return HB_ERR_ARG;
     }
-    if ((variant & HB_VAR_TC) && (prec != HB_F64 || m->N != 7)) {
-        hb_set_error("the tensor-core element kernel (variant %d) is built for HB_F64 at N = 7", HB_VAR_TC);
+    if ((variant & HB_VAR_TC) && (prec != HB_F64 || !hb_tc_degree(m->N))) {
+        hb_set_error("the tensor-core element kernel (variant %d) is built for HB_F64 at N = 3, 7, 15", HB_VAR_TC);
         return HB_ERR_ARG;
     }
     if (variant & HB_VAR_CSR) {
@@ -504,7 +504,7 @@ extern "C" hb_status hb_autotune(hb_mesh *m, hb_precision prec, hb_screen screen
     // variants differ in where that work runs (element kernel or gather)
     hb_cg_state *tmp = m->state + 1;
     for (int c : candidates) {
-        if ((c & HB_VAR_TC) && (prec != HB_F64 || m->N != 7)) continue;
+        if ((c & HB_VAR_TC) && (prec != HB_F64 || !hb_tc_degree(m->N))) continue;
         if (prec == HB_F64X && !hb_valid_variant_f64x(c)) continue;
         m->variant[pi] = c;
         // one untimed application (first launch, attribute setup), then `reps` timed ones

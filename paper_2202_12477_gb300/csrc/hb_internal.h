@@ -159,7 +159,10 @@ hb_status hb_launch_ax2_f64_range(int N, int64_t E, const double *x, const doubl
 hb_status hb_launch_ax2_f64x(const hb_mesh *m, const double *x, double *ysurf, double *y, double lambda, int screen,
                              double *partials, const int *run, int eb_mode, cudaStream_t s, int64_t *nblocks);
 hb_status hb_ax2_upload_f64x(const double *D_all);
-// Tensor-core FP64 element kernel (N = 7; see HB_VAR_TC) and its tables.
+// Tensor-core FP64 element kernel (see HB_VAR_TC), the degrees it is built for
+// (n = N + 1 = 4, 8, 16: the lines of whole elements fill the 128 rows of an
+// MMA) and its tables.
+static inline bool hb_tc_degree(int N) { return N == 3 || N == 7 || N == 15; }
 hb_status hb_tc_upload();
 hb_status hb_launch_ax_tc_f64(const hb_mesh *m, const double *x, double *ysurf, double *y, double lambda,
                               int screen, double *partials, const int *run, bool csr_store, cudaStream_t s,
@@ -180,7 +183,7 @@ hb_status hb_ax2_upload_f32(const double *D_all);
 // box's lattice arithmetic, one warp per lattice row (with PENCIL | EO, alone
 // or with ONE).
 // HB_VAR_TC = the tensor-core element kernel (alone or with HB_VAR_CSR; FP64,
-// N = 7): every derivative contraction exact on tcgen05 from FP16 digit
+// N = 3, 7, 15): every derivative contraction exact on tcgen05 from FP16 digit
 // slices, the metric step in FP64.
 enum { HB_VAR_PENCIL = 1, HB_VAR_EO = 2, HB_VAR_EB2 = 4, HB_VAR_ONE = 8, HB_VAR_TMA = 16, HB_VAR_WS = 32,
        HB_VAR_CSR = 64, HB_VAR_GRID = 128, HB_VAR_MAX = 255, HB_VAR_TC = 256 };

@@ -159,7 +159,7 @@ extern "C" hb_status hb_tc_selftest(int mode, const float *A_host, const float *
 
 // ---------------------------------------------------------------- tensor-core FP64 element kernel
 //
-// y_L = S_L Z x (Sec. 2, Eq. stiffness) for N = 7 with every derivative
+// y_L = S_L Z x (Sec. 2, Eq. stiffness) for N = 3, 7 and 15 with every derivative
 // contraction (D along r, s, t and D^T along r, s, t; 12 n^4 of the
 // 12 n^4 + 15 n^3 flops of an element) on the tensor cores, exactly, and the
 // metric step (the 6 geometric factors, 15 n^3 flops) in FP64 on the CUDA
@@ -172,7 +172,8 @@ extern "C" hb_status hb_tc_selftest(int mode, const float *A_host, const float *
 //     and written as seven base-256 digits, X = sum_j u_j 256^(6-j), u_0
 //     signed (|u_0| <= 32), u_1..u_6 unsigned bytes;
 //   - D is scaled to integers D_int = round(D 2^s) (|D_int| < 2^55) and written
-//     as seven balanced digits b_d in [-128, 128];
+//     as balanced digits b_d in [-128, 128] (seven, and an eighth below the
+//     binary point);
 //   - digit products are integers below 2^16 and every sum the tensor core
 //     forms stays below 2^24, so FP16 inputs with FP32 accumulation add them
 //     without rounding. For each diagonal t = j + d <= 7 the MMA forms
@@ -187,41 +188,78 @@ extern "C" hb_status hb_tc_selftest(int mode, const float *A_host, const float *
 //   - the exact integers S_t are read back (FP32 -> int32 by adding 1.5 2^23),
 //     combined in two int64 halves and turned into doubles with the exponent
 //     of the element's grid (exact), summed with one FP64 add.
-// Per two-element tile (128 lines per direction, M = 128) and direction: one
-// MMA chain of four K = 16 steps, A = the lines' digits (128 x 64, K-major,
-// K ordered (line position m, digit j) so that one node's seven digits and the
-// offset-correction slot j = 7 are one 16-byte row piece), B = the digit
-// stack of D (64 x 64: output index i x diagonal t by the same K), accumulator
-// 128 x 64 FP32 in TMEM (r and s in columns 0..127, then t in 0..63).
+// n = N + 1 is a power of two, so the lines of whole elements fill M-tiles of
+// 128 rows. Per M-tile and direction: one MMA chain of n / 2 K = 16 steps, A =
+// the lines' digits (128 x 8 n, K-major, K ordered (line position m, digit j)
+// so that one node's seven digits and the offset-correction slot j = 7 are one
+// 16-byte row piece), B = the digit stack of D (8 n x 8 n: output index i x
+// diagonal t by the same K), accumulator 128 x 8 n FP32 in TMEM.
 namespace {
 namespace tcax {
 
-constexpr int N = 7, n = 8, n2 = 64, n3 = 512;
-constexpr int NS = 2 * n2 + 4 * N * (N - 1);  // surface nodes of an element
-constexpr int THREADS = 256;                  // two threads per line of a two-element tile
-constexpr int KH = 4;                         // nodes of its line a thread owns (half of n)
-// One direction's A operand: 8 K chunks (m) of 128 rows x 8 FP16 (16 bytes);
-// rows 16 bytes apart, row chunks of 8 at 128 bytes, K chunks LBO apart. The
-// r operand's K chunks sit 2064 bytes apart (16 bytes more than a chunk), so
-// the eight threads of a store phase, which differ in m, hit different banks.
-constexpr int LBO_R = 2064, LBO_ST = 2048;
-constexpr int ABUF = 7 * LBO_R + 2048 + 112;  // 16,608 bytes, a multiple of 16
-constexpr int BIMG = 64 * 64 * 2;             // one B operand image (64 x 64 FP16)
-constexpr int EXS = 576;                      // padded node stride of an element in the exchange buffers
-constexpr int OFF_A = 0;
-constexpr int OFF_B = OFF_A + 3 * ABUF;
-constexpr int OFF_MISC = OFF_B + 2 * BIMG;
-constexpr int SMEM = OFF_MISC + 64;  // 66,272 bytes: three blocks per SM
-// The exchange buffers (two doubles or two int64 halves per node of the
-// tile) sit in the r and s operands, whose MMAs have completed by then.
-static_assert(4 * EXS * 8 <= 2 * ABUF, "exchange buffers fit in the r and s operands");
-// r and s accumulate in columns 0..127, then t in columns 0..63
-constexpr unsigned TMEM_COLS = 128;
+// Shapes. A tile is MT M-tiles of 128 lines, whole elements; KH = nodes of its
+// t-line (and outputs of its r-, s- and t-line rows) a thread owns.
+//   N = 3:  16 elements, 256 lines, a thread per line
+//   N = 7:  2 elements, 128 lines, two threads per line
+//   N = 15: 1 element, 256 lines, four threads per line (1024 threads)
+// Every shape puts 32 warps of 64 registers on an SM: four blocks, or the one
+// block that N = 15's operands leave room for. Measured at 1.28e8 local nodes,
+// ms per launch: N = 3 4.29 with three blocks, 4.13 with four; N = 7 4.52 with
+// three blocks of 78 registers and its own t operand, 4.42 with four; N = 15
+// 6.43 with 512 threads, 6.16 with 1024. (The FP64 pencil kernel: 8.68, 11.8
+// and 17.4.)
+template <int N_>
+struct shape {
+    static constexpr int N = N_, n = N + 1, n2 = n * n, n3 = n2 * n;
+    static_assert(n == 4 || n == 8 || n == 16, "the lines of whole elements fill M-tiles of 128 rows");
+    static constexpr int NS = 2 * n2 + 4 * N * (N - 1);  // surface nodes of an element
+    static constexpr int MT = n == 8 ? 1 : 2, EPT = MT * 128 / n2;
+    static constexpr int KH = 4, TPL = n / KH, THREADS = MT * 128 * TPL;
+    static constexpr int BLOCKS = n == 16 ? 1 : 4;  // resident per SM
+    // x and node ids of the current and the next tile in registers; else only
+    // the next tile's ids, and x and the ids read again (from L1 or L2)
+    static constexpr bool HOLD = n == 4;
+    // One direction's A operand and M-tile: n K chunks (m) of 128 rows x 8 FP16
+    // (16 bytes); rows 16 bytes apart, row chunks of 8 at 128 bytes, K chunks
+    // LBO apart: 2048 and what puts the eight threads of a store phase, which
+    // differ in (ti, tj), on different banks.
+    static constexpr int LBO_R = n == 4 ? 2080 : 2064, LBO_S = n == 4 ? 2112 : 2048, LBO_T = 2048;
+    static constexpr int A_R = MT * n * LBO_R, A_S = MT * n * LBO_S, A_T = MT * n * LBO_T;
+    // N = 7 and 15 stage t over r, whose MMAs are done by then: room for the
+    // fourth block, or for the B images
+    static constexpr bool RESTAGE = n != 4;
+    static constexpr int OFF_R = 0, OFF_S = A_R, OFF_T = RESTAGE ? 0 : A_R + A_S;
+    static constexpr int BIMG = n2 * 128;  // one B operand image (8 n x 8 n FP16)
+    static constexpr int OFF_B = RESTAGE ? A_R + A_S : A_R + A_S + A_T;
+    static constexpr int OFF_MISC = OFF_B + 2 * BIMG;
+    static constexpr int SMEM = OFF_MISC + 160;
+    // The exchange buffers (two doubles or two int64 halves per node of the
+    // tile) sit in operands whose MMAs are done by then: r and s, or s alone
+    static constexpr int EXS = n == 4 ? 80 : n3;  // node stride of an element
+    static constexpr int OFF_EX = RESTAGE ? OFF_S : 0;
+    static_assert(2 * EPT * EXS * 8 <= (RESTAGE ? A_S : A_R + A_S), "exchange buffers fit");
+    static_assert(A_T <= A_R, "t fits over r");
+    // r and s accumulate in DCOLS columns each, then t in r's
+    static constexpr int DCOLS = MT * n * 8;
+    static constexpr unsigned TMEM_COLS = 2 * DCOLS;
+
+    // node (i, j, k) of element el in the exchange buffers: strides, or at n =
+    // 8 and 16 exclusive ors, that keep a half warp's 8-byte accesses apart
+    static __device__ __forceinline__ int xq(int el, int i, int j, int k)
+    {
+        if constexpr (n == 4) return el * EXS + k * 20 + j * 5 + i;
+        else if constexpr (n == 8) return el * EXS + k * 64 + ((j * 8 + (i ^ j)) ^ ((k & 1) * 8));
+        else return k * 256 + j * 16 + (i ^ j);
+    }
+};
 
 // B operand images of D (0) and D^T (1) in the shared-memory layout (K-major,
-// N chunk stride 128 bytes, K chunk stride 1024), and s (D_int = D 2^s).
-__device__ __align__(16) uint16_t g_tc_bimg[2][64 * 64];
-__constant__ int c_tc_dshift;
+// N chunk stride 128 bytes, K chunk stride 128 n) for n = 4, 8, 16, one after
+// the other, and s (D_int = D 2^s) of each.
+__host__ __device__ constexpr int img_off(int N) { return N == 3 ? 0 : N == 7 ? 2 * 32 * 32 : 2 * 32 * 32 + 2 * 64 * 64; }
+__device__ __align__(16) uint16_t g_tc_bimg[2 * 32 * 32 + 2 * 64 * 64 + 2 * 128 * 128];
+__constant__ int c_tc_dshift[3];
+__host__ __device__ constexpr int tc_index(int N) { return N == 3 ? 0 : N == 7 ? 1 : N == 15 ? 2 : -1; }
 
 struct tc_args {
     const double *x;
@@ -237,9 +275,6 @@ struct tc_args {
     unsigned *err;
     const int32_t *spos;  // SP kernels: CSR position of every surface copy (-1 masked)
 };
-
-// node (i, j, k) of element el in the padded exchange buffers
-__device__ __forceinline__ int xq(int el, int i, int j, int k) { return el * EXS + k * 72 + j * 9 + i; }
 
 __device__ __forceinline__ unsigned exp_bits(double v)
 {
@@ -309,49 +344,38 @@ __device__ __forceinline__ uint4 row_piece(long long X)
     return r;
 }
 
-// Stores the row pieces of the thread's nodes (ti, tj, k0 + q) in the A
-// operands of the directions in `dirs` (bit 0 r, bit 1 s, bit 2 t):
-//   r: row (el, k, j), K chunk m = i;  s: row (el, k, i), m = j;  t: row (el, j, i), m = k.
-__device__ __forceinline__ void stage(unsigned char *Ab, int el, int ti, int tj, int k0, const long long (&X)[KH],
-                                      int dirs)
+// Stores the row pieces of the thread's nodes (ti, tj, k0 + q) of element el
+// in the A operand of direction DIR:
+//   r: line (el, k, j), K chunk m = i;  s: line (el, k, i), m = j;  t: line (el, j, i), m = k.
+template <class C, int DIR>
+__device__ __forceinline__ void stage(unsigned char *sm, int el, int ti, int tj, int k0, const long long (&X)[C::KH])
 {
+    constexpr int lbo = DIR == 0 ? C::LBO_R : DIR == 1 ? C::LBO_S : C::LBO_T;
+    unsigned char *A = sm + (DIR == 0 ? C::OFF_R : DIR == 1 ? C::OFF_S : C::OFF_T);
 #pragma unroll
-    for (int q = 0; q < KH; q++) {
+    for (int q = 0; q < C::KH; q++) {
         const int k = k0 + q;
-        const uint4 p = row_piece(X[q]);
-        if (dirs & 1) *reinterpret_cast<uint4 *>(Ab + 0 * ABUF + ti * LBO_R + (el * 8 + k) * 128 + tj * 16) = p;
-        if (dirs & 2) *reinterpret_cast<uint4 *>(Ab + 1 * ABUF + tj * LBO_ST + (el * 8 + k) * 128 + ti * 16) = p;
-        if (dirs & 4) *reinterpret_cast<uint4 *>(Ab + 2 * ABUF + k * LBO_ST + (el * 8 + tj) * 128 + ti * 16) = p;
+        const int line = el * C::n2 + (DIR == 0 ? k * C::n + tj : DIR == 1 ? k * C::n + ti : tj * C::n + ti);
+        const int m = DIR == 0 ? ti : DIR == 1 ? tj : k;
+        *reinterpret_cast<uint4 *>(A + (line >> 7) * C::n * lbo + m * lbo + (line & 127) * 16) = row_piece(X[q]);
     }
 }
 
-// The r and s chains (accumulator columns 0..63 and 64..127) and, once every
-// thread has read those, the t chain (columns 0..63). K step ks covers the K
-// chunks m = 2 ks, 2 ks + 1 of A and B.
-__device__ __forceinline__ void issue_rs(unsigned tmem, const unsigned char *Ab, const unsigned char *Bi)
+// The MMA chain of direction DIR into accumulator columns col: K step ks
+// covers the K chunks m = 2 ks, 2 ks + 1 of A and B.
+template <class C, int DIR>
+__device__ __forceinline__ void issue(unsigned tmem, unsigned col, const unsigned char *sm, const unsigned char *Bi)
 {
-    constexpr uint32_t idesc = hbtc::idesc_f16(128, 64, false, false);
+    constexpr uint32_t idesc = hbtc::idesc_f16(128, 8 * C::n, false, false);
+    constexpr unsigned lbo = DIR == 0 ? C::LBO_R : DIR == 1 ? C::LBO_S : C::LBO_T;
     const unsigned b0 = hbtc::smem_addr(Bi);
+    const unsigned a0 = hbtc::smem_addr(sm + (DIR == 0 ? C::OFF_R : DIR == 1 ? C::OFF_S : C::OFF_T));
 #pragma unroll
-    for (int dir = 0; dir < 2; dir++) {
-        const unsigned a0 = hbtc::smem_addr(Ab + dir * ABUF);
-        const unsigned lbo = dir == 0 ? LBO_R : LBO_ST;
+    for (int mt = 0; mt < C::MT; mt++)
 #pragma unroll
-        for (int ks = 0; ks < 4; ks++)
-            hbtc::mma_f16(tmem + dir * 64, hbtc::smem_desc(a0 + ks * 2 * lbo, lbo, 128),
-                          hbtc::smem_desc(b0 + ks * 2048, 1024, 128), idesc, ks > 0);
-    }
-}
-
-__device__ __forceinline__ void issue_t(unsigned tmem, const unsigned char *Ab, const unsigned char *Bi)
-{
-    constexpr uint32_t idesc = hbtc::idesc_f16(128, 64, false, false);
-    const unsigned b0 = hbtc::smem_addr(Bi);
-    const unsigned a0 = hbtc::smem_addr(Ab + 2 * ABUF);
-#pragma unroll
-    for (int ks = 0; ks < 4; ks++)
-        hbtc::mma_f16(tmem, hbtc::smem_desc(a0 + ks * 2 * LBO_ST, LBO_ST, 128),
-                      hbtc::smem_desc(b0 + ks * 2048, 1024, 128), idesc, ks > 0);
+        for (int ks = 0; ks < C::n / 2; ks++)
+            hbtc::mma_f16(tmem + col + mt * 8 * C::n, hbtc::smem_desc(a0 + mt * C::n * lbo + ks * 2 * lbo, lbo, 128),
+                          hbtc::smem_desc(b0 + ks * 2 * 128 * C::n, 128 * C::n, 128), idesc, ks > 0);
 }
 
 // Completion of the chain in flight: warp 0 polls the barrier (bounded), the
@@ -391,171 +415,178 @@ __device__ __forceinline__ void combine(const uint32_t (&v)[16], int o, long lon
     lo = (long long)m2 * 65536 + m3;
 }
 
-__device__ __forceinline__ int ring_index7(int i, int j)
+// Reads the thread's KH = 4 outputs of one direction out of tensor memory (its
+// lane, columns from taddr) and hands each one's two halves to f(q, hi, lo).
+template <class C, class F>
+__device__ __forceinline__ void read_out(unsigned taddr, F &&f)
 {
-    return j == 0 ? i : (j == N ? N + 1 + i : 2 * (N + 1) + 2 * (j - 1) + (i == N ? 1 : 0));
+    static_assert(C::KH == 4, "two loads of 16 columns");
+    uint32_t vv[2][16];
+    hbtc::tmem_ld16(taddr, vv[0]);
+    hbtc::tmem_ld16(taddr + 16, vv[1]);
+    hbtc::tmem_wait_ld(vv[0]);
+    hbtc::tmem_wait_ld(vv[1]);
+#pragma unroll
+    for (int c = 0; c < 2; c++)
+#pragma unroll
+        for (int o = 0; o < 2; o++) {
+            long long hi, lo;
+            combine(vv[c], o, hi, lo);
+            f(2 * c + o, hi, lo);
+        }
 }
 
-// Largest biased exponent over element el (warps 0, 1, 4, 5 hold element 0,
-// warps 2, 3, 6, 7 element 1). Every thread calls it; it synchronises.
+// Largest biased exponent over the thread's element. n = 4: its 16 lanes.
+// n = 8: warps 0, 1, 4, 5 hold element 0, warps 2, 3, 6, 7 element 1; n = 16:
+// the block's 32 warps. Every thread calls it; it synchronises the block.
+template <class C>
 __device__ __forceinline__ unsigned element_max(unsigned v, unsigned *wexp, int el)
 {
-    v = __reduce_max_sync(0xffffffffu, v);
-    if ((threadIdx.x & 31) == 0) wexp[threadIdx.x >> 5] = v;
-    __syncthreads();
-    return max(max(wexp[2 * el], wexp[2 * el + 1]), max(wexp[4 + 2 * el], wexp[5 + 2 * el]));
+    if constexpr (C::n == 4) {
+        for (int o = 8; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+        __syncthreads();
+        return v;
+    } else {
+        v = __reduce_max_sync(0xffffffffu, v);
+        if ((threadIdx.x & 31) == 0) wexp[threadIdx.x >> 5] = v;
+        __syncthreads();
+        if constexpr (C::n == 8)
+            return max(max(wexp[2 * el], wexp[2 * el + 1]), max(wexp[4 + 2 * el], wexp[5 + 2 * el]));
+        else
+            return __reduce_max_sync(0xffffffffu, wexp[threadIdx.x & 31]);
+    }
 }
 
-// Thread tid: line tau = tid % 128 of the tile (TMEM lane tau; element
-// el = tau / 64; t-line (ti, tj) = (tau % 8, tau / 8 % 8)) and half h = tid / 128:
-// nodes k = 4h .. 4h + 3 of its t-line, outputs 4h .. 4h + 3 of its r-, s-
-// and t-line rows. Per tile and phase (D, then D^T): stage the three operands,
-// run the r and s chains, read them out (gradients to the exchange buffers in
-// the r/s operands, or the exact sums of D^T along r and s), run the t chain
-// into the same columns, read it out. The six metric factors are prefetched
-// into L2 at the tile's start and loaded at the metric step, not held in
-// registers: with 80 registers, 66 KB of shared memory and 128 TMEM columns a
-// block, three blocks fit on an SM (two held 124 registers, 85 KB and 256
-// columns each: 14% slower, the same bits).
-template <bool SP>
-__global__ void __launch_bounds__(THREADS, 3) ax_tc_kernel(const tc_args A)
+// Thread tid: M-tile mt, TMEM lane tid % 128: line mt 128 + lane of the tile
+// (element el; t-line (ti, tj)), and part h of it: nodes k = k0 .. k0 + KH - 1
+// of its t-line, the same outputs of its r-, s- and t-line rows. Per tile and
+// phase (D, then D^T): stage the operands, run the r and s chains, read r out
+// (gradients to the exchange buffers, or the exact sums of D^T), start the t
+// chain into r's columns, read s out meanwhile, then t. The six metric factors
+// are prefetched into L2 at the tile's start and loaded at the metric step,
+// not held in registers. What bounds it (N = 7, ncu): the FP64 pipe 55 %, the
+// integer pipe 52 %, issue 55 % of the time; DRAM a quarter of the copy rate.
+template <class C, bool SP>
+__global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_args A)
 {
+    constexpr int N = C::N, n = C::n, n2 = C::n2, n3 = C::n3, NS = C::NS, KH = C::KH, EPT = C::EPT;
+    constexpr bool kHold = C::HOLD;
     if (A.run && *A.run == 0) return;
     extern __shared__ __align__(1024) unsigned char sm[];
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int tau = tid & 127, h = tid >> 7, k0 = KH * h;
-    const int el = tau >> 6, a = tau & 63, ti = a & 7, tj = a >> 3;
-    unsigned char *Ab = sm + OFF_A;
-    unsigned char *Bi = sm + OFF_B;
-    double *ExR = reinterpret_cast<double *>(sm + OFF_A);  // in the r/s operands once their MMAs are done
-    double *ExS = ExR + 2 * EXS;
+    const int mt = (tid >> 7) % C::MT, h = (tid >> 7) / C::MT, k0 = KH * h;
+    const int line = mt * 128 + (tid & 127), el = line / n2, a = line % n2, ti = a % n, tj = a / n;
+    unsigned char *Bi = sm + C::OFF_B;
+    double *ExR = reinterpret_cast<double *>(sm + C::OFF_EX);
+    double *ExS = ExR + EPT * C::EXS;
     long long *Yhi = reinterpret_cast<long long *>(ExR);
     long long *Ylo = reinterpret_cast<long long *>(ExS);
-    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + OFF_MISC);
-    unsigned *tptr = reinterpret_cast<unsigned *>(sm + OFF_MISC + 8);
-    unsigned *wexp = reinterpret_cast<unsigned *>(sm + OFF_MISC + 16);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + C::OFF_MISC);
+    unsigned *tptr = reinterpret_cast<unsigned *>(sm + C::OFF_MISC + 8);
+    unsigned *wexp = reinterpret_cast<unsigned *>(sm + C::OFF_MISC + 16);
 
-    for (int q = tid; q < 2 * BIMG / 16; q += THREADS)
-        reinterpret_cast<uint4 *>(Bi)[q] = reinterpret_cast<const uint4 *>(&g_tc_bimg[0][0])[q];
+    for (int q = tid; q < 2 * C::BIMG / 16; q += C::THREADS)
+        reinterpret_cast<uint4 *>(Bi)[q] = reinterpret_cast<const uint4 *>(g_tc_bimg + img_off(N))[q];
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(hbtc::smem_addr(bar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) hbtc::tmem_alloc(tptr, TMEM_COLS);
+    if (warp == 0) hbtc::tmem_alloc(tptr, C::TMEM_COLS);
     hbtc::fence_async_smem();
     hbtc::fence_before_sync();
     __syncthreads();
     hbtc::fence_after_sync();
     const unsigned tmem = *tptr;
-    const int dshift = c_tc_dshift;
-    const unsigned tl = tmem + ((unsigned)((warp & 3) * 32) << 16) + (unsigned)(32 * h);
+    const int dshift = c_tc_dshift[tc_index(N)];
+    const unsigned tl = tmem + ((unsigned)((warp & 3) * 32) << 16) + (unsigned)(8 * (mt * n + k0));
 
     hbacc::dot_acc<double> acc;
     unsigned phase = 0;
     int gave_up = 0;
-    const int64_t ntiles = (A.E + 1) / 2;
+    const int64_t ntiles = (A.E + EPT - 1) / EPT;
     int gid_n[KH];
-    double u_n[KH];
+    double u_n[kHold ? KH : 1];
     auto gather = [&](int64_t gg) {
-        const int64_t ee = 2 * gg + el;
+        const int64_t ee = EPT * gg + el;
         const bool act = gg < ntiles && ee < A.E;
         const int32_t *lg = A.l2g + ee * n3 + a;
 #pragma unroll
-        for (int q = 0; q < KH; q++) gid_n[q] = act ? __ldcs(lg + (k0 + q) * n2) : -1;
+        for (int q = 0; q < KH; q++) gid_n[q] = act ? (kHold ? __ldcs(lg + (k0 + q) * n2) : __ldg(lg + (k0 + q) * n2)) : -1;
+        if constexpr (kHold) {
 #pragma unroll
-        for (int q = 0; q < KH; q++) u_n[q] = gid_n[q] >= 0 ? __ldg(A.x + gid_n[q]) : 0.0;
+            for (int q = 0; q < KH; q++) u_n[q] = gid_n[q] >= 0 ? __ldg(A.x + gid_n[q]) : 0.0;
+        }
     };
     gather(blockIdx.x);
     for (int64_t g = blockIdx.x; g < ntiles; g += gridDim.x) {
-        const int64_t e = 2 * g + el;
+        const int64_t e = EPT * g + el;
         const bool active = e < A.E;
-        int gid[KH];
+        int gid[kHold ? KH : 1];
         double u[KH];
 #pragma unroll
         for (int q = 0; q < KH; q++) {
-            gid[q] = gid_n[q];
-            u[q] = u_n[q];
+            if constexpr (kHold) {
+                gid[q] = gid_n[q];
+                u[q] = u_n[q];
+            } else {
+                u[q] = gid_n[q] >= 0 ? __ldg(A.x + gid_n[q]) : 0.0;
+            }
         }
         {
             // the tile's six metric factors into L2 now (the first 6 n^2 values
             // of each element's k-slab of 7 n^2; J w only if screening reads
-            // it): 24 lines of 128 bytes per slab, read at the metric step
-            const int64_t e0 = 2 * g;
-            const int nel = e0 + 1 < A.E ? 2 : 1;
+            // it), read at the metric step
+            const int64_t e0 = EPT * g;
+            const int nel = e0 + EPT <= A.E ? EPT : (int)(A.E - e0);
             constexpr int kLines = 6 * n2 * 8 / 128;
-            for (int L = tid; L < nel * n * kLines; L += THREADS) {
-                const int eo = L / (n * kLines), k = (L / kLines) % n, line = L % kLines;
-                const double *p = A.geo + (e0 + eo) * 7 * n3 + k * 7 * n2 + line * 16;
+            for (int L = tid; L < nel * n * kLines; L += C::THREADS) {
+                const int sl = L / kLines, ln = L - sl * kLines;  // slab sl of the tile
+                const double *p = A.geo + e0 * 7 * n3 + (int64_t)sl * 7 * n2 + ln * 16;
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
             }
         }
         unsigned em = 0;
 #pragma unroll
         for (int q = 0; q < KH; q++) em = max(em, exp_bits(u[q]));
-        const unsigned eu = element_max(em, wexp, el);
-        {
-            long long X[KH];
+        const unsigned eu = element_max<C>(em, wexp, el);
+        long long X[KH];
 #pragma unroll
-            for (int q = 0; q < KH; q++) X[q] = eu == 0x7FFu ? 0 : to_fixed(u[q], eu);
-            stage(Ab, el, ti, tj, k0, X, 7);
-        }
+        for (int q = 0; q < KH; q++) X[q] = eu == 0x7FFu ? 0 : to_fixed(u[q], eu);
+        stage<C, 0>(sm, el, ti, tj, k0, X);
+        stage<C, 1>(sm, el, ti, tj, k0, X);
+        if constexpr (!C::RESTAGE) stage<C, 2>(sm, el, ti, tj, k0, X);
         hbtc::fence_async_smem();
         hbtc::fence_before_sync();
         __syncthreads();
         if (tid == 0) {
             hbtc::fence_after_sync();
-            issue_rs(tmem, Ab, Bi);
+            issue<C, 0>(tmem, 0, sm, Bi);
+            issue<C, 1>(tmem, C::DCOLS, sm, Bi);
             hbtc::mma_commit(bar);
         }
         mma_done(bar, phase, warp, A.err, gave_up);
         const int goff = (int)eu - 1075 - dshift + 40;
         const bool ubad = eu == 0x7FFu;
-        // ---- gradients along r and s into the exchange buffers
-#pragma unroll
-        for (int dir = 0; dir < 2; dir++) {
-            uint32_t vv[2][16];
-            hbtc::tmem_ld16(tl + dir * 64, vv[0]);
-            hbtc::tmem_ld16(tl + dir * 64 + 16, vv[1]);
-            hbtc::tmem_wait_ld(vv[0]);
-            hbtc::tmem_wait_ld(vv[1]);
-#pragma unroll
-            for (int c = 0; c < 2; c++) {
-#pragma unroll
-                for (int o = 0; o < 2; o++) {
-                    long long hi, lo;
-                    combine(vv[c], o, hi, lo);
-                    const double gv = ubad ? __longlong_as_double(0x7FF8000000000000ll) : halves_to_double(hi, lo, goff);
-                    const int out = k0 + 2 * c + o;
-                    if (dir == 0) ExR[xq(el, out, tau & 7, (tau >> 3) & 7)] = gv;
-                    else ExS[xq(el, tau & 7, out, (tau >> 3) & 7)] = gv;
-                }
-            }
-        }
-        // every thread has read columns 0..127: the t chain may reuse them
+        auto value = [&](long long hi, long long lo) {
+            return ubad ? __longlong_as_double(0x7FF8000000000000ll) : halves_to_double(hi, lo, goff);
+        };
+        if constexpr (C::RESTAGE) stage<C, 2>(sm, el, ti, tj, k0, X);
+        // ---- gradient along r into its exchange buffer; its columns are free
+        // for the t chain once every thread has read them
+        read_out<C>(tl, [&](int q, long long hi, long long lo) { ExR[C::xq(el, k0 + q, ti, tj)] = value(hi, lo); });
+        if constexpr (C::RESTAGE) hbtc::fence_async_smem();
         hbtc::fence_before_sync();
         __syncthreads();
         if (tid == 0) {
             hbtc::fence_after_sync();
-            issue_t(tmem, Ab, Bi);
+            issue<C, 2>(tmem, 0, sm, Bi);
             hbtc::mma_commit(bar);
         }
+        read_out<C>(tl + C::DCOLS,
+                    [&](int q, long long hi, long long lo) { ExS[C::xq(el, ti, k0 + q, tj)] = value(hi, lo); });
         mma_done(bar, phase, warp, A.err, gave_up);
         double gt[KH];
-        {
-            uint32_t vv[2][16];
-            hbtc::tmem_ld16(tl, vv[0]);
-            hbtc::tmem_ld16(tl + 16, vv[1]);
-            hbtc::tmem_wait_ld(vv[0]);
-            hbtc::tmem_wait_ld(vv[1]);
-#pragma unroll
-            for (int c = 0; c < 2; c++)
-#pragma unroll
-                for (int o = 0; o < 2; o++) {
-                    long long hi, lo;
-                    combine(vv[c], o, hi, lo);
-                    gt[2 * c + o] = ubad ? __longlong_as_double(0x7FF8000000000000ll) : halves_to_double(hi, lo, goff);
-                }
-        }
+        read_out<C>(tl, [&](int q, long long hi, long long lo) { gt[q] = value(hi, lo); });
         // ---- metric (FP64): v = G grad at the thread's nodes, factors loaded here
         double vr[KH], vs[KH], vt[KH];
         unsigned evm = 0;
@@ -566,7 +597,7 @@ __global__ void __launch_bounds__(THREADS, 3) ax_tc_kernel(const tc_args A)
                 double G[6];
 #pragma unroll
                 for (int c = 0; c < 6; c++) G[c] = active ? __ldcs(ge + (k0 + q) * 7 * n2 + c * n2) : 0.0;
-                const int xi = xq(el, ti, tj, k0 + q);
+                const int xi = C::xq(el, ti, tj, k0 + q);
                 const double ur = ExR[xi], us = ExS[xi], ut = gt[q];
                 vr[q] = fma(G[2], ut, fma(G[1], us, G[0] * ur));
                 vs[q] = fma(G[4], ut, fma(G[3], us, G[1] * ur));
@@ -576,108 +607,87 @@ __global__ void __launch_bounds__(THREADS, 3) ax_tc_kernel(const tc_args A)
         }
         // (element_max meets the block: every exchange read is done before
         // the operands are staged over the exchange buffers)
-        const unsigned ev = element_max(evm, wexp, el);
-        {
-            long long X[KH];
+        const unsigned ev = element_max<C>(evm, wexp, el);
 #pragma unroll
-            for (int q = 0; q < KH; q++) X[q] = ev == 0x7FFu ? 0 : to_fixed(vr[q], ev);
-            stage(Ab, el, ti, tj, k0, X, 1);
+        for (int q = 0; q < KH; q++) X[q] = ev == 0x7FFu ? 0 : to_fixed(vr[q], ev);
+        stage<C, 0>(sm, el, ti, tj, k0, X);
 #pragma unroll
-            for (int q = 0; q < KH; q++) X[q] = ev == 0x7FFu ? 0 : to_fixed(vs[q], ev);
-            stage(Ab, el, ti, tj, k0, X, 2);
+        for (int q = 0; q < KH; q++) X[q] = ev == 0x7FFu ? 0 : to_fixed(vs[q], ev);
+        stage<C, 1>(sm, el, ti, tj, k0, X);
 #pragma unroll
-            for (int q = 0; q < KH; q++) X[q] = ev == 0x7FFu ? 0 : to_fixed(vt[q], ev);
-            stage(Ab, el, ti, tj, k0, X, 4);
-        }
+        for (int q = 0; q < KH; q++) X[q] = ev == 0x7FFu ? 0 : to_fixed(vt[q], ev);
+        if constexpr (!C::RESTAGE) stage<C, 2>(sm, el, ti, tj, k0, X);
         hbtc::fence_async_smem();
         hbtc::fence_before_sync();
         __syncthreads();
         if (tid == 0) {
             hbtc::fence_after_sync();
-            issue_rs(tmem, Ab, Bi + BIMG);
+            issue<C, 0>(tmem, 0, sm, Bi + C::BIMG);
+            issue<C, 1>(tmem, C::DCOLS, sm, Bi + C::BIMG);
             hbtc::mma_commit(bar);
         }
         gather(g + gridDim.x);
         mma_done(bar, phase, warp, A.err, gave_up);
-        // ---- D^T along r and s summed exactly into the exchange buffers
-#pragma unroll
-        for (int dir = 0; dir < 2; dir++) {
-            uint32_t vv[2][16];
-            hbtc::tmem_ld16(tl + dir * 64, vv[0]);
-            hbtc::tmem_ld16(tl + dir * 64 + 16, vv[1]);
-            hbtc::tmem_wait_ld(vv[0]);
-            hbtc::tmem_wait_ld(vv[1]);
-#pragma unroll
-            for (int c = 0; c < 2; c++) {
-#pragma unroll
-                for (int o = 0; o < 2; o++) {
-                    long long hi, lo;
-                    combine(vv[c], o, hi, lo);
-                    const int out = k0 + 2 * c + o;
-                    if (dir == 0) {
-                        const int q = xq(el, out, tau & 7, (tau >> 3) & 7);
-                        Yhi[q] = hi;
-                        Ylo[q] = lo;
-                    } else {
-                        const int q = xq(el, tau & 7, out, (tau >> 3) & 7);
-                        Yhi[q] += hi;
-                        Ylo[q] += lo;
-                    }
-                }
-            }
-            if (dir == 0) __syncthreads();
-        }
+        if constexpr (C::RESTAGE) stage<C, 2>(sm, el, ti, tj, k0, X);
+        // ---- D^T along r and s summed exactly in the exchange buffers
+        read_out<C>(tl, [&](int q, long long hi, long long lo) {
+            const int xi = C::xq(el, k0 + q, ti, tj);
+            Yhi[xi] = hi;
+            Ylo[xi] = lo;
+        });
+        if constexpr (C::RESTAGE) hbtc::fence_async_smem();
         hbtc::fence_before_sync();
         __syncthreads();
         if (tid == 0) {
             hbtc::fence_after_sync();
-            issue_t(tmem, Ab, Bi + BIMG);
+            issue<C, 2>(tmem, 0, sm, Bi + C::BIMG);
             hbtc::mma_commit(bar);
         }
+        read_out<C>(tl + C::DCOLS, [&](int q, long long hi, long long lo) {
+            const int xi = C::xq(el, ti, k0 + q, tj);
+            Yhi[xi] += hi;
+            Ylo[xi] += lo;
+        });
         mma_done(bar, phase, warp, A.err, gave_up);
         {
             const int yoff = (int)ev - 1075 - dshift + 40;
             const bool vbad = ev == 0x7FFu;
             double *ys = A.ysurf + e * NS;
             const bool ring = ti == 0 || ti == N || tj == 0 || tj == N;
-            const int r = ring ? ring_index7(ti, tj) : 0;
-            uint32_t vv[2][16];
-            hbtc::tmem_ld16(tl, vv[0]);
-            hbtc::tmem_ld16(tl + 16, vv[1]);
-            hbtc::tmem_wait_ld(vv[0]);
-            hbtc::tmem_wait_ld(vv[1]);
-#pragma unroll
-            for (int c = 0; c < 2; c++) {
-#pragma unroll
-                for (int o = 0; o < 2; o++) {
-                    long long hi, lo;
-                    combine(vv[c], o, hi, lo);
-                    const int qq = 2 * c + o, k = k0 + qq;
-                    const int xi = xq(el, ti, tj, k);
-                    hi += Yhi[xi];
-                    lo += Ylo[xi];
-                    const double yc = vbad ? __longlong_as_double(0x7FF8000000000000ll) : halves_to_double(hi, lo, yoff);
-                    if (!active) continue;
-                    if (SP && (k == 0 || k == N || ring)) {
-                        const int sidx = k == 0 ? a : (k == N ? n2 + a : 2 * n2 + (k - 1) * 4 * N + r);
-                        const int pos = __ldg(A.spos + e * NS + sidx);
-                        if (pos >= 0) A.ysurf[pos] = yc;
-                    } else if (k == 0) {
-                        ys[a] = yc;
-                    } else if (k == N) {
-                        ys[n2 + a] = yc;
-                    } else if (ring) {
-                        ys[2 * n2 + (k - 1) * 4 * N + r] = yc;
+            const int r = tj == 0 ? ti : (tj == N ? n + ti : 2 * n + 2 * (tj - 1) + (ti == N ? 1 : 0));
+            read_out<C>(tl, [&](int q, long long hi, long long lo) {
+                const int k = k0 + q, xi = C::xq(el, ti, tj, k);
+                hi += Yhi[xi];
+                lo += Ylo[xi];
+                const double yc = vbad ? __longlong_as_double(0x7FF8000000000000ll) : halves_to_double(hi, lo, yoff);
+                if (!active) return;
+                if (SP && (k == 0 || k == N || ring)) {
+                    const int sidx = k == 0 ? a : (k == N ? n2 + a : 2 * n2 + (k - 1) * 4 * N + r);
+                    const int pos = __ldg(A.spos + e * NS + sidx);
+                    if (pos >= 0) A.ysurf[pos] = yc;
+                } else if (k == 0) {
+                    ys[a] = yc;
+                } else if (k == N) {
+                    ys[n2 + a] = yc;
+                } else if (ring) {
+                    ys[2 * n2 + (k - 1) * 4 * N + r] = yc;
+                } else {
+                    int gk;
+                    double xv;
+                    if constexpr (kHold) {
+                        gk = gid[q];
+                        xv = u[q];
                     } else {
-                        const double xv = u[qq];
-                        const double jw = A.screen ? __ldg(A.geo + (e * n + k) * 7 * n2 + 6 * n2 + a) : 1.0;
-                        double yy = yc;
-                        yy += A.lambda * (jw * xv);
-                        A.y[gid[qq]] = yy;
-                        acc.add(xv, yy);
+                        gk = __ldg(A.l2g + e * n3 + k * n2 + a);
+                        xv = __ldg(A.x + gk);
                     }
+                    const double jw = A.screen ? __ldg(A.geo + (e * n + k) * 7 * n2 + 6 * n2 + a) : 1.0;
+                    double yy = yc;
+                    yy += A.lambda * (jw * xv);
+                    A.y[gk] = yy;
+                    acc.add(xv, yy);
                 }
-            }
+            });
         }
         // the next tile stages over the exchange buffers read above
         hbtc::fence_before_sync();
@@ -694,7 +704,7 @@ __global__ void __launch_bounds__(THREADS, 3) ax_tc_kernel(const tc_args A)
     hbtc::fence_before_sync();
     __syncthreads();
     hbtc::fence_after_sync();
-    if (warp == 0) hbtc::tmem_free(tmem, TMEM_COLS);
+    if (warp == 0) hbtc::tmem_free(tmem, C::TMEM_COLS);
 }
 
 // ---- host: B images and launch
@@ -719,104 +729,205 @@ static long long fp16_part(long long c)
     return c < 0 ? -(long long)p : (long long)p;
 }
 
+// Double-double host arithmetic (Dekker 1971, Knuth: two-sum, two-product with
+// fma), about 106 bits, for the derivative matrix: its digits hold 63 bits,
+// more than a double's 53.
+struct dd {
+    double h, l;
+};
+static dd dd_norm(double a, double b)
+{
+    const double s = a + b;
+    return {s, b - (s - a)};
+}
+static dd operator+(dd a, dd b)
+{
+    const double s = a.h + b.h, v = s - a.h;
+    return dd_norm(s, (a.h - (s - v)) + (b.h - v) + (a.l + b.l));
+}
+static dd operator-(dd a, dd b) { return a + dd{-b.h, -b.l}; }
+static dd operator*(dd a, dd b)
+{
+    const double p = a.h * b.h;
+    return dd_norm(p, std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
+}
+static dd operator/(dd a, dd b)
+{
+    const double q = a.h / b.h;
+    const dd r = a - b * dd{q, 0.0};
+    const double q2 = r.h / b.h;
+    return dd_norm(q, q2 + (r - b * dd{q2, 0.0}).h / b.h);
+}
+
+// D of degree N in double-double at the GLL nodes that xi approximates: two
+// Newton steps on N (P_{N-1} - x P_N), derivative -N (N + 1) P_N; then
+// D_ij = P_N(x_i) / (P_N(x_j) (x_i - x_j)), corners -+N (N + 1) / 4.
+static void derivative_dd(int N, const double *xi, dd (&D)[16][16])
+{
+    const int n = N + 1;
+    dd x[16], P[16];
+    auto legendre = [N](dd z, dd &PN, dd &Pm) {
+        dd a{1.0, 0.0}, b = z;
+        for (int k = 2; k <= N; k++) {
+            const dd c = (dd{2.0 * k - 1.0, 0.0} * z * b - dd{k - 1.0, 0.0} * a) / dd{(double)k, 0.0};
+            a = b;
+            b = c;
+        }
+        PN = b;
+        Pm = a;
+    };
+    for (int i = 0; i < n; i++) {
+        x[i] = {xi[i], 0.0};
+        for (int it = 0; it < 2 && i > 0 && i < N; it++) {
+            dd PN, Pm;
+            legendre(x[i], PN, Pm);
+            x[i] = x[i] + (Pm - x[i] * PN) / (dd{N + 1.0, 0.0} * PN);
+        }
+    }
+    for (int i = 0; i < n; i++) {  // symmetric node set
+        dd Pm;
+        x[i] = (x[i] - x[N - i]) * dd{0.5, 0.0};
+        x[N - i] = {-x[i].h, -x[i].l};
+        legendre(x[i], P[i], Pm);
+        legendre(x[N - i], P[N - i], Pm);
+    }
+    for (int i = 0; i < n; i++)
+        for (int j = 0; j < n; j++) D[i][j] = i == j ? dd{0.0, 0.0} : P[i] / (P[j] * (x[i] - x[j]));
+    D[0][0] = {-N * (N + 1) / 4.0, 0.0};
+    D[N][N] = {N * (N + 1) / 4.0, 0.0};
+}
+
 }  // namespace tcax
 }  // namespace
 
-// Builds the B images from the degree-7 derivative matrix and uploads them to
-// the current device (once per device, from hb_ensure_device_tables).
+// Builds the B images of the degrees the kernel takes from their derivative
+// matrices and uploads them to the current device (once per device, from
+// hb_ensure_device_tables). D (in double-double: a double's rounding of D would
+// be most of the kernel's error) is split into eight digits: D_int = D 2^s,
+// with |D_int| < 2^55 and eight binary places (the eighth digit meets only the
+// leading digit of the values, on the last diagonal). Largest sum of magnitudes
+// an accumulator can meet (digits, offsets and the correction): 2^19.3, 2^21.0
+// and 2^22.0 for N = 3, 7, 15, below the 2^24 FP32 holds exactly; the sums S_t
+// stay below 2^20.7.
 hb_status hb_tc_upload()
 {
     using namespace tcax;
-    double xi[n], w[n], D[n * n];
-    hb_reference_element(N, xi, w, D);
-    double mx = 0.0;
-    for (int q = 0; q < n * n; q++) mx = std::fmax(mx, std::fabs(D[q]));
-    const int s = 55 - (std::ilogb(mx) + 1);
-    static uint16_t img[2][64 * 64];
-    for (int tr = 0; tr < 2; tr++) {
-        int b[7][n][n];  // digit d of D_int[i][m] (D^T for tr = 1), weight 256^(6-d)
-        for (int i = 0; i < n; i++)
-            for (int m = 0; m < n; m++) {
-                const double v = tr ? D[m * n + i] : D[i * n + m];
-                long long q = std::llround(std::ldexp(v, s));
-                for (int d = 6; d >= 1; d--) {
-                    const long long r = ((q + 128) & 255) - 128;
-                    b[d][i][m] = (int)r;
-                    q = (q - r) >> 8;
-                }
-                if (q < -128 || q > 128) {
-                    hb_set_error("tensor-core split: leading digit %lld out of range", q);
-                    return HB_ERR_ARG;
-                }
-                b[0][i][m] = (int)q;
-            }
-        uint16_t *im = img[tr];
-        std::memset(im, 0, sizeof img[0]);
-        // element (row (i, t), K (m, digit j)) at i * 128 + t * 16 + m * 1024 + j * 2
-        auto put = [&](int i, int t, int j, int m, long long val) {
-            im[(i * 128 + t * 16 + m * 1024 + j * 2) / 2] = fp16_exact(val);
-        };
-        for (int i = 0; i < n; i++)
-            for (int t = 0; t < 8; t++) {
-                long long beta = 0;  // what the digit offsets add to column (i, t)
-                for (int j = 0; j < 7; j++) {
-                    const int d = t - j;
-                    if (d < 0 || d > 6) continue;
-                    long long rs = 0;
-                    for (int m = 0; m < n; m++) {
-                        put(i, t, j, m, b[d][i][m]);
-                        rs += b[d][i][m];
+    static uint16_t img[sizeof(g_tc_bimg) / 2];
+    int shift[3];
+    std::memset(img, 0, sizeof img);
+    for (int N : {3, 7, 15}) {
+        const int n = N + 1;
+        double xi[16], w[16], D64[256];
+        dd D[16][16];
+        hb_reference_element(N, xi, w, D64);
+        derivative_dd(N, xi, D);
+        double mx = 0.0;
+        for (int q = 0; q < n * n; q++) mx = std::fmax(mx, std::fabs(D[q / n][q % n].h));
+        const int s = 55 - (std::ilogb(mx) + 1);
+        shift[tc_index(N)] = s;
+        for (int tr = 0; tr < 2; tr++) {
+            int b[8][16][16];  // digit d of D_int[i][m] (D^T for tr = 1), weight 256^(6-d)
+            for (int i = 0; i < n; i++)
+                for (int m = 0; m < n; m++) {
+                    const dd v = tr ? D[m][i] : D[i][m];
+                    // round(v 2^(s + 8)), |.| < 2^63
+                    const double vh = std::ldexp(v.h, s + 8), vr = std::rint(vh);
+                    __int128 q = (__int128)(long long)vr + std::llround((vh - vr) + std::ldexp(v.l, s + 8));
+                    for (int d = 7; d >= 1; d--) {
+                        const int r = (int)((q + 128) & 255) - 128;
+                        b[d][i][m] = r;
+                        q = (q - r) >> 8;
                     }
-                    beta += (j == 0 ? 384 : 256) * rs;
+                    if (q < -128 || q > 128) {
+                        hb_set_error("tensor-core split: leading digit %d out of range", (int)q);
+                        return HB_ERR_ARG;
+                    }
+                    b[0][i][m] = (int)q;
                 }
-                // slot j = 7 of each K chunk: 128 (A side) times parts summing to -beta / 128
-                long long c = -beta / 128;
-                for (int m = 0; m < n && c != 0; m++) {
-                    const long long p = fp16_part(c);
-                    put(i, t, 7, m, p);
-                    c -= p;
+            uint16_t *im = img + img_off(N) + tr * 64 * n * n;
+            // element (row (i, t), K (m, digit j)) at i * 128 + t * 16 + m * 128 n + j * 2
+            auto put = [&](int i, int t, int j, int m, long long val) {
+                im[(i * 128 + t * 16 + m * 128 * n + j * 2) / 2] = fp16_exact(val);
+            };
+            for (int i = 0; i < n; i++)
+                for (int t = 0; t < 8; t++) {
+                    long long beta = 0;  // what the digit offsets add to column (i, t)
+                    for (int j = 0; j < 7; j++) {
+                        const int d = t - j;
+                        if (d < 0 || d > 7) continue;
+                        long long rs = 0;
+                        for (int m = 0; m < n; m++) {
+                            put(i, t, j, m, b[d][i][m]);
+                            rs += b[d][i][m];
+                        }
+                        beta += (j == 0 ? 384 : 256) * rs;
+                    }
+                    // slot j = 7 of each K chunk: 128 (A side) times parts summing to -beta / 128
+                    long long c = -beta / 128;
+                    for (int m = 0; m < n && c != 0; m++) {
+                        const long long p = fp16_part(c);
+                        put(i, t, 7, m, p);
+                        c -= p;
+                    }
+                    if (c != 0) {
+                        hb_set_error("tensor-core split: offset correction does not fit");
+                        return HB_ERR_ARG;
+                    }
                 }
-                if (c != 0) {
-                    hb_set_error("tensor-core split: offset correction does not fit");
-                    return HB_ERR_ARG;
-                }
-            }
+        }
     }
     HB_TRY_CUDA(cudaMemcpyToSymbol(g_tc_bimg, img, sizeof img));
-    HB_TRY_CUDA(cudaMemcpyToSymbol(c_tc_dshift, &s, sizeof s));
+    HB_TRY_CUDA(cudaMemcpyToSymbol(c_tc_dshift, shift, sizeof shift));
     return HB_OK;
 }
 
-// Tensor-core FP64 element kernel (N = 7): interior DOFs finished here (y,
-// lambda term, partial of x.y per block), surface values to ysurf for the
-// surface gather. Persistent grid: three blocks per SM at most.
+namespace {
+namespace tcax {
+
+template <int N>
+hb_status launch(const tc_args &A, cudaStream_t s, int64_t *nblocks)
+{
+    using C = shape<N>;
+    int dev = 0;
+    HB_TRY_CUDA(cudaGetDevice(&dev));
+    static int attr_set[64] = {0}, sms[64] = {0};
+    if (dev < 0 || dev >= 64) { hb_set_error("device index %d unsupported", dev); return HB_ERR_ARG; }
+    if (!attr_set[dev]) {
+        HB_TRY_CUDA(cudaFuncSetAttribute(ax_tc_kernel<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+        HB_TRY_CUDA(cudaFuncSetAttribute(ax_tc_kernel<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+        HB_TRY_CUDA(cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev));
+        attr_set[dev] = 1;
+    }
+    const int64_t ntiles = (A.E + C::EPT - 1) / C::EPT, room = (int64_t)C::BLOCKS * sms[dev];
+    const int64_t grid = ntiles < room ? ntiles : room;
+    if (nblocks) *nblocks = grid;
+    hb_prof_scope prof("ax_local", s);
+    if (A.spos) ax_tc_kernel<C, true><<<(unsigned)grid, C::THREADS, C::SMEM, s>>>(A);
+    else ax_tc_kernel<C, false><<<(unsigned)grid, C::THREADS, C::SMEM, s>>>(A);
+    HB_CHECK_LAUNCH();
+    return HB_OK;
+}
+
+}  // namespace tcax
+}  // namespace
+
+// Tensor-core FP64 element kernel (N = 3, 7, 15): interior DOFs finished here
+// (y, lambda term, partial of x.y per block), surface values to ysurf for the
+// surface gather. Persistent grid: the blocks that fit on every SM at most.
 hb_status hb_launch_ax_tc_f64(const hb_mesh *m, const double *x, double *ysurf, double *y, double lambda,
                               int screen, double *partials, const int *run, bool csr_store, cudaStream_t s,
                               int64_t *nblocks)
 {
     using namespace tcax;
-    if (m->N != N) { hb_set_error("the tensor-core element kernel is built for N = 7 only"); return HB_ERR_ARG; }
     if (!m->geo) { hb_set_error("mesh has no double geometric factors"); return HB_ERR_ARG; }
-    if (m->E <= 0) return HB_OK;
-    int dev = 0;
-    HB_TRY_CUDA(cudaGetDevice(&dev));
-    static int attr_set[64] = {0}, sms[64] = {0};
-    if (dev < 0 || dev >= 64) { hb_set_error("device index %d unsupported", dev); return HB_ERR_ARG; }
     if (csr_store && !m->spos) { hb_set_error("surface positions missing"); return HB_ERR_ARG; }
-    if (!attr_set[dev]) {
-        HB_TRY_CUDA(cudaFuncSetAttribute(ax_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
-        HB_TRY_CUDA(cudaFuncSetAttribute(ax_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
-        HB_TRY_CUDA(cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev));
-        attr_set[dev] = 1;
+    if (m->E <= 0) return HB_OK;
+    const tc_args A{x, m->l2g, m->geo, ysurf, y, m->E, run, lambda, screen, partials, m->counters + 7,
+                    csr_store ? m->spos : nullptr};
+    switch (m->N) {
+    case 3: return launch<3>(A, s, nblocks);
+    case 7: return launch<7>(A, s, nblocks);
+    case 15: return launch<15>(A, s, nblocks);
+    default: hb_set_error("the tensor-core element kernel is built for N = 3, 7 and 15"); return HB_ERR_ARG;
     }
-    const int64_t ntiles = (m->E + 1) / 2;
-    const int64_t grid = ntiles < 3 * (int64_t)sms[dev] ? ntiles : 3 * (int64_t)sms[dev];
-    if (nblocks) *nblocks = grid;
-    tc_args A{x, m->l2g, m->geo, ysurf, y, m->E, run, lambda, screen, partials, m->counters + 7,
-              csr_store ? m->spos : nullptr};
-    hb_prof_scope prof("ax_local", s);
-    if (csr_store) ax_tc_kernel<true><<<(unsigned)grid, THREADS, SMEM, s>>>(A);
-    else ax_tc_kernel<false><<<(unsigned)grid, THREADS, SMEM, s>>>(A);
-    HB_CHECK_LAUNCH();
-    return HB_OK;
 }

@@ -230,7 +230,8 @@ HB_VARIANT_PENCIL, HB_VARIANT_EVEN_ODD, HB_VARIANT_EB2, HB_VARIANT_ONE, HB_VARIA
     1, 2, 4, 8, 16, 32
 HB_VARIANT_CSR = 64
 HB_VARIANT_GRID = 128
-HB_VARIANT_TC = 256  # tensor-core element kernel (HB_F64, N = 7)
+HB_VARIANT_TC = 256  # tensor-core element kernel (HB_F64, the degrees of TC_DEGREES)
+TC_DEGREES = (3, 7, 15)
 VARIANTS_TC = [HB_VARIANT_TC, HB_VARIANT_TC | HB_VARIANT_CSR]  # alone, and with the CSR-position store
 VARIANTS = [0, 1, 3, 5, 7, 11, 19, 35, 67, 75, 131, 139]  # every valid combination of the pencil flags
 VARIANTS_F64X = [3, 11, 67, 75, 131, 139]  # the shapes the double-float kernel is built in
