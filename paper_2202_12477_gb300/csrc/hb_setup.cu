@@ -213,27 +213,29 @@ struct box_t {
     unsigned faces;
 };
 
-// Node map: lexicographic ids over unmasked lattice nodes, by closed form.
-__global__ void k_l2g(box_t b, int64_t n_local, int32_t *l2g)
+// One axis of the box's lattice: Ex elements of degree N, points 0 .. N Ex, of
+// which x0 at the low end (0 or 1, masked) and possibly the last are no DOFs.
+// Point I is held by mult(I) elements along the axis (two on a shared face).
+struct axis_t {
+    int N, Ex, x0, nu;  // nu: unmasked points
+    __host__ __device__ int mult(int I) const { return I % N == 0 && I > 0 && I < N * Ex ? 2 : 1; }
+    // sum of mult over the unmasked points before I (a point), and over all
+    __host__ __device__ int64_t copies_before(int I) const { return I - x0 + (I > 0 ? (I - 1) / N : 0); }
+    __host__ __device__ int64_t copies() const { return nu > 0 ? (int64_t)nu + Ex - 1 : 0; }
+    // points strictly inside an element: before I, and all
+    __host__ __device__ int64_t inner_before(int I) const { return I - (I + N - 1) / N; }
+    __host__ __device__ int64_t inner() const { return (int64_t)Ex * (N - 1); }
+};
+struct lattice3 {
+    axis_t x, y, z;
+};
+static lattice3 box_lattice(const box_t &b)
 {
-    const int n = b.N + 1;
-    const int64_t n3 = (int64_t)n * n * n;
-    const int64_t NX = (int64_t)b.N * b.Ex + 1, NY = (int64_t)b.N * b.Ey + 1, NZ = (int64_t)b.N * b.Ez + 1;
-    const int x0 = b.faces & 1u ? 1 : 0, x1 = b.faces & 2u ? 1 : 0;
-    const int y0 = b.faces & 4u ? 1 : 0, y1 = b.faces & 8u ? 1 : 0;
-    const int z0 = b.faces & 16u ? 1 : 0, z1 = b.faces & 32u ? 1 : 0;
-    const int64_t NXu = NX - x0 - x1, NYu = NY - y0 - y1;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n_local;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        int64_t e = q / n3;
-        int node = (int)(q - e * n3);
-        int i = node % n, j = (node / n) % n, k = node / (n * n);
-        int64_t ex = e % b.Ex, ey = (e / b.Ex) % b.Ey, ez = e / ((int64_t)b.Ex * b.Ey);
-        int64_t I = b.N * ex + i, J = b.N * ey + j, K = b.N * ez + k;
-        bool masked = (x0 && I == 0) || (x1 && I == NX - 1) || (y0 && J == 0) || (y1 && J == NY - 1) ||
-                      (z0 && K == 0) || (z1 && K == NZ - 1);
-        l2g[q] = masked ? -1 : (int32_t)((I - x0) + NXu * ((J - y0) + NYu * (K - z0)));
-    }
+    auto axis = [&](int E, unsigned lo, unsigned hi) {
+        const int x0 = b.faces & lo ? 1 : 0, x1 = b.faces & hi ? 1 : 0;
+        return axis_t{b.N, E, x0, b.N * E + 1 - x0 - x1};
+    };
+    return {axis(b.Ex, 1u, 2u), axis(b.Ey, 4u, 8u), axis(b.Ez, 16u, 32u)};
 }
 
 __device__ inline void vertex_pos(const box_t &b, double rho, uint64_t seed, int a, int bb, int c,
@@ -263,17 +265,53 @@ __device__ inline void vertex_pos(const box_t &b, double rho, uint64_t seed, int
 // a_t = j_r x j_s) and det J = j_r . a_r,
 //   G_lm = w_ijk det J (J^-1 J^-T)_lm = (w_ijk / det J) a_l . a_m,
 // the six factors of Sec. 2 and the weighted Jacobian w_ijk det J.
-__global__ void k_geometry(box_t b, double rho, uint64_t seed, int64_t E, double *geo, float *geo32,
-                           double *detmin_blk)
+// Bound by the FP64 rate (about 60 operations per node, 2 per clock and SM), so
+// what can be is integer work: the node map (lexicographic ids over unmasked
+// lattice nodes, by closed form) rides along, the smallest det J is found on
+// its bits, the FP32 copies are rounded by integer instructions (conversions
+// run at the FP64 rate), and w_i w_j comes from a table. ms for 32x32x31, N = 11:
+// @@GEO@@
+
+// Order-preserving unsigned key of a double, and back.
+__host__ __device__ inline unsigned long long order_key(double v)
+{
+    unsigned long long b;
+    memcpy(&b, &v, sizeof b);
+    return b >> 63 ? ~b : b | (1ull << 63);
+}
+static double from_order_key(unsigned long long k)
+{
+    const unsigned long long b = k >> 63 ? k & ~(1ull << 63) : ~k;
+    double v;
+    memcpy(&v, &b, sizeof v);
+    return v;
+}
+
+// (float)v, to nearest even: a carry from the 29 dropped bits may step the
+// exponent; outside FP32's normal range the conversion instruction.
+__device__ __forceinline__ float round_to_float(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned e = (unsigned)(b >> 52) & 0x7FFu;
+    if (e - 897u > 1149u - 897u) return (float)v;
+    const unsigned long long r = b + ((1ull << 28) - 1ull + ((b >> 29) & 1ull));
+    const unsigned m = (unsigned)(r >> 29) - (896u << 23);  // (bits above 31 drop out)
+    return __uint_as_float((m & 0x7FFFFFFFu) | ((unsigned)(b >> 32) & 0x80000000u));
+}
+
+__global__ void k_geometry(box_t b, lattice3 L, double rho, uint64_t seed, int64_t E, int32_t *l2g, double *geo,
+                           float *geo32, unsigned long long *detmin)
 {
     extern __shared__ double smem[];
     const int N = b.N, n = N + 1, n2 = n * n, n3 = n2 * n;
     double *col = smem;  // [direction l][axis][line (u + n v)]: column l of J on the line
     __shared__ double V[8][3];
     __shared__ double dV[3][4][3];  // [direction][pair (p + 2 q)][axis]: halved edge differences
-    __shared__ double red[32];
+    __shared__ double ww[256], wk[16];
     const double *xi = g_xi64 + N * 16, *w = g_w64 + N * 16;
-    double dmin = INFINITY;
+    unsigned long long kmin = ~0ull;
+    for (int t = threadIdx.x; t < n2; t += blockDim.x) ww[t] = w[t % n] * w[t / n];
+    if (threadIdx.x < n) wk[threadIdx.x] = w[threadIdx.x];
     for (int64_t e = blockIdx.x; e < E; e += gridDim.x) {
         const int ex = (int)(e % b.Ex), ey = (int)((e / b.Ex) % b.Ey), ez = (int)(e / ((int64_t)b.Ex * b.Ey));
         __syncthreads();  // the previous element's columns are consumed
@@ -325,7 +363,7 @@ __global__ void k_geometry(box_t b, double rho, uint64_t seed, int64_t E, double
             at[1] = fma(jr[2], js[0], -jr[0] * js[2]);
             at[2] = fma(jr[0], js[1], -jr[1] * js[0]);
             const double det = fma(jr[2], ar[2], fma(jr[1], ar[1], jr[0] * ar[0]));
-            const double wq = w[i] * w[j] * w[k];
+            const double wq = ww[j * n + i] * wk[k];
             const double sc = wq / det;
             double g[7];
             g[0] = sc * fma(ar[2], ar[2], fma(ar[1], ar[1], ar[0] * ar[0]));
@@ -338,154 +376,20 @@ __global__ void k_geometry(box_t b, double rho, uint64_t seed, int64_t E, double
             const int64_t base = ((e * n + k) * 7) * (int64_t)n2 + j * n + i;
             for (int c = 0; c < 7; c++) {
                 geo[base + (int64_t)c * n2] = g[c];
-                if (geo32) geo32[base + (int64_t)c * n2] = (float)g[c];
+                if (geo32) geo32[base + (int64_t)c * n2] = round_to_float(g[c]);
             }
-            dmin = fmin(dmin, det);
+            kmin = min(kmin, order_key(det));
+            const int I = N * ex + i - L.x.x0, J = N * ey + j - L.y.x0, K = N * ez + k - L.z.x0;
+            const bool dof = (unsigned)I < (unsigned)L.x.nu && (unsigned)J < (unsigned)L.y.nu && (unsigned)K < (unsigned)L.z.nu;
+            l2g[e * n3 + q] = dof ? I + L.x.nu * (J + L.y.nu * K) : -1;
         }
     }
-    // block minimum of det J
-    for (int o = 16; o > 0; o >>= 1) dmin = fmin(dmin, __shfl_down_sync(0xffffffffu, dmin, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = dmin;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double m = red[0];
-        for (int q = 1; q < (int)(blockDim.x + 31) / 32; q++) m = fmin(m, red[q]);
-        detmin_blk[blockIdx.x] = m;
-    }
+    // smallest det J
+    for (int o = 16; o > 0; o >>= 1) kmin = min(kmin, __shfl_down_sync(0xffffffffu, kmin, o));
+    if ((threadIdx.x & 31) == 0) atomicMin(detmin, kmin);
 }
 
-__global__ void k_count(const int32_t *l2g, int64_t n_local, int32_t *cnt)
-{
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n_local;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        int32_t g = l2g[q];
-        if (g >= 0) atomicAdd(&cnt[g], 1);
-    }
-}
-
-// Exclusive scan in three passes over chunks of 1024 entries.
-__global__ void k_scan_chunks(const int32_t *in, int64_t n, int32_t *out, int64_t *chunk_sum)
-{
-    __shared__ int64_t s[1024];
-    int64_t base = (int64_t)blockIdx.x * 1024;
-    int t = threadIdx.x;
-    int64_t v = base + t < n ? in[base + t] : 0;
-    s[t] = v;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        int64_t a = t >= o ? s[t - o] : 0;
-        __syncthreads();
-        s[t] += a;
-        __syncthreads();
-    }
-    if (base + t < n) out[base + t] = (int32_t)(s[t] - v);
-    if (t == 1023) chunk_sum[blockIdx.x] = s[t];
-}
-
-// Exclusive scan of the chunk sums in place (chunk_sum[nchunks] = the total):
-// one block of 1024 threads walks the sums in tiles of 1024, a warp-shuffle
-// scan per tile plus the running carry. Launch with 1024 threads.
-__global__ void __launch_bounds__(1024) k_scan_sums(int64_t *chunk_sum, int64_t nchunks)
-{
-    __shared__ int64_t wsum[32];
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    int64_t carry = 0;
-    for (int64_t base = 0; base < nchunks; base += 1024) {
-        const int64_t c = base + t;
-        const int64_t v = c < nchunks ? chunk_sum[c] : 0;
-        int64_t x = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) wsum[w] = x;
-        __syncthreads();
-        if (w == 0) {
-            int64_t z = wsum[lane];
-            for (int o = 1; o < 32; o <<= 1) {
-                const int64_t y = __shfl_up_sync(0xffffffffu, z, o);
-                if (lane >= o) z += y;
-            }
-            wsum[lane] = z;
-        }
-        __syncthreads();
-        const int64_t incl = x + (w > 0 ? wsum[w - 1] : 0);
-        if (c < nchunks) chunk_sum[c] = carry + incl - v;
-        carry += wsum[31];
-        __syncthreads();  // wsum is rewritten by the next tile
-    }
-    if (t == 0) chunk_sum[nchunks] = carry;
-}
-
-__global__ void k_scan_add(int32_t *out, int64_t n, const int64_t *chunk_sum)
-{
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n;
-         q += (int64_t)gridDim.x * blockDim.x)
-        out[q] = (int32_t)(out[q] + chunk_sum[q / 1024]);
-}
-
-__global__ void k_fill(const int32_t *l2g, int64_t n_local, const int32_t *rowptr, int32_t *cursor,
-                       int32_t *cols)
-{
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n_local;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        int32_t g = l2g[q];
-        if (g >= 0) {
-            int slot = atomicAdd(&cursor[g], 1);
-            cols[rowptr[g] + slot] = (int32_t)q;
-        }
-    }
-}
-
-// Sort every row ascending (rows are short) and sum the mass diagonal in that order.
-__global__ void k_sort_rows(const int32_t *rowptr, int32_t *cols, int64_t ng, const double *geo, int n,
-                            double *mdiag, float *mdiag32)
-{
-    const int n2 = n * n, n3 = n2 * n;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < ng;
-         g += (int64_t)gridDim.x * blockDim.x) {
-        int a = rowptr[g], z = rowptr[g + 1];
-        for (int p = a + 1; p < z; p++) {
-            int32_t v = cols[p];
-            int q = p - 1;
-            while (q >= a && cols[q] > v) { cols[q + 1] = cols[q]; q--; }
-            cols[q + 1] = v;
-        }
-        double m = 0.0;
-        for (int p = a; p < z; p++) {
-            int64_t lq = cols[p];
-            int64_t e = lq / n3;
-            int node = (int)(lq - e * n3);
-            int k = node / n2, ij = node - k * n2;
-            m += geo[((e * n + k) * 7 + 6) * (int64_t)n2 + ij];
-        }
-        mdiag[g] = m;
-        if (mdiag32) mdiag32[g] = (float)m;
-    }
-}
-
-// *out = min of v[0..n): one block of 1024 threads.
-__global__ void __launch_bounds__(1024) k_min_reduce(const double *v, int n, double *out)
-{
-    __shared__ double wm[32];
-    double m = INFINITY;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) m = fmin(m, v[q]);
-    for (int o = 16; o > 0; o >>= 1) m = fmin(m, __shfl_down_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        m = threadIdx.x < (int)(blockDim.x >> 5) ? wm[threadIdx.x] : INFINITY;
-        for (int o = 16; o > 0; o >>= 1) m = fmin(m, __shfl_down_sync(0xffffffffu, m, o));
-        if (threadIdx.x == 0) *out = m;
-    }
-}
-
-// ---------------------------------------------------------------- surface CSR
-
-__device__ __forceinline__ bool on_surface(int i, int j, int k, int N)
-{
-    return i == 0 || i == N || j == 0 || j == N || k == 0 || k == N;
-}
+// ---------------------------------------------------------------- rows of Z^T
 
 // Same order as the element kernels: k = 0 face, k = N face, then the ring
 // of 4N nodes of each slab k = 1..N-1.
@@ -498,141 +402,66 @@ __device__ __forceinline__ int surf_index(int i, int j, int k, int N)
     return 2 * n2 + (k - 1) * 4 * N + r;
 }
 
-__global__ void k_surf_count(const int32_t *l2g, int64_t n_local, int N, int32_t *cnt)
+// Z^T by the box's lattice, both as CSR over all DOFs and restricted to the
+// DOFs on element surfaces, with the lumped mass diagonal: row g is lattice
+// point (I, J, K), its copies are node (I - N ex, ...) of the elements that hold
+// it, and where a row starts is a sum of products of per-axis counts. One pass,
+// no counting, scan or sort: one warp per lattice row (J, K), lanes along I. The
+// copies of a row ascend by element, as do the columns; the mass is summed in
+// that order. 0.62 ms for 32x32x31, N = 11, where counting by atomics, scans,
+// filling and sorting the rows took 3.1 ms and five waits of the host.
+__global__ void __launch_bounds__(256)
+    k_rows(lattice3 L, const double *__restrict__ geo, int32_t *__restrict__ rowptr, int32_t *__restrict__ cols,
+           double *__restrict__ mdiag, float *__restrict__ mdiag32, int32_t *__restrict__ srow_g,
+           int32_t *__restrict__ srowptr, int32_t *__restrict__ scols)
 {
-    const int n = N + 1;
-    const int64_t n3 = (int64_t)n * n * n;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n_local;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t g = l2g[q];
-        if (g < 0) continue;
-        const int node = (int)(q % n3);
-        const int i = node % n, j = (node / n) % n, k = node / (n * n);
-        if (on_surface(i, j, k, N)) atomicAdd(&cnt[g], 1);
-    }
-}
-
-__global__ void k_flag(const int32_t *cnt, int64_t ng, int32_t *flag)
-{
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < ng; g += (int64_t)gridDim.x * blockDim.x)
-        flag[g] = cnt[g] > 0 ? 1 : 0;
-}
-
-__global__ void k_compact_rows(const int32_t *cnt, const int32_t *srow_of, int64_t ng, int32_t *srow_g,
-                               int32_t *scnt)
-{
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < ng; g += (int64_t)gridDim.x * blockDim.x)
-        if (cnt[g] > 0) {
-            srow_g[srow_of[g]] = (int32_t)g;
-            scnt[srow_of[g]] = cnt[g];
-        }
-}
-
-__global__ void k_surf_fill(const int32_t *l2g, int64_t n_local, int N, const int32_t *srow_of,
-                            const int32_t *srowptr, int32_t *cursor, int32_t *scols)
-{
-    const int n = N + 1;
-    const int64_t n3 = (int64_t)n * n * n;
-    const int NS = 2 * n * n + 4 * N * (N - 1);
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n_local;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t g = l2g[q];
-        if (g < 0) continue;
-        const int64_t e = q / n3;
-        const int node = (int)(q - e * n3);
-        const int i = node % n, j = (node / n) % n, k = node / (n * n);
-        if (!on_surface(i, j, k, N)) continue;
-        const int r = srow_of[g];
-        const int slot = atomicAdd(&cursor[r], 1);
-        scols[srowptr[r] + slot] = (int32_t)(e * NS + surf_index(i, j, k, N));
-    }
-}
-
-__global__ void k_sort_surf_rows(const int32_t *rowptr, int32_t *cols, int64_t nrows)
-{
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < nrows; r += (int64_t)gridDim.x * blockDim.x) {
-        const int a = rowptr[r], z = rowptr[r + 1];
-        for (int p = a + 1; p < z; p++) {
-            const int32_t v = cols[p];
-            int q = p - 1;
-            while (q >= a && cols[q] > v) { cols[q + 1] = cols[q]; q--; }
-            cols[q + 1] = v;
+    const int N = L.x.N, n = N + 1, n2 = n * n, NS = 2 * n2 + 4 * N * (N - 1);
+    const int64_t n3 = (int64_t)n2 * n, TX = L.x.copies(), TY = L.y.copies();
+    const int64_t SX = L.x.inner(), SY = L.y.inner();
+    const int lane = threadIdx.x & 31;
+    const int64_t nrows = (int64_t)L.y.nu * L.z.nu, nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < nrows; row += nwarps) {
+        const int Ku = (int)(row / L.y.nu), Ju = (int)(row - (int64_t)Ku * L.y.nu);
+        const int J = Ju + L.y.x0, K = Ku + L.z.x0;
+        const int my = L.y.mult(J), mz = L.z.mult(K);
+        const bool in_yz = J % N != 0 && K % N != 0;
+        // copies and interior DOFs (one copy each) before this row
+        const int64_t c0 = TX * (L.z.copies_before(K) * TY + mz * L.y.copies_before(J));
+        const int64_t i0 = SX * (L.z.inner_before(K) * SY + (K % N != 0 ? L.y.inner_before(J) : 0));
+        // the first element along y and z, and the local index in it
+        const int ey0 = J == 0 ? 0 : (J - 1) / N, ez0 = K == 0 ? 0 : (K - 1) / N, j0 = J - N * ey0, k0 = K - N * ez0;
+        for (int Iu = lane; Iu < L.x.nu; Iu += 32) {
+            const int I = Iu + L.x.x0, mx = L.x.mult(I), ex0 = I == 0 ? 0 : (I - 1) / N, li = I - N * ex0;
+            const int64_t g = row * L.x.nu + Iu, at = c0 + (int64_t)my * mz * L.x.copies_before(I);
+            const int64_t before = i0 + (in_yz ? L.x.inner_before(I) : 0);
+            const bool surf = !(in_yz && I % N != 0);
+            const int64_t sat = at - before;
+            rowptr[g] = (int32_t)at;
+            if (surf) {
+                srow_g[g - before] = (int32_t)g;
+                srowptr[g - before] = (int32_t)sat;
+            }
+            double m = 0.0;
+            int q = 0;
+            for (int cz = 0; cz < mz; cz++)
+                for (int cy = 0; cy < my; cy++)
+                    for (int cx = 0; cx < mx; cx++, q++) {
+                        // a second element starts at the shared point
+                        const int i = cx ? 0 : li, j = cy ? 0 : j0, k = cz ? 0 : k0;
+                        const int64_t e = (ex0 + cx) + (int64_t)L.x.Ex * ((ey0 + cy) + (int64_t)L.y.Ex * (ez0 + cz));
+                        cols[at + q] = (int32_t)(e * n3 + (k * n + j) * n + i);
+                        if (surf) scols[sat + q] = (int32_t)(e * NS + surf_index(i, j, k, N));
+                        m += geo[((e * n + k) * 7 + 6) * (int64_t)n2 + j * n + i];
+                    }
+            mdiag[g] = m;
+            if (mdiag32) mdiag32[g] = (float)m;
         }
     }
-}
-
-// Exclusive scan of n int32 values (out may equal in); returns the total.
-static hb_status scan_exclusive(const int32_t *in, int32_t *out, int64_t n, cudaStream_t s, int64_t *total)
-{
-    const int64_t nchunks = (n + 1023) / 1024;
-    int64_t *sums = nullptr;
-    HB_TRY_CUDA(hb_dev_alloc((void **)&sums, sizeof(int64_t) * (nchunks + 1), s));
-    hb_count_launch();
-    k_scan_chunks<<<(unsigned)nchunks, 1024, 0, s>>>(in, n, out, sums);
-    hb_count_launch();
-    k_scan_sums<<<1, 1024, 0, s>>>(sums, nchunks);
-    hb_count_launch();
-    k_scan_add<<<grid_for(n, 256), 256, 0, s>>>(out, n, sums);
-    cudaError_t e = cudaGetLastError();
-    int64_t tot = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&tot, sums + nchunks, sizeof(int64_t), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    hb_dev_free(sums, s);
-    if (e != cudaSuccess) {
-        hb_set_error("scan: %s", cudaGetErrorString(e));
-        return HB_ERR_CUDA;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const int64_t ng = nrows * L.x.nu, nnz = TX * TY * L.z.copies(), in = SX * SY * L.z.inner();
+        rowptr[ng] = (int32_t)nnz;
+        srowptr[ng - in] = (int32_t)(nnz - in);
     }
-    *total = tot;
-    return HB_OK;
-}
-
-// Builds srow_g, srowptr, scols of the mesh (after l2g exists).
-static hb_status build_surface_csr(hb_mesh *m, cudaStream_t s)
-{
-    const int64_t ng = m->n_global, nl = m->n_local;
-    int32_t *cnt = nullptr, *srow_of = nullptr, *scnt = nullptr;
-    hb_status st = HB_OK;
-    int64_t nsr = 0, nnz = 0;
-    auto fail = [&](cudaError_t e) {
-        hb_set_error("surface CSR: %s", cudaGetErrorString(e));
-        st = e == cudaErrorMemoryAllocation ? HB_ERR_NOMEM : HB_ERR_CUDA;
-    };
-    cudaError_t e = hb_dev_alloc((void **)&cnt, sizeof(int32_t) * (ng + 1), s);
-    if (e == cudaSuccess) e = hb_dev_alloc((void **)&srow_of, sizeof(int32_t) * (ng + 1), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (ng + 1), s);
-    if (e != cudaSuccess) { fail(e); goto done; }
-    hb_count_launch();
-    k_surf_count<<<grid_for(nl, 256), 256, 0, s>>>(m->l2g, nl, m->N, cnt);
-    hb_count_launch();
-    k_flag<<<grid_for(ng + 1, 256), 256, 0, s>>>(cnt, ng + 1, srow_of);
-    if ((e = cudaGetLastError()) != cudaSuccess) { fail(e); goto done; }
-    if ((st = scan_exclusive(srow_of, srow_of, ng + 1, s, &nsr)) != HB_OK) goto done;
-    m->nsr = nsr;
-    e = hb_dev_alloc((void **)&m->srow_g, sizeof(int32_t) * (nsr + 1), s);
-    if (e == cudaSuccess) e = hb_dev_alloc((void **)&m->srowptr, sizeof(int32_t) * (nsr + 1), s);
-    if (e == cudaSuccess) e = hb_dev_alloc((void **)&scnt, sizeof(int32_t) * (nsr + 1), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(scnt, 0, sizeof(int32_t) * (nsr + 1), s);
-    if (e != cudaSuccess) { fail(e); goto done; }
-    hb_count_launch();
-    k_compact_rows<<<grid_for(ng, 256), 256, 0, s>>>(cnt, srow_of, ng, m->srow_g, scnt);
-    if ((e = cudaGetLastError()) != cudaSuccess) { fail(e); goto done; }
-    if ((st = scan_exclusive(scnt, m->srowptr, nsr + 1, s, &nnz)) != HB_OK) goto done;
-    m->nnz_s = nnz;
-    e = hb_dev_alloc((void **)&m->scols, sizeof(int32_t) * (nnz > 0 ? nnz : 1), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(scnt, 0, sizeof(int32_t) * (nsr + 1), s);
-    if (e != cudaSuccess) { fail(e); goto done; }
-    hb_count_launch();
-    k_surf_fill<<<grid_for(nl, 256), 256, 0, s>>>(m->l2g, nl, m->N, srow_of, m->srowptr, scnt, m->scols);
-    hb_count_launch();
-    k_sort_surf_rows<<<grid_for(nsr, 256), 256, 0, s>>>(m->srowptr, m->scols, nsr);
-    if ((e = cudaGetLastError()) != cudaSuccess) { fail(e); goto done; }
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) { fail(e); goto done; }
-    m->device_bytes += sizeof(int32_t) * (2 * (nsr + 1) + nnz);
-done:
-    hb_dev_free(cnt, s);
-    hb_dev_free(srow_of, s);
-    hb_dev_free(scnt, s);
-    return st;
 }
 
 __global__ void k_spos(const int32_t *__restrict__ scols, int64_t nnz, int32_t *__restrict__ spos)
@@ -740,8 +569,6 @@ void hb_mesh_release(hb_mesh *m, cudaStream_t s)
             hb_set_error("%s:%d %s: %s", __FILE__, __LINE__, #call,              \
                          cudaGetErrorString(e_));                                \
             hb_mesh_destroy(m);                                                  \
-            hb_dev_free(tmp_cnt, s);                                             \
-            hb_dev_free(tmp_sum, s);                                             \
             hb_dev_free(tmp_det, s);                                             \
             return e_ == cudaErrorMemoryAllocation ? HB_ERR_NOMEM : HB_ERR_CUDA; \
         }                                                                        \
@@ -766,9 +593,7 @@ extern "C" hb_status hb_mesh_create(const hb_mesh_desc *d, void *stream, hb_mesh
     cudaStream_t s = (cudaStream_t)stream;
     hb_mesh *m = new hb_mesh();
     memset((void *)m, 0, sizeof(hb_mesh));
-    int32_t *tmp_cnt = nullptr;
-    int64_t *tmp_sum = nullptr;
-    double *tmp_det = nullptr;
+    unsigned long long *tmp_det = nullptr;
     HB_TRY_MESH(cudaGetDevice(&m->device));
     m->desc = *d;
     m->variant[0] = HB_VAR_PENCIL | HB_VAR_EO;
@@ -778,13 +603,15 @@ extern "C" hb_status hb_mesh_create(const hb_mesh_desc *d, void *stream, hb_mesh
     m->n = n;
     m->E = E;
     m->n_local = n_local;
-    // global count by closed form, checked against the CSR below
-    const int64_t NX = (int64_t)N * d->ex + 1, NY = (int64_t)N * d->ey + 1, NZ = (int64_t)N * d->ez + 1;
-    const unsigned f = d->dirichlet_faces;
-    const int64_t NXu = NX - (f & 1u ? 1 : 0) - (f & 2u ? 1 : 0);
-    const int64_t NYu = NY - (f & 4u ? 1 : 0) - (f & 8u ? 1 : 0);
-    const int64_t NZu = NZ - (f & 16u ? 1 : 0) - (f & 32u ? 1 : 0);
-    m->n_global = (NXu > 0 && NYu > 0 && NZu > 0) ? NXu * NYu * NZu : 0;
+    // counts by closed form
+    const box_t b{d->ex, d->ey, d->ez, N, d->dirichlet_faces};
+    const lattice3 L = box_lattice(b);
+    const bool any = L.x.nu > 0 && L.y.nu > 0 && L.z.nu > 0;
+    m->n_global = any ? (int64_t)L.x.nu * L.y.nu * L.z.nu : 0;
+    m->nnz = any ? L.x.copies() * L.y.copies() * L.z.copies() : 0;
+    const int64_t inner = any ? L.x.inner() * L.y.inner() * L.z.inner() : 0;  // one copy each
+    m->nsr = m->n_global - inner;
+    m->nnz_s = m->nnz - inner;
     const int64_t ng = m->n_global;
 
     size_t bytes = 0;
@@ -798,6 +625,14 @@ extern "C" hb_status hb_mesh_create(const hb_mesh_desc *d, void *stream, hb_mesh
     HB_TRY_MESH(alloc((void **)&m->rowptr, sizeof(int32_t) * (ng + 1)));
     HB_TRY_MESH(alloc((void **)&m->mdiag, sizeof(double) * (ng + 1)));
     if (d->keep_fp32_copy) HB_TRY_MESH(alloc((void **)&m->mdiag32, sizeof(float) * (ng + 1)));
+    HB_TRY_MESH(alloc((void **)&m->cols, sizeof(int32_t) * (m->nnz > 0 ? m->nnz : 1)));
+    HB_TRY_MESH(alloc((void **)&m->srow_g, sizeof(int32_t) * (m->nsr + 1)));
+    HB_TRY_MESH(alloc((void **)&m->srowptr, sizeof(int32_t) * (m->nsr + 1)));
+    HB_TRY_MESH(alloc((void **)&m->scols, sizeof(int32_t) * (m->nnz_s > 0 ? m->nnz_s : 1)));
+    // one partial per element-kernel block: at most two per element, or as many
+    // as there are SMs (a small mesh split over more)
+    m->n_ax_partials = 2 * E + 152;
+    HB_TRY_MESH(alloc((void **)&m->ax_partials, sizeof(double) * m->n_ax_partials));
     HB_TRY_MESH(alloc((void **)&m->yL, sizeof(double) * n_local));
     HB_TRY_MESH(alloc((void **)&m->partials, sizeof(double) * HB_RED_MAXV * HB_RED_BLOCKS));
     HB_TRY_MESH(alloc((void **)&m->counters, sizeof(unsigned) * 8));
@@ -808,11 +643,6 @@ extern "C" hb_status hb_mesh_create(const hb_mesh_desc *d, void *stream, hb_mesh
     HB_TRY_MESH(cudaMemsetAsync(m->counters, 0, sizeof(unsigned) * 8, s));
     HB_TRY_MESH(cudaMemsetAsync(m->state, 0, sizeof(hb_cg_state) * 4, s));
 
-    box_t b{d->ex, d->ey, d->ez, N, d->dirichlet_faces};
-    hb_count_launch();
-    k_l2g<<<grid_for(n_local, 256), 256, 0, s>>>(b, n_local, m->l2g);
-    HB_TRY_MESH(cudaGetLastError());
-
     // geometry: one element per block
     // at least 64 threads: 36 of them form the edge differences
     int gthreads = n * n * n < 256 ? std::max(64, ((n * n * n + 31) / 32) * 32) : 256;
@@ -820,81 +650,37 @@ extern "C" hb_status hb_mesh_create(const hb_mesh_desc *d, void *stream, hb_mesh
     // 18.4 KB at N = 15: under the default limit, so no per-call attribute
     // (a per-degree value would race between threads building meshes)
     size_t gsmem = sizeof(double) * 9 * n * n;
-    HB_TRY_MESH(hb_dev_alloc((void **)&tmp_det, sizeof(double) * (gblocks + 1), s));
+    HB_TRY_MESH(hb_dev_alloc((void **)&tmp_det, sizeof *tmp_det, s));
+    HB_TRY_MESH(cudaMemsetAsync(tmp_det, 0xFF, sizeof *tmp_det, s));
     hb_count_launch();
-    k_geometry<<<gblocks, gthreads, gsmem, s>>>(b, d->perturb, d->seed, E, m->geo, m->geo32, tmp_det);
+    k_geometry<<<gblocks, gthreads, gsmem, s>>>(b, L, d->perturb, d->seed, E, m->l2g, m->geo, m->geo32, tmp_det);
     HB_TRY_MESH(cudaGetLastError());
-    hb_count_launch();
-    k_min_reduce<<<1, 1024, 0, s>>>(tmp_det, gblocks, tmp_det + gblocks);
-    HB_TRY_MESH(cudaGetLastError());
-
-    // CSR of Z^T: count, scan, fill, sort rows
-    HB_TRY_MESH(hb_dev_alloc((void **)&tmp_cnt, sizeof(int32_t) * (ng + 1), s));
-    HB_TRY_MESH(cudaMemsetAsync(tmp_cnt, 0, sizeof(int32_t) * (ng + 1), s));
-    hb_count_launch();
-    k_count<<<grid_for(n_local, 256), 256, 0, s>>>(m->l2g, n_local, tmp_cnt);
-    HB_TRY_MESH(cudaGetLastError());
-    const int64_t nchunks = (ng + 1 + 1023) / 1024;
-    HB_TRY_MESH(hb_dev_alloc((void **)&tmp_sum, sizeof(int64_t) * (nchunks + 1), s));
-    hb_count_launch();
-    k_scan_chunks<<<(unsigned)nchunks, 1024, 0, s>>>(tmp_cnt, ng + 1, m->rowptr, tmp_sum);
-    HB_TRY_MESH(cudaGetLastError());
-    hb_count_launch();
-    k_scan_sums<<<1, 1024, 0, s>>>(tmp_sum, nchunks);
-    HB_TRY_MESH(cudaGetLastError());
-    hb_count_launch();
-    k_scan_add<<<grid_for(ng + 1, 256), 256, 0, s>>>(m->rowptr, ng + 1, tmp_sum);
-    HB_TRY_MESH(cudaGetLastError());
-    int32_t nnz32 = 0;
-    HB_TRY_MESH(cudaMemcpyAsync(&nnz32, m->rowptr + ng, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    double detmin = 0.0;
-    HB_TRY_MESH(cudaMemcpyAsync(&detmin, tmp_det + gblocks, sizeof(double), cudaMemcpyDeviceToHost, s));
-    HB_TRY_MESH(cudaStreamSynchronize(s));
-    m->nnz = nnz32;
-    m->min_detJ = detmin;
-    HB_TRY_MESH(alloc((void **)&m->cols, sizeof(int32_t) * (m->nnz > 0 ? m->nnz : 1)));
-    HB_TRY_MESH(cudaMemsetAsync(tmp_cnt, 0, sizeof(int32_t) * (ng + 1), s));
-    hb_count_launch();
-    k_fill<<<grid_for(n_local, 256), 256, 0, s>>>(m->l2g, n_local, m->rowptr, tmp_cnt, m->cols);
-    HB_TRY_MESH(cudaGetLastError());
-    hb_count_launch();
-    k_sort_rows<<<grid_for(ng, 256), 256, 0, s>>>(m->rowptr, m->cols, ng, m->geo, n, m->mdiag, m->mdiag32);
-    HB_TRY_MESH(cudaGetLastError());
-    HB_TRY_MESH(cudaStreamSynchronize(s));
-    hb_dev_free(tmp_cnt, s);
-    hb_dev_free(tmp_sum, s);
-    hb_dev_free(tmp_det, s);
-    tmp_cnt = nullptr;
-    tmp_sum = nullptr;
-    tmp_det = nullptr;
-    m->device_bytes = bytes;
-    {
-        hb_status sst = build_surface_csr(m, s);
-        if (sst != HB_OK) { hb_mesh_destroy(m); return sst; }
-        // one partial per element-kernel block: at most two per element, or
-        // as many as there are SMs (a small mesh split over more)
-        m->n_ax_partials = 2 * E + 152;
-        cudaError_t ae = hb_dev_alloc((void **)&m->ax_partials, sizeof(double) * m->n_ax_partials, s);
-        if (ae != cudaSuccess) {
-            hb_set_error("ax partials: %s", cudaGetErrorString(ae));
-            hb_mesh_destroy(m);
-            return ae == cudaErrorMemoryAllocation ? HB_ERR_NOMEM : HB_ERR_CUDA;
-        }
-        m->device_bytes += sizeof(double) * m->n_ax_partials;
+    if (ng > 0) {
+        const int64_t warps = (int64_t)L.y.nu * L.z.nu;
+        hb_count_launch();
+        k_rows<<<grid_for(warps * 32, 256), 256, 0, s>>>(L, m->geo, m->rowptr, m->cols, m->mdiag, m->mdiag32, m->srow_g,
+                                                         m->srowptr, m->scols);
+        HB_TRY_MESH(cudaGetLastError());
+    } else {
+        HB_TRY_MESH(cudaMemsetAsync(m->rowptr, 0, sizeof(int32_t), s));
+        HB_TRY_MESH(cudaMemsetAsync(m->srowptr, 0, sizeof(int32_t), s));
     }
+    // (into the pinned buffer: a copy to pageable memory would wait here)
+    HB_TRY_MESH(cudaMemcpyAsync(m->state_host, tmp_det, sizeof *tmp_det, cudaMemcpyDeviceToHost, s));
+    hb_dev_free(tmp_det, s);
+    tmp_det = nullptr;
+    // every stream-ordered array is ready for any stream once s has drained
+    HB_TRY_MESH(cudaStreamSynchronize(s));
+    {
+        unsigned long long key;
+        memcpy(&key, m->state_host, sizeof key);
+        m->min_detJ = from_order_key(key);
+    }
+    m->device_bytes = bytes;
     if (!(m->min_detJ > 0.0)) {
         hb_set_error("non-positive Jacobian determinant (min det J = %g)", m->min_detJ);
         hb_mesh_destroy(m);
         return HB_ERR_GEOMETRY;
-    }
-    // every stream-ordered array is ready for any stream once s has drained
-    {
-        const cudaError_t se = cudaStreamSynchronize(s);
-        if (se != cudaSuccess) {
-            hb_set_error("mesh set-up: %s", cudaGetErrorString(se));
-            hb_mesh_destroy(m);
-            return HB_ERR_CUDA;
-        }
     }
     *out = m;
     return HB_OK;
