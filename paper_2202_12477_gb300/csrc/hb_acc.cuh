@@ -3,6 +3,16 @@
 
 namespace hbacc {
 
+// First statement of a kernel that hb_launch_after starts: waits until every
+// kernel before it on the stream is complete and its writes are visible (a
+// kernel that an ordinary launch started is so already), then lets the next
+// one's blocks start as soon as all blocks of this grid run.
+__device__ __forceinline__ void wait_before()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // FP64 accumulation of products. For FP32 operands the FP64 pipe of GB300 is
 // slow, so the running sum is carried as an unevaluated pair of floats with
 // error-free transformations (Dekker's two-product via fma, Knuth's two-sum):

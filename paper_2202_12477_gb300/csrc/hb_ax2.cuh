@@ -902,6 +902,7 @@ __device__ __forceinline__ bool pencil_split(const pencil_args &A, int64_t e, in
 template <int N>
 __global__ void __launch_bounds__(split<N>::MAXT) ax_split_kernel(const pencil_args A, int C)
 {
+    hbacc::wait_before();
     if (A.run && *A.run == 0) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     hbacc::dot_acc<S> acc;
@@ -1107,16 +1108,25 @@ hb_status launch(const pencil_args &A, int eb_mode, cudaStream_t s, int64_t *nbl
                 }
                 if (nblocks_out) *nblocks_out = A.E * C;
                 cudaLaunchConfig_t cfg = {};
-                cudaLaunchAttribute at[1];
-                at[0].id = cudaLaunchAttributeClusterDimension;
-                at[0].val.clusterDim.x = C;
-                at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+                cudaLaunchAttribute at[2];
+                int na = 0;
+                if (C > 1) {
+                    at[na].id = cudaLaunchAttributeClusterDimension;
+                    at[na].val.clusterDim.x = C;
+                    at[na].val.clusterDim.y = at[na].val.clusterDim.z = 1;
+                    na++;
+                }
+                if (hb_overlap_launch(s)) {  // (as hb_launch_after)
+                    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+                    at[na].val.programmaticStreamSerializationAllowed = 1;
+                    na++;
+                }
                 cfg.gridDim = dim3((unsigned)(A.E * C));
                 cfg.blockDim = dim3((unsigned)split<N>::threads(C));
                 cfg.dynamicSmemBytes = split<N>::smem(C);
                 cfg.stream = s;
                 cfg.attrs = at;
-                cfg.numAttrs = C > 1 ? 1 : 0;
+                cfg.numAttrs = na;
                 hb_prof_scope prof("ax_local", s);
                 HB_TRY_CUDA(cudaLaunchKernelEx(&cfg, kern, A, C));
                 return HB_OK;

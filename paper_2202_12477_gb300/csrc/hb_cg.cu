@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(HB_RED_THREADS)
                          int64_t nrows, const double *__restrict__ ax_partials, int64_t n_axp, double *partials,
                          unsigned *counter, hb_cg_state *st)
 {
+    if (DOT == HB_DOT_NONE) hbacc::wait_before();  // (the launches of A x alone)
     assemble_surf_body<T, SCREEN, DOT, CONTIG, WIDE>(ys, srow_g, rowptr, cols, x, mdiag, lambda, y, nrows,
                                                      ax_partials, n_axp, partials, counter, st);
 }
@@ -157,6 +158,7 @@ hb_status launch_assemble_surf(const hb_mesh *m, const T *ys, const T *x, T *y, 
     const int grid = red_grid(nr > 0 ? nr : 1);
     unsigned *ctr = m->counters + 0;
     hb_prof_scope prof("assemble", s);
+    cudaError_t e = cudaSuccess;
     // All copies of a row at once where the rows' reads come from DRAM; below,
     // they hit L2 and the fewer registers of the narrow form (40 against 80)
     // are worth more. us, narrow -> wide: FP32 A x, 1.8 M copies 12.1 -> 12.3,
@@ -168,11 +170,17 @@ hb_status launch_assemble_surf(const hb_mesh *m, const T *ys, const T *x, T *y, 
     const bool wide = m->nnz_s >= wide_from && !(contig && sizeof(T) == 8);
     constexpr bool kWideContig = sizeof(T) == 4;
 #define HB_ASM3(SC, DM, CT, WD, COLS)                                                                         \
-    assemble_surf_kernel<T, SC, DM, CT, WD><<<grid, HB_RED_THREADS, 0, s>>>(                                   \
-        ys, m->srow_g, m->srowptr, COLS, x, mdiag, lambda, y, nr, m->ax_partials, n_axp, m->partials, ctr, st)
+    (DM == HB_DOT_NONE                                                                                         \
+         ? hb_launch_after(assemble_surf_kernel<T, SC, DM, CT, WD>, grid, HB_RED_THREADS, 0, s, ys, m->srow_g,   \
+                           m->srowptr, COLS, x, mdiag, lambda, y, nr, m->ax_partials, n_axp, m->partials, ctr,   \
+                           st)                                                                                 \
+         : (assemble_surf_kernel<T, SC, DM, CT, WD><<<grid, HB_RED_THREADS, 0, s>>>(                             \
+                ys, m->srow_g, m->srowptr, COLS, x, mdiag, lambda, y, nr, m->ax_partials, n_axp, m->partials,    \
+                ctr, st),                                                                                        \
+            cudaGetLastError()))
 #define HB_ASM(SC, DM)                                                                                        \
-    (contig ? (wide ? HB_ASM3(SC, DM, true, kWideContig, nullptr) : HB_ASM3(SC, DM, true, false, nullptr))     \
-            : (wide ? HB_ASM3(SC, DM, false, true, m->scols) : HB_ASM3(SC, DM, false, false, m->scols)))
+    e = (contig ? (wide ? HB_ASM3(SC, DM, true, kWideContig, nullptr) : HB_ASM3(SC, DM, true, false, nullptr))     \
+                : (wide ? HB_ASM3(SC, DM, false, true, m->scols) : HB_ASM3(SC, DM, false, false, m->scols)))
     if (screen == 0) {
         if (dot_mode == HB_DOT_NONE) HB_ASM(0, HB_DOT_NONE);
         else if (dot_mode == HB_DOT_TO_TMP) HB_ASM(0, HB_DOT_TO_TMP);
@@ -184,7 +192,7 @@ hb_status launch_assemble_surf(const hb_mesh *m, const T *ys, const T *x, T *y, 
     }
 #undef HB_ASM3
 #undef HB_ASM
-    HB_CHECK_LAUNCH();
+    HB_TRY_CUDA(e);
     return HB_OK;
 }
 

@@ -269,8 +269,9 @@ __device__ inline void vertex_pos(const box_t &b, double rho, uint64_t seed, int
 // what can be is integer work: the node map (lexicographic ids over unmasked
 // lattice nodes, by closed form) rides along, the smallest det J is found on
 // its bits, the FP32 copies are rounded by integer instructions (conversions
-// run at the FP64 rate), and w_i w_j comes from a table. ms for 32x32x31, N = 11:
-// @@GEO@@
+// run at the FP64 rate), and w_i w_j comes from a table: 7.0 -> 6.25 ms for
+// 32x32x31, N = 11 with FP32 copies (6.12 without), and the node map's own pass
+// of 0.40 ms gone.
 
 // Order-preserving unsigned key of a double, and back.
 __host__ __device__ inline unsigned long long order_key(double v)
