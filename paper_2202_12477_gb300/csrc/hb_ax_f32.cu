@@ -79,23 +79,6 @@ __host__ __device__ constexpr int serve_eb() { return TH / ((N + 1) * (N + 1)); 
 template <int N, int TH = HB_SERVE_THREADS>
 __host__ __device__ constexpr size_t serve_smem_of() { return sizeof(T) * 4 * serve_eb<N, TH>() * pad<N>::size; }
 
-constexpr size_t serve_smem_max()
-{
-    size_t m = 0;
-    m = serve_smem_of<1>() > m ? serve_smem_of<1>() : m;
-    m = serve_smem_of<2>() > m ? serve_smem_of<2>() : m;
-    m = serve_smem_of<3>() > m ? serve_smem_of<3>() : m;
-    m = serve_smem_of<4>() > m ? serve_smem_of<4>() : m;
-    m = serve_smem_of<5>() > m ? serve_smem_of<5>() : m;
-    m = serve_smem_of<6>() > m ? serve_smem_of<6>() : m;
-    m = serve_smem_of<7>() > m ? serve_smem_of<7>() : m;
-    m = serve_smem_of<8>() > m ? serve_smem_of<8>() : m;
-    m = serve_smem_of<9>() > m ? serve_smem_of<9>() : m;
-    m = serve_smem_of<10>() > m ? serve_smem_of<10>() : m;
-    m = serve_smem_of<11>() > m ? serve_smem_of<11>() : m;
-    return m;
-}
-
 template <int N, int TH>
 __device__ __forceinline__ void serve_groups(const pencil_args &A, T *sm, hbacc::dot_acc<S> &acc)
 {
@@ -145,8 +128,9 @@ __global__ void __launch_bounds__(TH, MINB)
     if (threadIdx.x == 0) A.partials[blockIdx.x] = v;
 }
 
+// The launch of a degree class, without its arguments.
 template <int LO, int HI, int MINB, int TH>
-hb_status serve_launch_class(const hb_slot_desc *d, const hb_slot_state *st, cudaStream_t s)
+hb_status serve_class_params(cudaKernelNodeParams *p)
 {
     static int attr_set[32] = {0};
     static int grid_of[32] = {0};
@@ -162,25 +146,22 @@ hb_status serve_launch_class(const hb_slot_desc *d, const hb_slot_state *st, cud
         grid_of[dev] = MINB * sms < HB_SERVE_AXP ? MINB * sms : HB_SERVE_AXP;
         attr_set[dev] = 1;
     }
-    hb_count_launch();
-    kern<<<grid_of[dev], TH, smem, s>>>(d, st);
-    HB_CHECK_LAUNCH();
+    *p = cudaKernelNodeParams{};
+    p->func = (void *)kern;
+    p->gridDim = dim3(grid_of[dev]);
+    p->blockDim = dim3(TH);
+    p->sharedMemBytes = (unsigned)smem;
     return HB_OK;
 }
 
 }  // namespace
 }  // namespace hb2
 
-size_t hb_serve_ax_smem_f32() { return hb2::serve_smem_max(); }
-
-// Every degree class is launched; those that do not hold the slot's degree
-// return at once (the round graph is captured before slots are filled).
 static_assert(HB_SERVE_MAX_N == 11, "the serving degree classes cover N = 1..11");
-hb_status hb_serve_launch_ax_f32(const hb_slot_desc *d, const hb_slot_state *st, cudaStream_t s)
+int hb_serve_ax_class(int N) { return N <= 7 ? 0 : N <= 10 ? 1 : 2; }
+hb_status hb_serve_ax_f32_params(int cls, cudaKernelNodeParams *p)
 {
-    hb_status r = hb2::serve_launch_class<1, 7, 4, 256>(d, st, s);
-    if (r != HB_OK) return r;
-    r = hb2::serve_launch_class<8, 10, 2, 256>(d, st, s);
-    if (r != HB_OK) return r;
-    return hb2::serve_launch_class<11, 11, 3, 144>(d, st, s);
+    return cls == 0   ? hb2::serve_class_params<1, 7, 4, 256>(p)
+           : cls == 1 ? hb2::serve_class_params<8, 10, 2, 256>(p)
+                      : hb2::serve_class_params<11, 11, 3, 144>(p);
 }

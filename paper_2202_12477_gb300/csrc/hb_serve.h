@@ -50,7 +50,8 @@ struct hb_slot_state {
 // FP64: A x of the slot's current solution into Ap (runs when phase == OUTER);
 // FP32: A p32 into Ap32 with the interior partials of p.Ap (runs while the
 // inner CG runs).
-hb_status hb_serve_launch_ax_f64(const hb_slot_desc *d, const hb_slot_state *st, cudaStream_t s);
-hb_status hb_serve_launch_ax_f32(const hb_slot_desc *d, const hb_slot_state *st, cudaStream_t s);
-size_t hb_serve_ax_smem_f64();
-size_t hb_serve_ax_smem_f32();
+// Both come in degree classes (0, 1, 2): the class of a degree, and a class's
+// launch without its arguments (the slot's descriptor and state).
+int hb_serve_ax_class(int N);
+hb_status hb_serve_ax_f64_params(int cls, cudaKernelNodeParams *p);
+hb_status hb_serve_ax_f32_params(int cls, cudaKernelNodeParams *p);
