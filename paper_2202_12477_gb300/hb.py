@@ -171,13 +171,23 @@ def _check(status):
     return status
 
 
+_raw_stream = None  # torch's current raw stream of a device, once torch has set CUDA up
+
+
 def _stream_ptr(stream):
+    """The cudaStream_t of `stream` (None: torch's current stream) as an integer."""
+    global _raw_stream
     if stream is None:
+        if _raw_stream is not None:
+            # without the Stream object that torch.cuda.current_stream() makes (3 us of a small A x's 10)
+            return _raw_stream[0](_raw_stream[1]())
         import torch
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
-    if isinstance(stream, int):
-        return C.c_void_p(stream)
-    return C.c_void_p(stream.cuda_stream)
+        ptr = torch.cuda.current_stream().cuda_stream  # sets CUDA up
+        raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if raw is not None and dev is not None:
+            _raw_stream = (raw, dev)
+        return ptr
+    return stream if isinstance(stream, int) else stream.cuda_stream
 
 
 # ---------------------------------------------------------------- C names
@@ -199,7 +209,7 @@ def hb_mesh_info(h) -> hb_mesh_info_t:
 
 
 def hb_apply_A(h, prec, screen, lam, x_ptr, y_ptr, stream=None) -> None:
-    _check(lib().hb_apply_A(h, prec, screen, lam, C.c_void_p(x_ptr), C.c_void_p(y_ptr), _stream_ptr(stream)))
+    _check(lib().hb_apply_A(h, prec, screen, lam, x_ptr, y_ptr, _stream_ptr(stream)))
 
 
 def hb_dot(h, prec, a_ptr, b_ptr, out_dev_ptr=None, want_host=True, stream=None):
