@@ -499,8 +499,9 @@ double hb_u01(uint64_t seed, uint64_t stream, uint64_t idx);
  * Each of HB_F64, HB_F32 and HB_F64X keeps its own variant. HB_F64X takes
  * PENCIL | EVEN_ODD with or without ONE, and with CSR or GRID or neither (the
  * six shapes its double-float kernel is built in); other variants return
- * HB_ERR_ARG for it. The default is PENCIL | EVEN_ODD; hb_autotune measures
- * and picks per mesh and precision. */
+ * HB_ERR_ARG for it. The default is PENCIL | EVEN_ODD (A x alone takes Z^T as
+ * GRID does on meshes of about 30 million local nodes on: the same values);
+ * hb_autotune measures and picks per mesh and precision. */
 enum { HB_VARIANT_PENCIL = 1, HB_VARIANT_EVEN_ODD = 2, HB_VARIANT_EB2 = 4, HB_VARIANT_ONE = 8,
        HB_VARIANT_TMA = 16, HB_VARIANT_WS = 32, HB_VARIANT_CSR = 64, HB_VARIANT_GRID = 128,
        HB_VARIANT_TC = 256 };

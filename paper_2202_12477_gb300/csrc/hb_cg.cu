@@ -266,6 +266,21 @@ hb_status hb_launch_assemble_f32(const hb_mesh *m, const float *yL, const float 
     return launch_assemble<float>(m, yL, x, y, m->mdiag32, screen, lambda, st, dot_mode, s);
 }
 
+// Whether A x alone (no dot) of the default variant runs with the lattice
+// gather (HB_VAR_GRID) in place of the surface rows: the same values (both sum a
+// DOF's copies in element order), and faster where the mesh is far larger than
+// L2: the element kernel stores whole elements, coalesced, and finishes no
+// interior DOF. us, surface rows -> lattice: FP32 N = 3 455 -> 380 at 39 M local
+// nodes, N = 7 1155 -> 1012 at 122 M, N = 15 410 -> 362 at 38 M; FP64 N = 7 3937
+// -> 3837 at 41 M, N = 12 5809 -> 5330; double-float N = 7 4035 -> 3749 at 122 M.
+// At 4 M FP32 loses up to 14 %; N = 8 gains only from about 60 M on (432 -> 464
+// at 40 M); double-float from N = 11 on has its own element kernel (split).
+static bool lattice_for_Ax(const hb_mesh *m, hb_precision prec)
+{
+    if (prec == HB_F64X && m->N > 10) return false;
+    return m->n_local >= (m->N == 8 ? 60000000 : 30000000);
+}
+
 // A x: the element kernel, then Z^T. Pencil variants finish element-interior
 // DOFs in the element kernel and gather only surface DOFs; variant 0 writes
 // every local node and gathers all DOFs.
@@ -279,7 +294,8 @@ hb_status hb_apply_A_impl(const hb_mesh *m, hb_precision prec, int screen, doubl
     }
     if (prec == HB_F64X) {
         // double-float element kernel (pencil, even-odd) in its own variant's block shape
-        const int v64 = m->variant[2];
+        int v64 = m->variant[2];
+        if (dot_mode == HB_DOT_NONE && v64 == (HB_VAR_PENCIL | HB_VAR_EO) && lattice_for_Ax(m, prec)) v64 |= HB_VAR_GRID;
         const int ebm = hb_variant_eb_mode(v64);
         if ((ebm & 8) && !m->spos) { hb_set_error("surface positions missing for variant %d", v64); return HB_ERR_ARG; }
         const bool grid = (ebm & 16) != 0;
@@ -294,7 +310,8 @@ hb_status hb_apply_A_impl(const hb_mesh *m, hb_precision prec, int screen, doubl
         return launch_assemble_surf<double>(m, (const double *)m->yL, (const double *)x, (double *)y, m->mdiag,
                                             screen, lambda, partials ? nblk : 0, st, dot_mode, s, (ebm & 8) != 0);
     }
-    const int v = m->variant[hb_variant_slot(prec)];
+    int v = m->variant[hb_variant_slot(prec)];
+    if (dot_mode == HB_DOT_NONE && v == (HB_VAR_PENCIL | HB_VAR_EO) && lattice_for_Ax(m, prec)) v |= HB_VAR_GRID;
     if (v & HB_VAR_TC) {
         if (prec != HB_F64) { hb_set_error("the tensor-core element kernel is FP64 only"); return HB_ERR_ARG; }
         const bool csr = (v & HB_VAR_CSR) != 0;

@@ -69,3 +69,20 @@ def test_fused_cg_equals_launched(dims, N, screen):
     xz, rz = m.cg(b, x0.clone(), lam=0.3, screen=screen, max_it=0)
     assert rz.iters == 0 and torch.equal(xz, x0)
     m.close()
+
+
+@pytest.mark.parametrize("dims,N,prec", [((80, 81, 80), 3, hb.HB_F32), ((80, 81, 80), 3, hb.HB_F64),
+                                         ((40, 39, 41), 7, hb.HB_F64X), ((20, 20, 19), 15, hb.HB_F32)])
+def test_large_Ax_by_lattice_equals_surface_rows(dims, N, prec):
+    """From 30 million local nodes on A x alone takes Z^T by the lattice: the
+    same values as through the surface rows, which the dot modes (CG) keep."""
+    m = hb.Mesh(*dims, N, perturb=0.1, seed=2, faces=0x15, fp32=prec == hb.HB_F32)
+    assert m.n_local >= 30_000_000
+    dt = torch.float32 if prec == hb.HB_F32 else torch.float64
+    x = torch.from_numpy(inputs.random_vector(m.n_global, seed=6)).to(dt).cuda()
+    y = {}
+    for v in (3, 67):
+        hb.hb_set_kernel_variant(m.handle, prec, v)
+        y[v] = m.apply_A(x, lam=0.4, screen=1, prec=prec)
+    assert torch.equal(y[3], y[67])
+    m.close()
