@@ -182,12 +182,13 @@ extern "C" hb_status hb_tc_selftest(int mode, const float *A_host, const float *
 //     t >= 8, which weigh below 2^-58 of the largest term;
 //   - a digit enters the MMA as the FP16 number 256 + u_j (384 + u_0), whose
 //     bit pattern is 0x5C00 | (u_j << 2): no conversion instruction. The
-//     offsets contribute a constant per accumulator column, removed inside the
-//     same MMA by an eighth K block: 128 in the A operand times the constant's
-//     negative / 128 (split into FP16-exact parts) in the B operand;
-//   - the exact integers S_t are read back (FP32 -> int32 by adding 1.5 2^23),
-//     combined in two int64 halves and turned into doubles with the exponent
-//     of the element's grid (exact), summed with one FP64 add.
+//     offsets contribute a constant per accumulator column, replaced inside the
+//     same MMA by 1.5 2^23 with an eighth K block: 128 in the A operand times
+//     (1.5 2^23 - constant) / 128 (split into FP16-exact parts) in the B operand;
+//   - so a column's bits are 0x4B400000 + S_t: the exact integers are combined in
+//     two int64 halves and turned into doubles by integer instructions; the
+//     gradients stay in units of the element's grid (the scale rejoins at the
+//     end, in the exponent).
 // n = N + 1 is a power of two, so the lines of whole elements fill M-tiles of
 // 128 rows. Per M-tile and direction: one MMA chain of n / 2 K = 16 steps, A =
 // the lines' digits (128 x 8 n, K-major, K ordered (line position m, digit j)
@@ -206,8 +207,10 @@ namespace tcax {
 // block that N = 15's operands leave room for. Measured at 1.28e8 local nodes,
 // ms per launch: N = 3 4.29 with three blocks, 4.13 with four; N = 7 4.52 with
 // three blocks of 78 registers and its own t operand, 4.42 with four; N = 15
-// 6.43 with 512 threads, 6.16 with 1024. (The FP64 pencil kernel: 8.68, 11.8
-// and 17.4.)
+// 6.43 with 512 threads, 6.16 with 1024. With the accumulators biased, the
+// gradients left unscaled and one 64-bit value per sum (fewer integer
+// instructions, the busiest pipe beside FP64) 3.94, 4.25 and 5.85. (The FP64
+// pencil kernel: 8.68, 11.8 and 17.4.)
 template <int N_>
 struct shape {
     static constexpr int N = N_, n = N + 1, n2 = n * n, n3 = n2 * n;
@@ -276,10 +279,8 @@ struct tc_args {
     const int32_t *spos;  // SP kernels: CSR position of every surface copy (-1 masked)
 };
 
-__device__ __forceinline__ unsigned exp_bits(double v)
-{
-    return (unsigned)(__double_as_longlong(v) >> 52) & 0x7FFu;
-}
+// |v|'s high word: the largest of several carries the largest exponent (>> 20)
+__device__ __forceinline__ unsigned abs_hi(double v) { return (unsigned)__double2hiint(v) & 0x7FFFFFFFu; }
 
 // v on the grid of unit 2^(emax - 1075): round(|v| / unit) with the sign of v
 // (|result| < 2^53; zero and subnormal v give 0). Integer instructions only:
@@ -288,42 +289,41 @@ __device__ __forceinline__ long long to_fixed(double v, unsigned emax)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     const unsigned e = (unsigned)(b >> 52) & 0x7FFu;
-    // 2m with the implicit bit (m the 53-bit significand), 0 for zero and subnormals
-    const unsigned long long m2 = e ? ((b << 1) & 0x1FFFFFFFFFFFFEull) | (1ull << 53) : 0ull;
-    const unsigned sh = min(emax - e, 62u);
+    // 2m with the implicit bit (m the 53-bit significand), shifted out whole
+    // for zero and subnormals
+    const unsigned long long m2 = ((b << 1) & 0x1FFFFFFFFFFFFEull) | (1ull << 53);
+    const unsigned sh = e ? min(emax - e, 62u) : 62u;
     // round(m / 2^sh), halves up: (floor(2m / 2^sh) + 1) / 2
     const long long X = (long long)(((m2 >> sh) + 1ull) >> 1);
     return (b >> 63) ? -X : X;
 }
 
-// T 2^off as a double, rounded to nearest (ties away from zero) from the
-// integer T (any int64): normalise |T| so its top bit is bit 63, keep 53 bits,
-// round on the 11 below, and let a carry out of the mantissa step into the
-// exponent. Results below the normal range flush to zero, above it give
-// infinity.
+// The integer T as a double, rounded to nearest (ties away from zero):
+// normalise |T| so its top bit is bit 63, keep 53 bits, round on the 11 below,
+// and let a carry out of the mantissa step into the exponent. With OFF, T
+// 2^off: results below the normal range flush to zero, above it give infinity.
+template <bool OFF>
 __device__ __forceinline__ double i64_to_double(long long T, int off)
 {
-    if (T == 0) return 0.0;
     const unsigned long long sgn = (unsigned long long)T & 0x8000000000000000ull;
     unsigned long long M = T < 0 ? 0ull - (unsigned long long)T : (unsigned long long)T;
     const int lz = __clzll((long long)M);
     M <<= lz;
     const unsigned long long mant = (M >> 11) + ((M >> 10) & 1ull);  // 2^52 .. 2^53
-    const int ex = 1023 + 63 - lz + off;
-    if (ex <= 0) return __longlong_as_double((long long)sgn);
-    if (ex >= 2047) return __longlong_as_double((long long)(sgn | 0x7FF0000000000000ull));
-    return __longlong_as_double((long long)(sgn | (((unsigned long long)(ex - 1) << 52) + mant)));
+    const int ex = 1023 + 63 - lz + (OFF ? off : 0);
+    unsigned long long r = sgn | (((unsigned long long)(ex - 1) << 52) + mant);
+    if (OFF && ex >= 2047) r = sgn | 0x7FF0000000000000ull;
+    if (T == 0 || (OFF && ex <= 0)) r = sgn;
+    return __longlong_as_double((long long)r);
 }
 
-// 2^off (2^32 hi + lo) as a double: exactly as one int64 while that fits
-// (|hi| < 2^30), else from its value / 2^10 rounded down (the dropped bits
-// are below 2^-53 of a value of at least 2^63).
-__device__ __forceinline__ double halves_to_double(long long hi, long long lo, int off)
+// floor((2^32 hi + lo) / 2^10) for |hi| < 2^41: what an int64 holds of the sum.
+// (Its unit is a sixteenth of the error that rounding the values to the
+// element's grid leaves in it.)
+__device__ __forceinline__ long long halves(long long hi, long long lo)
 {
-    const bool small = (unsigned long long)(hi + (1ll << 30)) < (1ull << 31);
-    const int sh = small ? 0 : 10;
-    const long long T = (long long)((unsigned long long)hi << (32 - sh)) + (lo >> sh);
-    return i64_to_double(T, off + sh);
+    hi += lo >> 32;
+    return (long long)(((unsigned long long)hi << 22) | ((unsigned)lo >> 10));
 }
 
 // The A-operand row piece of one node: the FP16 bit patterns of the seven
@@ -391,26 +391,17 @@ __device__ __forceinline__ void mma_done(uint64_t *bar, unsigned &phase, int war
 // The exact diagonal sums of output o of a 16-column chunk (diagonals 0..7)
 // as the halves hi = sum_{t<4} S_t 256^(3-t), lo = sum_{t>=4} S_t 256^(7-t):
 // the output is 2^72 hi + 2^40 lo in units of the element's grid times 2^-s.
-// Each S_t is an integer below 2^22 in magnitude, read exactly from its float
-// f as bits(f + 1.5 2^23) - 0x4B400000.
+// A column holds S_t + 1.5 2^23 (the bias comes with the offset correction), so
+// S_t, an integer below 2^22 in magnitude, is its bits - 0x4B400000.
 __device__ __forceinline__ void combine(const uint32_t (&v)[16], int o, long long &hi, long long &lo)
 {
-    // two accumulators per packed FP32 add (add.rn.f32x2): the same
-    // round-to-nearest sums as one add each, half the instructions
-    unsigned B[8];
-#pragma unroll
-    for (int t = 0; t < 8; t += 2) {
-        unsigned long long pa, pr;
-        asm("mov.b64 %0, {%1, %2};" : "=l"(pa) : "r"(v[o * 8 + t]), "r"(v[o * 8 + t + 1]));
-        asm("add.rn.f32x2 %0, %1, %2;" : "=l"(pr) : "l"(pa), "l"(0x4B4000004B400000ull));
-        asm("mov.b64 {%0, %1}, %2;" : "=r"(B[t]), "=r"(B[t + 1]) : "l"(pr));
-    }
+    const uint32_t *B = v + o * 8;
     // S_a 256 + S_b fits an int32: form it modulo 2^32 from the raw bits
     constexpr unsigned kBias = 0x4B400000u * 257u;
-    const int m0 = (int)((unsigned)B[0] * 256u + (unsigned)B[1] - kBias);
-    const int m1 = (int)((unsigned)B[2] * 256u + (unsigned)B[3] - kBias);
-    const int m2 = (int)((unsigned)B[4] * 256u + (unsigned)B[5] - kBias);
-    const int m3 = (int)((unsigned)B[6] * 256u + (unsigned)B[7] - kBias);
+    const int m0 = (int)(B[0] * 256u + B[1] - kBias);
+    const int m1 = (int)(B[2] * 256u + B[3] - kBias);
+    const int m2 = (int)(B[4] * 256u + B[5] - kBias);
+    const int m3 = (int)(B[6] * 256u + B[7] - kBias);
     hi = (long long)m0 * 65536 + m1;
     lo = (long long)m2 * 65536 + m3;
 }
@@ -436,7 +427,7 @@ __device__ __forceinline__ void read_out(unsigned taddr, F &&f)
         }
 }
 
-// Largest biased exponent over the thread's element. n = 4: its 16 lanes.
+// Largest v over the thread's element. n = 4: its 16 lanes.
 // n = 8: warps 0, 1, 4, 5 hold element 0, warps 2, 3, 6, 7 element 1; n = 16:
 // the block's 32 warps. Every thread calls it; it synchronises the block.
 template <class C>
@@ -464,8 +455,9 @@ __device__ __forceinline__ unsigned element_max(unsigned v, unsigned *wexp, int 
 // (gradients to the exchange buffers, or the exact sums of D^T), start the t
 // chain into r's columns, read s out meanwhile, then t. The six metric factors
 // are prefetched into L2 at the tile's start and loaded at the metric step,
-// not held in registers. What bounds it (N = 7, ncu): the FP64 pipe 55 %, the
-// integer pipe 52 %, issue 55 % of the time; DRAM a quarter of the copy rate.
+// not held in registers. What bounds it (N = 7, ncu, before the integer work was
+// cut by a seventh): the FP64 pipe 55 %, the integer pipe 52 %, issue 55 % of the
+// time; DRAM a quarter of the copy rate.
 template <class C, bool SP>
 __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_args A)
 {
@@ -547,8 +539,8 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
         }
         unsigned em = 0;
 #pragma unroll
-        for (int q = 0; q < KH; q++) em = max(em, exp_bits(u[q]));
-        const unsigned eu = element_max<C>(em, wexp, el);
+        for (int q = 0; q < KH; q++) em = max(em, abs_hi(u[q]));
+        const unsigned eu = element_max<C>(em, wexp, el) >> 20;
         long long X[KH];
 #pragma unroll
         for (int q = 0; q < KH; q++) X[q] = eu == 0x7FFu ? 0 : to_fixed(u[q], eu);
@@ -565,10 +557,11 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
             hbtc::mma_commit(bar);
         }
         mma_done(bar, phase, warp, A.err, gave_up);
-        const int goff = (int)eu - 1075 - dshift + 40;
+        // gradients in units of 2^goff: their scale meets only the exponents
+        const int goff = (int)eu - 1075 - dshift + 40 + 10;
         const bool ubad = eu == 0x7FFu;
         auto value = [&](long long hi, long long lo) {
-            return ubad ? __longlong_as_double(0x7FF8000000000000ll) : halves_to_double(hi, lo, goff);
+            return ubad ? __longlong_as_double(0x7FF8000000000000ll) : i64_to_double<false>(halves(hi, lo), 0);
         };
         if constexpr (C::RESTAGE) stage<C, 2>(sm, el, ti, tj, k0, X);
         // ---- gradient along r into its exchange buffer; its columns are free
@@ -602,12 +595,12 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
                 vr[q] = fma(G[2], ut, fma(G[1], us, G[0] * ur));
                 vs[q] = fma(G[4], ut, fma(G[3], us, G[1] * ur));
                 vt[q] = fma(G[5], ut, fma(G[4], us, G[2] * ur));
-                evm = max(evm, max(exp_bits(vr[q]), max(exp_bits(vs[q]), exp_bits(vt[q]))));
+                evm = max(evm, max(abs_hi(vr[q]), max(abs_hi(vs[q]), abs_hi(vt[q]))));
             }
         }
         // (element_max meets the block: every exchange read is done before
         // the operands are staged over the exchange buffers)
-        const unsigned ev = element_max<C>(evm, wexp, el);
+        const unsigned ev = element_max<C>(evm, wexp, el) >> 20;
 #pragma unroll
         for (int q = 0; q < KH; q++) X[q] = ev == 0x7FFu ? 0 : to_fixed(vr[q], ev);
         stage<C, 0>(sm, el, ti, tj, k0, X);
@@ -650,7 +643,7 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
         });
         mma_done(bar, phase, warp, A.err, gave_up);
         {
-            const int yoff = (int)ev - 1075 - dshift + 40;
+            const int yoff = (int)ev - 1075 - dshift + 40 + 10 + goff;
             const bool vbad = ev == 0x7FFu;
             double *ys = A.ysurf + e * NS;
             const bool ring = ti == 0 || ti == N || tj == 0 || tj == N;
@@ -659,7 +652,7 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
                 const int k = k0 + q, xi = C::xq(el, ti, tj, k);
                 hi += Yhi[xi];
                 lo += Ylo[xi];
-                const double yc = vbad ? __longlong_as_double(0x7FF8000000000000ll) : halves_to_double(hi, lo, yoff);
+                const double yc = vbad ? __longlong_as_double(0x7FF8000000000000ll) : i64_to_double<true>(halves(hi, lo), yoff);
                 if (!active) return;
                 if (SP && (k == 0 || k == N || ring)) {
                     const int sidx = k == 0 ? a : (k == N ? n2 + a : 2 * n2 + (k - 1) * 4 * N + r);
@@ -806,9 +799,9 @@ static void derivative_dd(int N, const double *xi, dd (&D)[16][16])
 // be most of the kernel's error) is split into eight digits: D_int = D 2^s,
 // with |D_int| < 2^55 and eight binary places (the eighth digit meets only the
 // leading digit of the values, on the last diagonal). Largest sum of magnitudes
-// an accumulator can meet (digits, offsets and the correction): 2^19.3, 2^21.0
-// and 2^22.0 for N = 3, 7, 15, below the 2^24 FP32 holds exactly; the sums S_t
-// stay below 2^20.7.
+// an accumulator can meet (digits, offsets and the correction), without the bias:
+// 2^19.3, 2^21.0 and 2^22.0 for N = 3, 7, 15; with the bias, 1.5 2^23, below the
+// 2^24 that FP32 holds exactly. The sums S_t stay below 2^20.7.
 hb_status hb_tc_upload()
 {
     using namespace tcax;
@@ -862,10 +855,11 @@ hb_status hb_tc_upload()
                         }
                         beta += (j == 0 ? 384 : 256) * rs;
                     }
-                    // slot j = 7 of each K chunk: 128 (A side) times parts summing to -beta / 128
-                    long long c = -beta / 128;
+                    // slot j = 7 of each K chunk: 128 (A side) times parts summing to
+                    // (1.5 2^23 - beta) / 128
+                    long long c = (3 * (1 << 22) - beta) / 128;
                     for (int m = 0; m < n && c != 0; m++) {
-                        const long long p = fp16_part(c);
+                        const long long p = c > 49152 ? 49152 : fp16_part(c);
                         put(i, t, 7, m, p);
                         c -= p;
                     }
