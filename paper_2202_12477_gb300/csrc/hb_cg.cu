@@ -274,11 +274,15 @@ hb_status hb_launch_assemble_f32(const hb_mesh *m, const float *yL, const float 
 // nodes, N = 7 1155 -> 1012 at 122 M, N = 15 410 -> 362 at 38 M; FP64 N = 7 3937
 // -> 3837 at 41 M, N = 12 5809 -> 5330; double-float N = 7 4035 -> 3749 at 122 M.
 // At 4 M FP32 loses up to 14 %; N = 8 gains only from about 60 M on (432 -> 464
-// at 40 M); double-float from N = 11 on has its own element kernel (split).
+// at 40 M); double-float from N = 11 on has its own element kernel (split). The
+// gather takes a warp per lattice row, so boxes with few or short rows keep the
+// surface rows.
 static bool lattice_for_Ax(const hb_mesh *m, hb_precision prec)
 {
     if (prec == HB_F64X && m->N > 10) return false;
-    return m->n_local >= (m->N == 8 ? 60000000 : 30000000);
+    if (m->n_local < (m->N == 8 ? 60000000 : 30000000)) return false;
+    const lattice_t L = mesh_lattice(m);
+    return L.NXu >= 128 && (int64_t)L.NYu * L.NZu >= 40000;
 }
 
 // A x: the element kernel, then Z^T. Pencil variants finish element-interior

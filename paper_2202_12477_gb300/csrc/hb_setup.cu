@@ -411,6 +411,7 @@ __device__ __forceinline__ int surf_index(int i, int j, int k, int N)
 // copies of a row ascend by element, as do the columns; the mass is summed in
 // that order. 0.62 ms for 32x32x31, N = 11, where counting by atomics, scans,
 // filling and sorting the rows took 3.1 ms and five waits of the host.
+constexpr int kRowChunk = 1024;
 __global__ void __launch_bounds__(256)
     k_rows(lattice3 L, const double *__restrict__ geo, int32_t *__restrict__ rowptr, int32_t *__restrict__ cols,
            double *__restrict__ mdiag, float *__restrict__ mdiag32, int32_t *__restrict__ srow_g,
@@ -421,7 +422,10 @@ __global__ void __launch_bounds__(256)
     const int64_t SX = L.x.inner(), SY = L.y.inner();
     const int lane = threadIdx.x & 31;
     const int64_t nrows = (int64_t)L.y.nu * L.z.nu, nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < nrows; row += nwarps) {
+    const int nch = (L.x.nu + kRowChunk - 1) / kRowChunk;  // (long rows go to several warps)
+    for (int64_t unit = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; unit < nrows * nch; unit += nwarps) {
+        const int64_t row = unit / nch;
+        const int I0 = (int)(unit - row * nch) * kRowChunk, I1 = min(I0 + kRowChunk, L.x.nu);
         const int Ku = (int)(row / L.y.nu), Ju = (int)(row - (int64_t)Ku * L.y.nu);
         const int J = Ju + L.y.x0, K = Ku + L.z.x0;
         const int my = L.y.mult(J), mz = L.z.mult(K);
@@ -431,7 +435,7 @@ __global__ void __launch_bounds__(256)
         const int64_t i0 = SX * (L.z.inner_before(K) * SY + (K % N != 0 ? L.y.inner_before(J) : 0));
         // the first element along y and z, and the local index in it
         const int ey0 = J == 0 ? 0 : (J - 1) / N, ez0 = K == 0 ? 0 : (K - 1) / N, j0 = J - N * ey0, k0 = K - N * ez0;
-        for (int Iu = lane; Iu < L.x.nu; Iu += 32) {
+        for (int Iu = I0 + lane; Iu < I1; Iu += 32) {
             const int I = Iu + L.x.x0, mx = L.x.mult(I), ex0 = I == 0 ? 0 : (I - 1) / N, li = I - N * ex0;
             const int64_t g = row * L.x.nu + Iu, at = c0 + (int64_t)my * mz * L.x.copies_before(I);
             const int64_t before = i0 + (in_yz ? L.x.inner_before(I) : 0);
@@ -657,7 +661,7 @@ extern "C" hb_status hb_mesh_create(const hb_mesh_desc *d, void *stream, hb_mesh
     k_geometry<<<gblocks, gthreads, gsmem, s>>>(b, L, d->perturb, d->seed, E, m->l2g, m->geo, m->geo32, tmp_det);
     HB_TRY_MESH(cudaGetLastError());
     if (ng > 0) {
-        const int64_t warps = (int64_t)L.y.nu * L.z.nu;
+        const int64_t warps = (int64_t)L.y.nu * L.z.nu * ((L.x.nu + kRowChunk - 1) / kRowChunk);
         hb_count_launch();
         k_rows<<<grid_for(warps * 32, 256), 256, 0, s>>>(L, m->geo, m->rowptr, m->cols, m->mdiag, m->mdiag32, m->srow_g,
                                                          m->srowptr, m->scols);

@@ -29,7 +29,8 @@ def _host(ptr, n, kind):
 
 
 @pytest.mark.parametrize("dims,N", [((1, 1, 1), 1), ((1, 1, 1), 2), ((2, 1, 3), 1), ((3, 2, 2), 3), ((1, 4, 2), 5),
-                                    ((2, 2, 2), 8), ((5, 1, 1), 15), ((7, 9, 11), 2)])
+                                    ((2, 2, 2), 8), ((5, 1, 1), 15), ((7, 9, 11), 2),
+                                    ((700, 1, 2), 2)])
 @pytest.mark.parametrize("faces", [0x3F, 0x00, 0x15, 0x2A, 0x07])
 @pytest.mark.parametrize("perturb", [0.0, 0.2])
 def test_rows_and_copies(dims, N, faces, perturb):
