@@ -697,7 +697,7 @@ inline int cluster_blocks(int64_t E)
 // Double-float: the same rule (N = 7, 64 elements 18.4 -> 12.5), and from N =
 // 11 on at every size: its 256 threads a block whatever n^2 is, without the
 // node ids, leave registers and shared memory for more warps than the base
-// shape (us on 24^3 elements, base -> split: N = 11 1535 -> 1186, 12 2555 ->
+// shape (us on 24^3 elements, base -> split: N = 11 1535 -> 1110, 12 2555 ->
 // 1515, 13 2853 -> 2252, 14 3269 -> 2975; N = 15 6986 -> 4861 with one block
 // per element, one an SM for its shared memory, 3660 with two).
 template <int N>
@@ -803,16 +803,25 @@ __device__ __forceinline__ bool pencil_split(const pencil_args &A, int64_t e, in
     }
     cluster_arrive();  // (waited for before the first store to a peer)
     __syncthreads();
-    // lines: 2 ns n along r and s in the own slabs, then n^2 along t
-    const int nl = ns * n;
+    // lines: 2 ns n along r and s in the own slabs, then n^2 along t. A block
+    // that owns every slab (C = 1) takes whole t-lines like the others, so no
+    // warp holds two kinds of line.
+    const int nl = ns * n, whole = C == 1 ? 3 * nl : 2 * nl;
+    auto line_of = [&](int w, int &at, int &own, int &full, int &step) {
+        const int d = w / nl, wl = w - d * nl, q = wl / n, b = wl - q * n;
+        at = d == 0 ? b * rs : d == 1 ? b : q * rs + b;
+        own = d == 2 ? 0 : q * ss;         // in B1, B2, B3
+        full = d == 2 ? 0 : slab(q) * ss;  // in U
+        step = d == 0 ? 1 : d == 1 ? rs : ss;
+        return d == 0 ? B1 : d == 1 ? B2 : B3;
+    };
     for (int w = tid; w < 2 * nl + n2; w += nt) {
         T in[n];
-        if (w < 2 * nl) {
-            const bool s = w >= nl;
-            const int wl = s ? w - nl : w, q = wl / n, b = wl - q * n;
-            const int at = s ? b : b * rs, step = s ? rs : 1;
-            const T *src = U + slab(q) * ss + at;
-            T *dst = (s ? B2 : B1) + q * ss + at;
+        if (w < whole) {
+            int at, own, full, step;
+            T *dst = line_of(w, at, own, full, step);
+            const T *src = U + full + at;
+            dst += own + at;
 #pragma unroll
             for (int m = 0; m < n; m++) in[m] = src[m * step];
             line_st<N, false, true>(in, [&](int m, T v) { dst[m * step] = v; });
@@ -854,10 +863,10 @@ __device__ __forceinline__ bool pencil_split(const pencil_args &A, int64_t e, in
     cluster_arrive();
     __syncthreads();
     // D^T in place along the lines (each is read whole before it is written)
-    for (int w = tid; w < 2 * nl; w += nt) {
-        const bool s = w >= nl;
-        const int wl = s ? w - nl : w, q = wl / n, b = wl - q * n, step = s ? rs : 1;
-        T *dst = (s ? B2 : B1) + q * ss + (s ? b : b * rs);
+    for (int w = tid; w < whole; w += nt) {
+        int at, own, full, step;
+        T *dst = line_of(w, at, own, full, step);
+        dst += own + at;
         T in[n];
 #pragma unroll
         for (int m = 0; m < n; m++) in[m] = dst[m * step];
@@ -865,7 +874,7 @@ __device__ __forceinline__ bool pencil_split(const pencil_args &A, int64_t e, in
     }
     cluster_wait();  // the peers' v_t is here
     // the threads past the r- and s-lines first: the t-lines go to them
-    for (int w = (tid + nt - 2 * nl % nt) % nt; w < n2; w += nt) {
+    for (int w = C == 1 ? n2 : (tid + nt - 2 * nl % nt) % nt; w < n2; w += nt) {
         const int at = w / n * rs + w % n;
         T in[n];
 #pragma unroll

@@ -114,12 +114,13 @@ __device__ bool grid_wait_sum(const fused_args &F, double v, unsigned seq, doubl
     return true;
 }
 
-// Block size for degree N: the tasks of pencil_split, at least 256 threads
-// for the vector phases.
+// Block size for degree N: the tasks of pencil_split, at least 256 threads for
+// the vector phases; from N = 12 on 384, at some spills (125 elements, N = 15,
+// one block each: 128 us per iteration with 256, 124 with 384).
 template <int N>
 constexpr int fused_threads()
 {
-    return hb2::split<N>::MAXT < 256 ? 256 : hb2::split<N>::MAXT;
+    return N >= 12 ? 384 : hb2::split<N>::MAXT < 256 ? 256 : hb2::split<N>::MAXT;
 }
 // Shared memory: pencil_split's buffers and the element's node ids.
 template <int N>
