@@ -247,9 +247,11 @@ hb_status hb_cg_solve(const hb_mesh *mesh, const hb_cg_opts *opts, const double 
 
 /* How hb_cg_solve runs HB_F64 without a preconditioner: mode 0 (default) runs
  * every iteration inside one cooperative kernel (the phases of an iteration
- * separated by grid-wide barriers instead of launches, an element on one to
- * four blocks) when the mesh has at
- * most 300 elements and one block per element fits on the GPU at once;
+ * separated by grid-wide barriers instead of launches, one block per element
+ * with its three line directions contracted at once) when the mesh has at
+ * most 300 elements, one block per element fits on the GPU at once, and the
+ * elements are not few and large (N >= 11 on at most 76, N = 10 on at most 38:
+ * there the launched kernels give an element several blocks);
  * mode 1 never does; mode 2 does whenever they fit. The fused run computes the same
  * Algorithm 1 with its own fixed-order reductions (results agree with the
  * launched kernels to rounding, not bitwise). */

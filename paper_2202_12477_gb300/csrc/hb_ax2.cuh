@@ -763,14 +763,10 @@ __device__ __forceinline__ void line_part(T (&in)[N + 1], int c, int C, F &&stor
 
 // Element e by the C blocks of this cluster, this one being block c; sm holds
 // split<N>::smem(C) bytes. load(q, g) gives node q's value of u from its DOF
-// id g >= 0, id(q) the id itself. stop (null: never) points to one flag per
-// block of the cluster in shared memory, which the callers set in every peer
-// before the call: if one is set, all blocks of the cluster return false
-// after their first cluster barrier, nothing stored in a peer since. Every
-// thread of every block must call it.
+// id g >= 0, id(q) the id itself. Every thread of every block must call it.
 template <int N, class FI, class FL>
-__device__ __forceinline__ bool pencil_split(const pencil_args &A, int64_t e, int c, int C, T *sm,
-                                             hbacc::dot_acc<S> &acc, FI &&id, FL &&load, const int *stop = nullptr)
+__device__ __forceinline__ void pencil_split(const pencil_args &A, int64_t e, int c, int C, T *sm,
+                                             hbacc::dot_acc<S> &acc, FI &&id, FL &&load)
 {
     using L = split<N>;
     using P = pad<N>;
@@ -834,11 +830,6 @@ __device__ __forceinline__ bool pencil_split(const pencil_args &A, int64_t e, in
     }
     __syncthreads();
     cluster_wait();
-    if (stop) {
-        int any = 0;
-        for (int r = 0; r < C; r++) any |= stop[r];
-        if (any) return false;
-    }
     auto metric = [&](int w, const S (&g)[6]) {
         const int q = w / n2, a = w - q * n2, at = a / n * rs + a % n, own = q * ss + at, full = slab(q) * ss + at;
         const T grr = to_c(g[0]), grs = to_c(g[1]), grt = to_c(g[2]), gss = to_c(g[3]), gst = to_c(g[4]),
@@ -904,7 +895,6 @@ __device__ __forceinline__ bool pencil_split(const pencil_args &A, int64_t e, in
         }
     }
     __syncthreads();  // the buffers are reused by the next element
-    return true;
 }
 
 // Grid: E * C blocks in clusters of C.

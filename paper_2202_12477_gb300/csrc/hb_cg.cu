@@ -721,16 +721,23 @@ static hb_status cg_true_residual(const hb_mesh *m, const hb_cg_opts *o, const d
 }
 
 // Fused CG: FP64 without a preconditioner, when every element of the mesh
-// fits in one cooperative launch (one per block; mode 0: and the mesh is
-// small enough that latency sets the time, at most 300 elements, where it
-// measured faster than the launched kernels; mode 2: whenever it fits).
+// fits in one cooperative launch, one per block. Mode 2: whenever it fits.
+// Mode 0: where it measured faster than the launched kernels, which is up to
+// 300 elements (latency sets the time), less the few large elements that the
+// launched element kernel spreads over clusters of four or two blocks
+// (cluster_blocks; a block here has its element alone). us per iteration,
+// launched / fused: N = 7, 64 elements 27.0 / 21.2, 294: 37.2 / 32.1; N = 9,
+// 64: 35.1 / 32.3; N = 10, 27: 35.0 / 39.2, 64: 40.9 / 39.2; N = 11, 64: 44.9 /
+// 48.8, 125: 58.6 / 49.2; N = 15, 27: 49.0 / 110.6, 64: 72.6 / 111.6, 125: 110.4
+// / 112.6.
 static bool use_fused_cg(const hb_mesh *m, const hb_cg_opts *o)
 {
     if (o->prec != HB_F64 || o->precond || m->fused_mode == 1) return false;
-    const int64_t groups = m->E;  // one element per block
     const int cap = hb_cg_fused_capacity(m->N);
-    if (cap <= 0 || groups > cap) return false;
-    return m->fused_mode == 2 || groups <= 300;
+    if (cap <= 0 || m->E > cap) return false;
+    if (m->fused_mode == 2) return true;
+    if ((m->N >= 11 && 2 * m->E <= 152) || (m->N == 10 && 4 * m->E <= 152)) return false;
+    return m->E <= 300;
 }
 
 extern "C" hb_status hb_cg_solve(const hb_mesh *mc, const hb_cg_opts *o, const double *b, double *x,

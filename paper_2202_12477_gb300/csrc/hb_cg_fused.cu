@@ -3,9 +3,9 @@
 // itself needs a few microseconds of FP64 work, and launching the four
 // kernels of an iteration costs more than that; here the phases of an
 // iteration are separated by three grid-wide waits instead of launches:
-//   x += alpha p, p = r + beta p (each DOF by its owner), and A p by element
-//     (pencil_split, over a cluster of C blocks: each node forms its p from r
-//     and the old p itself, with the owner's arithmetic, so no wait lies
+//   x += alpha p, p = r + beta p (each DOF by its owner), and A p, one element
+//     per block, its three line directions at once (each node forms its p from
+//     r and the old p itself, with the owner's arithmetic, so no wait lies
 //     between; p has two buffers)
 //   | Z^T on surface DOFs, p.Ap
 //   | r -= alpha Ap, r.r
@@ -16,9 +16,8 @@
 // second records bit 1 in the mesh's error word and every block then leaves
 // the iteration loop (the host reports HB_ERR_TIMEOUT).
 // Measured, us per iteration (with four waits, the barrier's arrival returning
-// a value, one block per element -> this form): 4x4x4 elements at N = 7 27.6
-// -> 17.8, at N = 3 16.7 -> 14.5. At N = 7 a wait takes 2.2 us, the element
-// phase 6.9 (2.9 of it FP64 operations), the vector phases 1.1 each.
+// a value -> this form): 4x4x4 elements at N = 7 26.1 -> 21.2, at N = 3 18.5 ->
+// 14.5, 125 elements at N = 15 117.8 -> 112.6. A wait takes about 2.2 us.
 #include "hb_internal.h"
 #define HB_AX2_T double
 #include "hb_ax2.cuh"
@@ -114,46 +113,119 @@ __device__ bool grid_wait_sum(const fused_args &F, double v, unsigned seq, doubl
     return true;
 }
 
-// Block size for degree N: the tasks of pencil_split, at least 256 threads for
-// the vector phases; from N = 12 on 384, at some spills (125 elements, N = 15,
-// one block each: 128 us per iteration with 256, 124 with 384).
+// The element's A p: one element per block on 3 (N+1)^2 threads. Group d = 0, 1,
+// 2 of n^2 threads contracts the r-, s- or t-lines (the three directions at
+// once), and the gather, metric and epilogue phases split each t-line's k range
+// over the groups (k = d, d + 3, ...). For a small mesh, where the element's own
+// latency sets the time, this keeps all four FP64 units of an SM busy instead
+// of the two that n^2 threads reach. Same arithmetic as hb2::pencil_group per
+// node. load(g) gives the value of u at DOF g. Every thread of the block must
+// call it. (The launch is a plain cooperative one: an element spread over a
+// cluster of blocks, which store into each other's shared memory, took 17.8 us
+// per iteration at N = 7 on 64 elements, but a profiler's run of that kernel,
+// cooperative and in clusters at once, ended in an illegal access on the GPU
+// for which no cause was found, so no block here reaches outside itself.)
+template <int N, class FL>
+__device__ __forceinline__ void element_lines(const hb2::pencil_args &A, int64_t e, double *sm,
+                                              hbacc::dot_acc<double> &acc, FL &&load)
+{
+    using P = hb2::pad<N>;
+    constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
+    const int tid = threadIdx.x, d = tid / n2, a = tid - d * n2, p0 = a % n, p1 = a / n;  // d: 0 r, 1 s, 2 t; 3+ idle
+    const bool active = d < 3;
+    const int32_t *__restrict__ lg = A.l2g + e * n3 + a;
+    const double *__restrict__ ge = A.geo + e * 7 * n3 + a;
+    double *U = sm, *B1 = U + P::size, *B2 = B1 + P::size, *B3 = B2 + P::size;
+    double *Bd = d == 0 ? B1 : (d == 1 ? B2 : B3);
+    if (active)
+        for (int k = d; k < n; k += 3) {
+            const int g = __ldg(lg + k * n2);
+            U[P::at(p0, p1, k)] = g >= 0 ? load(g) : 0.0;
+        }
+    __syncthreads();
+    // node m of the line this thread owns: r (m, p0, p1), s (p0, m, p1), t (p0, p1, m)
+    auto at_line = [&](int m) { return d == 0 ? P::at(m, p0, p1) : (d == 1 ? P::at(p0, m, p1) : P::at(p0, p1, m)); };
+    double in[n];
+    if (active) {
+#pragma unroll
+        for (int m = 0; m < n; m++) in[m] = U[at_line(m)];
+        hb2::line_st<N, false, true>(in, [&](int m, double v) { Bd[at_line(m)] = v; });
+    }
+    __syncthreads();
+    if (active)
+        for (int k = d; k < n; k += 3) {
+            const double *g = ge + k * 7 * n2;
+            const double grr = __ldcs(g), grs = __ldcs(g + n2), grt = __ldcs(g + 2 * n2);
+            const double gss = __ldcs(g + 3 * n2), gst = __ldcs(g + 4 * n2), gtt = __ldcs(g + 5 * n2);
+            const int q = P::at(p0, p1, k);
+            const double ur = B1[q], us = B2[q], ut = B3[q];
+            B1[q] = fma(grt, ut, fma(grs, us, grr * ur));
+            B2[q] = fma(gst, ut, fma(gss, us, grs * ur));
+            B3[q] = fma(gtt, ut, fma(gst, us, grt * ur));
+        }
+    __syncthreads();
+    if (active) {
+#pragma unroll
+        for (int m = 0; m < n; m++) in[m] = Bd[at_line(m)];
+        hb2::line_st<N, true, true>(in, [&](int m, double v) { Bd[at_line(m)] = v; });
+    }
+    __syncthreads();
+    if (active) {
+        double *ys = A.ysurf + e * hb2::surf_count<N>();
+        const bool ring = p0 == 0 || p0 == N || p1 == 0 || p1 == N;
+        const int r = ring ? hb2::ring_index<N>(p0, p1) : 0;
+        for (int k = d; k < n; k += 3) {
+            const int q = P::at(p0, p1, k);
+            const double yc = B1[q] + B2[q] + B3[q];
+            if (k == 0) {
+                ys[a] = yc;
+            } else if (k == N) {
+                ys[n2 + a] = yc;
+            } else if (ring) {
+                ys[2 * n2 + (k - 1) * 4 * N + r] = yc;
+            } else {
+                const double xv = U[q], jw = A.screen ? __ldg(ge + (k * 7 + 6) * n2) : 1.0;
+                double y = yc;
+                y += A.lambda * (jw * xv);
+                A.y[__ldg(lg + k * n2)] = y;
+                acc.add(xv, y);
+            }
+        }
+    }
+    __syncthreads();  // the buffers are reused by the next element
+}
+
+// Block size for degree N: the three thread groups of element_lines, at least
+// 256 threads for the vector phases. Shared memory: its four buffers.
 template <int N>
 constexpr int fused_threads()
 {
-    return N >= 12 ? 384 : hb2::split<N>::MAXT < 256 ? 256 : hb2::split<N>::MAXT;
+    constexpr int t = 3 * (N + 1) * (N + 1);
+    return t < 256 ? 256 : (t + 31) / 32 * 32;
 }
-// Shared memory: pencil_split's buffers and the element's node ids.
 template <int N>
-size_t fused_smem(int C)
-{
-    return hb2::split<N>::smem(C) + sizeof(int32_t) * hb2::split<N>::n3;
-}
+constexpr size_t fused_smem() { return sizeof(double) * 4 * (size_t)hb2::pad<N>::size; }
 
-// Grid: E * C blocks in clusters of C (hb2::cluster_blocks), all resident at
-// once.
+// Grid: at most as many blocks as are resident at once, an element (or several)
+// each.
 template <int N>
-__global__ void __launch_bounds__(fused_threads<N>()) cg_fused_kernel(const fused_args F, int C)
+__global__ void __launch_bounds__(fused_threads<N>()) cg_fused_kernel(const fused_args F)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ int s_stop[8];  // one per block of the cluster (pencil_split)
     double *sm = reinterpret_cast<double *>(smem_raw);
-    int32_t *ids = reinterpret_cast<int32_t *>(smem_raw + hb2::split<N>::smem(C));
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gthreads = (int64_t)gridDim.x * blockDim.x;
-    const int64_t e = blockIdx.x / C;
-    const int c = blockIdx.x % C;
 
     double rr = F.st->rr;
     const double tol2 = F.st->tol2;
     const int max_it = F.st->max_it;
-    int stop = F.st->run == 0;
+    bool stop = F.st->run == 0;
     int it = 0;
     unsigned seq = 0;
     int status = HB_OK;
     double alpha = 0.0, beta = 0.0, pAp = 0.0;
     double *pold = F.p2, *p = F.p;  // p_{j-1} and p_j
 
-    for (int q = threadIdx.x; q < hb2::split<N>::n3; q += blockDim.x) ids[q] = F.l2g[e * hb2::split<N>::n3 + q];
     // this thread's first surface row (its only one on the smallest meshes)
     int row_g = -1, row_a = 0, row_z = 0, row_c[4] = {0, 0, 0, 0};
     if (gtid < F.nsr) {
@@ -164,35 +236,27 @@ __global__ void __launch_bounds__(fused_threads<N>()) cg_fused_kernel(const fuse
         for (int q = 0; q < 4; q++)
             if (row_a + q < row_z) row_c[q] = F.scols[row_a + q];
     }
-    // the peers' shared memory is there from here on, and stays until all
-    // blocks of the cluster have agreed to leave (the return of pencil_split)
-    hb2::cluster_arrive();
-    hb2::cluster_wait();
-    __syncthreads();
-
     hb2::pencil_args A{nullptr, F.l2g, F.geo, F.ysurf, F.Ap, F.E, nullptr, F.lambda, F.screen, nullptr};
     for (;;) {
         // x += alpha p_{j-1}, p_j = r + beta p_{j-1} (j > 0) at this thread's DOFs
         // (data written by other blocks in this launch is read through L2)
-        if (it > 0 && status == HB_OK)
+        if (it > 0)
             for (int64_t i = gtid; i < F.n_global; i += gthreads) {
                 const double po = __ldcg(pold + i);
                 F.x[i] += alpha * po;
                 if (!stop) p[i] = fma(beta, po, F.r[i]);
             }
-        if (threadIdx.x < C) *hb2::peer(&s_stop[c], threadIdx.x) = stop;
+        if (stop) break;
         // A p: interior DOFs finished, surface values to ysurf
         hbacc::dot_acc<double> acc;
         const bool first = it == 0;
-        if (!hb2::pencil_split<N>(
-                A, e, c, C, sm, acc, [&](int q) { return ids[q]; },
-                [&](int, int g) { return first ? __ldcg(p + g) : fma(beta, __ldcg(pold + g), __ldcg(F.r + g)); },
-                s_stop))
-            break;
+        for (int64_t e = blockIdx.x; e < F.E; e += gridDim.x)
+            element_lines<N>(A, e, sm, acc, [&](int g) {
+                return first ? __ldcg(p + g) : fma(beta, __ldcg(pold + g), __ldcg(F.r + g));
+            });
         if (grid_barrier(F.bar, gridDim.x, ++seq, F.err)) {
             status = HB_ERR_TIMEOUT;
-            stop = 1;
-            continue;
+            break;
         }
         // Z^T on the surface DOFs
         auto row = [&](int g, int a, int z, const int (&c4)[4]) {
@@ -217,13 +281,11 @@ __global__ void __launch_bounds__(fused_threads<N>()) cg_fused_kernel(const fuse
         double v = hbacc::block_sum(acc.value());
         if (!grid_wait_sum(F, v, ++seq, pAp)) {
             status = HB_ERR_TIMEOUT;
-            stop = 1;
-            continue;
+            break;
         }
         if (!(pAp > 0.0) || !isfinite(pAp)) {
-            status = HB_ERR_BREAKDOWN;  // every block takes the same branch
-            stop = 1;
-            continue;
+            status = HB_ERR_BREAKDOWN;
+            break;  // every block takes the same branch
         }
         alpha = rr / pAp;
         // r -= alpha Ap and r.r
@@ -237,8 +299,7 @@ __global__ void __launch_bounds__(fused_threads<N>()) cg_fused_kernel(const fuse
         double rr_new;
         if (!grid_wait_sum(F, v, ++seq, rr_new)) {
             status = HB_ERR_TIMEOUT;
-            stop = 1;
-            continue;
+            break;
         }
         beta = rr_new / rr;
         rr = rr_new;
@@ -262,59 +323,37 @@ __global__ void __launch_bounds__(fused_threads<N>()) cg_fused_kernel(const fuse
     }
 }
 
-// Blocks of a cluster of C that are resident at once (0: cannot launch).
+// Blocks that are resident at once.
 template <int N>
-hb_status fused_resident(int C, cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&at)[2], int64_t *blocks)
+hb_status fused_resident(int64_t *blocks)
 {
     auto kern = cg_fused_kernel<N>;
     static int attr_set[32] = {0};
-    int dev = 0;
+    int dev = 0, per_sm = 0, sms = 0;
     HB_TRY_CUDA(cudaGetDevice(&dev));
-    if (dev >= 0 && dev < 32 && !attr_set[dev]) {
-        HB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused_smem<N>(1)));
-        attr_set[dev] = 1;
+    if (dev < 0 || dev >= 32 || !attr_set[dev]) {
+        HB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused_smem<N>()));
+        if (dev >= 0 && dev < 32) attr_set[dev] = 1;
     }
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = C;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    at[1].id = cudaLaunchAttributeCooperative;
-    at[1].val.cooperative = 1;
-    cfg.gridDim = dim3((unsigned)C);
-    cfg.blockDim = dim3(fused_threads<N>());
-    cfg.dynamicSmemBytes = fused_smem<N>(C);
-    cfg.attrs = at;
-    cfg.numAttrs = 2;
-    if (C == 1) {
-        int per_sm = 0, sms = 0;
-        HB_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, fused_threads<N>(), fused_smem<N>(1)));
-        HB_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        *blocks = (int64_t)per_sm * sms;
-    } else {
-        int clusters = 0;
-        HB_TRY_CUDA(cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg));
-        *blocks = (int64_t)clusters * C;
-    }
+    HB_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, fused_threads<N>(), fused_smem<N>()));
+    HB_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    *blocks = (int64_t)per_sm * sms;
     return HB_OK;
 }
 
 template <int N>
-hb_status launch_fused(fused_args &F, cudaStream_t s, bool probe_only, int64_t *capacity)
+hb_status launch_fused(fused_args &F, cudaStream_t s)
 {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[2];
     int64_t blocks = 0;
-    if (probe_only) return fused_resident<N>(1, cfg, at, capacity);
-    int C = hb2::cluster_blocks<N>(F.E);
-    for (;; C /= 2) {
-        hb_status r = fused_resident<N>(C, cfg, at, &blocks);
-        if (r != HB_OK) return r;
-        if (F.E * C <= blocks && F.E * C <= HB_RED_BLOCKS) break;
-        if (C == 1) { hb_set_error("fused CG: %lld elements do not fit", (long long)F.E); return HB_ERR_ARG; }
-    }
-    cfg.gridDim = dim3((unsigned)(F.E * C));
-    cfg.stream = s;
+    hb_status st = fused_resident<N>(&blocks);
+    if (st != HB_OK) return st;
+    if (blocks > HB_RED_BLOCKS) blocks = HB_RED_BLOCKS;
+    if (blocks > F.E) blocks = F.E;
+    if (blocks < 1) { hb_set_error("fused CG: no block fits"); return HB_ERR_ARG; }
+    void *args[] = {(void *)&F};
     hb_prof_scope prof("cg_fused", s);
-    HB_TRY_CUDA(cudaLaunchKernelEx(&cfg, cg_fused_kernel<N>, (const fused_args)F, C));
+    HB_TRY_CUDA(cudaLaunchCooperativeKernel((const void *)cg_fused_kernel<N>, dim3((unsigned)blocks),
+                                            dim3(fused_threads<N>()), args, fused_smem<N>(), s));
     return HB_OK;
 }
 
@@ -342,18 +381,17 @@ int hb_cg_fused_capacity(int N)
     int dev = 0, coop = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return 0;
-    fused_args F{};
     int64_t cap = 0;
     hb_status st;
     switch (N) {
 #define HB_CASE(NN) \
-    case NN: st = launch_fused<NN>(F, nullptr, true, &cap); break;
+    case NN: st = fused_resident<NN>(&cap); break;
         HB_CASE(1) HB_CASE(2) HB_CASE(3) HB_CASE(4) HB_CASE(5) HB_CASE(6) HB_CASE(7) HB_CASE(8)
         HB_CASE(9) HB_CASE(10) HB_CASE(11) HB_CASE(12) HB_CASE(13) HB_CASE(14) HB_CASE(15)
 #undef HB_CASE
     default: return 0;
     }
-    return st == HB_OK ? (int)(cap < HB_RED_BLOCKS ? cap : HB_RED_BLOCKS) : 0;
+    return st == HB_OK ? (int)cap : 0;
 }
 
 // max_it iterations (or until the state's tolerance) of Algorithm 1 on
@@ -387,7 +425,7 @@ hb_status hb_cg_fused_run(const hb_mesh *m, int screen, double lambda, double *x
     HB_TRY_CUDA(cudaMemsetAsync(F.bar, 0, sizeof(unsigned), s));
     switch (m->N) {
 #define HB_CASE(NN) \
-    case NN: return launch_fused<NN>(F, s, false, nullptr);
+    case NN: return launch_fused<NN>(F, s);
         HB_CASE(1) HB_CASE(2) HB_CASE(3) HB_CASE(4) HB_CASE(5) HB_CASE(6) HB_CASE(7) HB_CASE(8)
         HB_CASE(9) HB_CASE(10) HB_CASE(11) HB_CASE(12) HB_CASE(13) HB_CASE(14) HB_CASE(15)
 #undef HB_CASE
