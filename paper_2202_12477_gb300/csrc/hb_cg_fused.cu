@@ -203,13 +203,21 @@ constexpr int fused_threads()
     constexpr int t = 3 * (N + 1) * (N + 1);
     return t < 256 ? 256 : (t + 31) / 32 * 32;
 }
+// Blocks per SM asked of the compiler. What fits on the GPU at once is what this
+// solver takes (hb_cg_fused_capacity), and left to itself the compiler uses up
+// to 135 registers, which fits two blocks at N = 7 and one at N = 10 (304 and
+// 152 elements, for 608 and 304 with these bounds). The times are the same
+// (N = 7, 64 elements 20.9 us an iteration without, 21.2 with them; N = 10, 294
+// elements 70.8 by the launched kernels, 68.8 here).
+template <int N>
+constexpr int fused_blocks() { return N <= 3 || N == 6 ? 5 : N <= 8 ? 4 : N <= 10 ? 2 : 1; }
 template <int N>
 constexpr size_t fused_smem() { return sizeof(double) * 4 * (size_t)hb2::pad<N>::size; }
 
 // Grid: at most as many blocks as are resident at once, an element (or several)
 // each.
 template <int N>
-__global__ void __launch_bounds__(fused_threads<N>()) cg_fused_kernel(const fused_args F)
+__global__ void __launch_bounds__(fused_threads<N>(), fused_blocks<N>()) cg_fused_kernel(const fused_args F)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     double *sm = reinterpret_cast<double *>(smem_raw);
