@@ -570,6 +570,15 @@ hb_status hb_probe(int kind, hb_precision prec, size_t bytes, int reps, double *
  * nothing. Takes about a second; synchronises `stream`. */
 hb_status hb_selftest_wait(int which, hb_status *status, void *stream);
 
+/* Self-test of the check that kernels running in thread-block clusters make
+ * before they store into another block's shared memory. Runs one such kernel
+ * told that its cluster has two blocks, which the launch makes (clustered = 1)
+ * or does not (0). No block then touches another: the kernel writes NaN for its
+ * results and sets the error word that the solvers turn into HB_ERR_CUDA.
+ * *status receives what a solver would return: HB_OK for 1, HB_ERR_CUDA for 0.
+ * Synchronises `stream`. */
+hb_status hb_selftest_cluster(int clustered, hb_status *status, void *stream);
+
 /* Self-check of the tensor-core operand layouts the tensor-core element
  * kernel uses (no paper counterpart: a check of the hardware interface).
  * Computes D = A B^T through tcgen05.mma kind::f16 (M = 128, N = 48, K = 48 in

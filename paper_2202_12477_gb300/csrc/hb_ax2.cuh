@@ -290,7 +290,7 @@ struct pencil_args {
     // l2g entries g <= -2 read halo[-2 - g] (values of DOFs another partition
     // owns, filled by a halo exchange); -1 is a masked node
     const S *halo;
-    unsigned *err;  // WS kernels: bit 0 set when a bounded wait gave up
+    unsigned *err;  // WS kernels: bit 0 set when a bounded wait gave up; split kernel: bit 2 if not in its clusters
     // SP kernels: CSR position of every surface copy (e * surface nodes +
     // surface index; -1 masked); ysurf is then indexed by CSR position
     const int32_t *spos;
@@ -714,6 +714,18 @@ inline int split_blocks(int64_t E)
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ int cluster_size()
+{
+    int c;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(c));
+    return c;
+}
+__device__ __forceinline__ int cluster_rank()
+{
+    int c;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(c));
+    return c;
+}
 // Address of this block's shared-memory object in block `rank` of the cluster.
 template <typename V>
 __device__ __forceinline__ V *peer(V *p, int rank)
@@ -897,7 +909,26 @@ __device__ __forceinline__ void pencil_split(const pencil_args &A, int64_t e, in
     __syncthreads();  // the buffers are reused by the next element
 }
 
-// Grid: E * C blocks in clusters of C.
+// NaN for every value the split kernel owes for element e.
+template <int N>
+__device__ __noinline__ void split_refuse(const pencil_args &A, int64_t e)
+{
+    constexpr int n = N + 1, n3 = n * n * n, NS = surf_count<N>();
+    for (int q = threadIdx.x; q < NS; q += blockDim.x) A.ysurf[e * NS + q] = S(NAN);
+    for (int q = threadIdx.x; q < n3; q += blockDim.x) {
+        const int i = q % n, j = q / n % n, k = q / (n * n);
+        if (i > 0 && i < N && j > 0 && j < N && k > 0 && k < N) A.y[A.l2g[e * n3 + q]] = S(NAN);
+    }
+    if (threadIdx.x == 0) {
+        if (A.partials) A.partials[blockIdx.x] = NAN;
+        if (A.err) atomicOr(A.err, 4u);
+    }
+}
+
+// Grid: E * C blocks in clusters of C. A block stores into its peers' shared
+// memory, so it takes its rank and the cluster's size from the hardware, and
+// if those are not the shape asked for (a launch whose cluster attribute was
+// lost on its way), no block touches a peer: bit 2 of the error word and NaN.
 template <int N>
 __global__ void __launch_bounds__(split<N>::MAXT) ax_split_kernel(const pencil_args A, int C)
 {
@@ -906,9 +937,14 @@ __global__ void __launch_bounds__(split<N>::MAXT) ax_split_kernel(const pencil_a
     extern __shared__ __align__(128) unsigned char smem_raw[];
     hbacc::dot_acc<S> acc;
     const int64_t e = blockIdx.x / C;
+    const int c = cluster_rank();
+    if (cluster_size() != C || c != (int)(blockIdx.x % C)) {
+        split_refuse<N>(A, e);
+        return;
+    }
     const int32_t *__restrict__ lg = A.l2g + e * split<N>::n3;
     const S *__restrict__ x = A.x;
-    pencil_split<N>(A, e, blockIdx.x % C, C, reinterpret_cast<T *>(smem_raw), acc,
+    pencil_split<N>(A, e, c, C, reinterpret_cast<T *>(smem_raw), acc,
                     [&](int q) { return __ldg(lg + q); }, [&](int, int g) { return __ldg(x + g); });
     if (A.partials) {
         const double v = hbacc::block_sum(acc.value());

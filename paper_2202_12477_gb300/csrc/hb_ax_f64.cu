@@ -28,8 +28,8 @@ hb_status hb_launch_ax2_f64(const hb_mesh *m, const double *x, double *ysurf, do
                             int64_t *nblocks)
 {
     if (!m->geo) { hb_set_error("mesh has no double geometric factors"); return HB_ERR_ARG; }
-    hb2::pencil_args A{x, m->l2g, m->geo, ysurf, y, m->E, run, (double)lambda, screen, partials, nullptr, nullptr,
-                       (eb_mult & 8) ? m->spos : nullptr};
+    hb2::pencil_args A{x, m->l2g, m->geo, ysurf, y, m->E, run, (double)lambda, screen, partials, nullptr,
+                       m->counters + 7, (eb_mult & 8) ? m->spos : nullptr};
     switch (m->N) {
 #define HB_CASE(NN) \
     case NN: return eo ? hb2::launch<NN, true>(A, eb_mult, s, nblocks) : hb2::launch<NN, false>(A, eb_mult, s, nblocks);
@@ -80,6 +80,58 @@ hb_status hb_launch_ax2_f64_scat(const hb_mesh *m, const double *xL, double *ysu
 #undef HB_CASE
     default: hb_set_error("unsupported N=%d", m->N); return HB_ERR_ARG;
     }
+}
+
+// One element of N = 3 on zeros through the split kernel told that it runs in a
+// cluster of two, which the launch makes or (clustered = 0) does not.
+extern "C" hb_status hb_selftest_cluster(int clustered, hb_status *status, void *stream)
+{
+    hb_clear_error();
+    if (!status) { hb_set_error("null argument"); return HB_ERR_ARG; }
+    if (clustered != 0 && clustered != 1) { hb_set_error("clustered must be 0 or 1"); return HB_ERR_ARG; }
+    hb_status st = hb_ensure_device_tables();
+    if (st != HB_OK) return st;
+    cudaStream_t s = (cudaStream_t)stream;
+    constexpr int N = 3, n3 = 64, NS = hb2::surf_count<N>();
+    struct buf {
+        double geo[7 * n3], ysurf[NS], x[1], y[1], partials[2];
+        int32_t l2g[n3];
+        unsigned err;
+    } *d = nullptr, h{};
+    HB_TRY_CUDA(cudaMalloc((void **)&d, sizeof(buf)));
+    cudaError_t e = cudaMemsetAsync(d, 0, sizeof(buf), s);
+    if (e == cudaSuccess) {
+        const hb2::pencil_args A{d->x, d->l2g, d->geo, d->ysurf, d->y, 1, nullptr, 0.0, 0, d->partials, nullptr, &d->err};
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 2;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(2);
+        cfg.blockDim = dim3((unsigned)hb2::split<N>::threads(2));
+        cfg.dynamicSmemBytes = hb2::split<N>::smem(2);
+        cfg.stream = s;
+        cfg.attrs = at;
+        cfg.numAttrs = clustered;
+        hb_count_launch();
+        e = cudaLaunchKernelEx(&cfg, hb2::ax_split_kernel<N>, A, 2);
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d, sizeof(buf), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaFree(d);
+    if (e != cudaSuccess) {
+        hb_set_error("self-test: %s", cudaGetErrorString(e));
+        return HB_ERR_CUDA;
+    }
+    bool nan = std::isnan(h.y[0]) && std::isnan(h.partials[0]) && std::isnan(h.partials[1]);
+    bool zero = h.y[0] == 0.0 && h.partials[0] == 0.0 && h.partials[1] == 0.0;
+    for (double v : h.ysurf) {
+        nan = nan && std::isnan(v);
+        zero = zero && v == 0.0;
+    }
+    *status = hb_dev_err_status(h.err);
+    if (*status == HB_OK ? !zero : !nan) { hb_set_error("self-test: unexpected values"); return HB_ERR_CUDA; }
+    return HB_OK;
 }
 
 int hb_surf_count(int N) { return 2 * (N + 1) * (N + 1) + 4 * N * (N - 1); }

@@ -463,9 +463,22 @@ extern "C" hb_status hb_dot(const hb_mesh *m, hb_precision prec, const void *a, 
     return HB_OK;
 }
 
-// Error word the kernels set when a bounded wait gave up (bit 0: a
-// staged-pipeline wait, bit 1: a fused-CG grid barrier); read and cleared at
-// the solvers' sync points.
+// What an error word of the kernels means: a bounded wait gave up (bit 0: a
+// staged-pipeline or tensor-core wait, bit 1: a fused-CG grid barrier), or a
+// kernel was not run in the clusters it was launched with (bit 2). Sets the
+// message; HB_OK for 0.
+hb_status hb_dev_err_status(unsigned v)
+{
+    if (v == 0) return HB_OK;
+    if (v & 4u) {
+        hb_set_error("a kernel did not run in the thread-block clusters it was launched with");
+        return HB_ERR_CUDA;
+    }
+    hb_set_error("a kernel gave up waiting (%s)", (v & 2u) ? "fused CG grid barrier" : "staged data");
+    return HB_ERR_TIMEOUT;
+}
+
+// The mesh's error word, read and cleared at the solvers' sync points.
 static hb_status check_dev_err(hb_mesh *m, cudaStream_t s)
 {
     unsigned v = 0;
@@ -473,10 +486,8 @@ static hb_status check_dev_err(hb_mesh *m, cudaStream_t s)
     HB_TRY_CUDA(cudaStreamSynchronize(s));
     if (v) {
         HB_TRY_CUDA(cudaMemsetAsync(m->counters + 7, 0, sizeof(unsigned), s));
-        hb_set_error("a kernel gave up waiting (%s)", (v & 2u) ? "fused CG grid barrier" : "staged data");
-        return HB_ERR_TIMEOUT;
     }
-    return HB_OK;
+    return hb_dev_err_status(v);
 }
 
 // ---------------------------------------------------------------- autotuner

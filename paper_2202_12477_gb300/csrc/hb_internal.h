@@ -262,6 +262,8 @@ int hb_cg_fused_capacity(int N);
 hb_status hb_cg_fused_upload(const double *D_all);
 hb_status hb_cg_fused_run(const hb_mesh *m, int screen, double lambda, double *x, double *r, double *p, double *p2,
                           double *Ap, hb_cg_state *st, cudaStream_t s);
+// Status of an error word set by kernels (with its message); HB_OK for 0.
+hb_status hb_dev_err_status(unsigned v);
 // Self-tests of the bounded device waits (hb_selftest_wait): the staged
 // pipeline's mbarrier wait (sets bit 0 of *err) and the fused CG's grid
 // barrier (bar: a zeroed word; sets bit 1).

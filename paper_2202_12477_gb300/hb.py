@@ -137,6 +137,7 @@ _SIGS = [
                               C.POINTER(C.c_double), C.c_void_p]),
     ("hb_probe", C.c_int, [C.c_int, C.c_int, C.c_size_t, C.c_int, C.POINTER(C.c_double)]),
     ("hb_selftest_wait", C.c_int, [C.c_int, C.POINTER(C.c_int), C.c_void_p]),
+    ("hb_selftest_cluster", C.c_int, [C.c_int, C.POINTER(C.c_int), C.c_void_p]),
     ("hb_kernel_launches", C.c_ulonglong, []),
     ("hb_profile_enable", C.c_int, [C.c_int]),
     ("hb_profile_reset", C.c_int, []),
@@ -275,6 +276,14 @@ def hb_probe(kind, prec=HB_F64, nbytes=4 << 30, reps=5) -> float:
     r = C.c_double(0.0)
     _check(lib().hb_probe(kind, prec, nbytes, reps, C.byref(r)))
     return r.value
+
+
+def hb_selftest_cluster(clustered, stream=None) -> int:
+    """Runs a kernel told that it is in a cluster of two blocks, which its launch
+    makes or not; returns the status it reported (HB_OK, HB_ERR_CUDA)."""
+    st = C.c_int(-1)
+    _check(lib().hb_selftest_cluster(int(clustered), C.byref(st), _stream_ptr(stream)))
+    return st.value
 
 
 def hb_selftest_wait(which, stream=None) -> int:

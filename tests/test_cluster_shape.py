@@ -1,5 +1,5 @@
 """Static checks of the CUDA sources (no GPU): which kernels may reach into the
-shared memory of other blocks."""
+shared memory of other blocks, and that they look at their cluster first."""
 import os
 import re
 
@@ -23,3 +23,18 @@ def test_cooperative_kernels_launch_without_clusters():
         seen += 1
         assert not re.search(r"ClusterDimension|mapa|\bpeer\(|barrier\.cluster|cluster_(arrive|wait)|pencil_split", text), f
     assert seen
+
+
+def test_kernels_with_peers_check_their_cluster():
+    """Every kernel that calls pencil_split (stores to peers) compares the
+    cluster it runs in with the one it was launched for before that call."""
+    seen = 0
+    for f in sorted(os.listdir(CSRC)):
+        for k in re.split(r"__global__", _code(f))[1:]:
+            at = k.find("pencil_split<")
+            if at < 0:
+                continue
+            seen += 1
+            check = re.search(r"if \(cluster_size\(\) != C \|\| c != \(int\)\(blockIdx\.x % C\)\)", k[:at])
+            assert check and "return;" in k[check.end():at], f
+    assert seen == 1
