@@ -911,7 +911,7 @@ __device__ __forceinline__ void pencil_split(const pencil_args &A, int64_t e, in
 
 // NaN for every value the split kernel owes for element e.
 template <int N>
-__device__ __noinline__ void split_refuse(const pencil_args &A, int64_t e)
+__device__ __forceinline__ void split_refuse(const pencil_args &A, int64_t e)
 {
     constexpr int n = N + 1, n3 = n * n * n, NS = surf_count<N>();
     for (int q = threadIdx.x; q < NS; q += blockDim.x) A.ysurf[e * NS + q] = S(NAN);
