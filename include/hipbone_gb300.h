@@ -501,14 +501,20 @@ double hb_u01(uint64_t seed, uint64_t stream, uint64_t idx);
  * Each of HB_F64, HB_F32 and HB_F64X keeps its own variant. HB_F64X takes
  * PENCIL | EVEN_ODD with or without ONE, and with CSR or GRID or neither (the
  * six shapes its double-float kernel is built in); other variants return
- * HB_ERR_ARG for it. The default is PENCIL | EVEN_ODD (A x alone takes Z^T as
- * GRID does on meshes of about 30 million local nodes on: the same values);
- * hb_autotune measures and picks per mesh and precision. */
+ * HB_ERR_ARG for it. The default is PENCIL | EVEN_ODD; hb_autotune measures and
+ * picks per mesh and precision.
+ * A x alone (hb_apply_A, the solvers' residuals) has a variant of its own.
+ * hb_set_kernel_variant sets both; hb_set_apply_variant sets that one;
+ * hb_get_apply_variant tells which variant A x alone runs. On a mesh whose
+ * variant was neither set nor tuned it is PENCIL | EVEN_ODD, with GRID (the same
+ * values) from about 30 million local nodes on. */
 enum { HB_VARIANT_PENCIL = 1, HB_VARIANT_EVEN_ODD = 2, HB_VARIANT_EB2 = 4, HB_VARIANT_ONE = 8,
        HB_VARIANT_TMA = 16, HB_VARIANT_WS = 32, HB_VARIANT_CSR = 64, HB_VARIANT_GRID = 128,
        HB_VARIANT_TC = 256 };
 hb_status hb_set_kernel_variant(hb_mesh *mesh, hb_precision prec, int variant);
 hb_status hb_get_kernel_variant(const hb_mesh *mesh, hb_precision prec, int *variant);
+hb_status hb_set_apply_variant(hb_mesh *mesh, hb_precision prec, int variant);
+hb_status hb_get_apply_variant(const hb_mesh *mesh, hb_precision prec, int *variant);
 
 /* Autotuner (the paper makes its 3-D / 2-D kernel switch a configurable choice
  * made from measurements, Sec. 3.2; here every variant is timed on the mesh
@@ -519,7 +525,9 @@ hb_status hb_get_kernel_variant(const hb_mesh *mesh, hb_precision prec, int *var
  * PENCIL|EVEN_ODD|ONE|CSR, PENCIL|EVEN_ODD|GRID, PENCIL|EVEN_ODD|ONE|GRID, and TC,
  * TC|CSR for HB_F64 at N = 3, 7, 15; for HB_F64X the six it takes) on `stream`, keeps the
  * fastest for `prec` (HB_F64, HB_F32 or HB_F64X) on this mesh and returns it in
- * *best_variant. ms_per_variant (may be NULL) has 512 slots
+ * *best_variant. On meshes of about 30 million local nodes on, A x alone of that
+ * variant is timed with and without GRID, and the faster kept for A x alone
+ * (hb_get_apply_variant). ms_per_variant (may be NULL) has 512 slots
  * indexed by variant and receives the mean time of each. Allocates two scratch vectors for the
  * duration of the call; synchronises `stream`. */
 hb_status hb_autotune(hb_mesh *mesh, hb_precision prec, hb_screen screen, double lambda, int reps,

@@ -54,18 +54,21 @@ def store(cache: dict, path: str | None = None) -> None:
     os.replace(tmp, path)
 
 
-def lookup(cache: dict, dev: str, N: int, prec: int, exclude: int = 0):
+def lookup(cache: dict, dev: str, N: int, prec: int, exclude: int = 0, field: str = "variant"):
+    """The stored variant, or with field="apply" that of A x alone (None: no entry, or not a valid one)."""
     e = cache.get(dev, {}).get(entry_key(N, prec, exclude))
     valid = hb.VARIANTS_F64X if prec == hb.HB_F64X else (
         hb.VARIANTS + hb.VARIANTS_TC if prec == hb.HB_F64 and N in hb.TC_DEGREES else hb.VARIANTS)
-    if isinstance(e, dict) and e.get("variant") in valid and not (e["variant"] & exclude):
-        return e["variant"]
+    if isinstance(e, dict) and e.get(field) in valid and not (e[field] & exclude):
+        return e[field]
     return None
 
 
-def record(cache: dict, dev: str, N: int, prec: int, variant: int, timings: dict, exclude: int = 0) -> dict:
+def record(cache: dict, dev: str, N: int, prec: int, variant: int, timings: dict, exclude: int = 0,
+           apply: int | None = None) -> dict:
     cache.setdefault(dev, {})[entry_key(N, prec, exclude)] = {
-        "variant": int(variant), "ms": {str(k): float(v) for k, v in timings.items()}}
+        "variant": int(variant), "apply": int(variant if apply is None else apply),
+        "ms": {str(k): float(v) for k, v in timings.items()}}
     return cache
 
 
@@ -99,13 +102,17 @@ def tune_mesh(mesh, precs=(hb.HB_F64, hb.HB_F32), screen=hb.HB_SCREEN_IDENTITY, 
             v = None if force else lookup(cache, dev, mesh.N, prec, exclude)
             if v is None:
                 v, timings = hb.hb_autotune(mesh.handle, prec, screen, lam, reps)
-                if exclude and v & exclude:
+                if exclude:
+                    # also where the winner is allowed: A x alone may have been tuned to its lattice form
                     v = best_allowed(timings, exclude)
                     hb.hb_set_kernel_variant(mesh.handle, prec, v)
-                record(cache, dev, mesh.N, prec, v, timings, exclude)
+                record(cache, dev, mesh.N, prec, v, timings, exclude, hb.hb_get_apply_variant(mesh.handle, prec))
                 changed = True
             else:
                 hb.hb_set_kernel_variant(mesh.handle, prec, v)
+                ax = lookup(cache, dev, mesh.N, prec, exclude, "apply")
+                if ax is not None and ax != v:
+                    hb.hb_set_apply_variant(mesh.handle, prec, ax)
             chosen[prec] = v
         if changed:
             store(cache, path)

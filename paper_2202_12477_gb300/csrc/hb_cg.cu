@@ -266,8 +266,8 @@ hb_status hb_launch_assemble_f32(const hb_mesh *m, const float *yL, const float 
     return launch_assemble<float>(m, yL, x, y, m->mdiag32, screen, lambda, st, dot_mode, s);
 }
 
-// Whether A x alone (no dot) of the default variant runs with the lattice
-// gather (HB_VAR_GRID) in place of the surface rows: the same values (both sum a
+// Whether A x alone (no dot) gains by the lattice gather (HB_VAR_GRID) in place
+// of the surface rows: the same values (both sum a
 // DOF's copies in element order), and faster where the mesh is far larger than
 // L2: the element kernel stores whole elements, coalesced, and finishes no
 // interior DOF. us, surface rows -> lattice: FP32 N = 3 455 -> 380 at 39 M local
@@ -285,6 +285,15 @@ static bool lattice_for_Ax(const hb_mesh *m, hb_precision prec)
     return L.NXu >= 128 && (int64_t)L.NYu * L.NZu >= 40000;
 }
 
+// The variant that A x alone runs: what was set or tuned, and on a mesh whose
+// variant nobody chose the default's lattice form where that is the faster.
+static int apply_variant(const hb_mesh *m, hb_precision prec)
+{
+    const int slot = hb_variant_slot(prec);
+    if (m->variant_ax[slot] >= 0) return m->variant_ax[slot];
+    return m->variant[slot] | (lattice_for_Ax(m, prec) ? HB_VAR_GRID : 0);
+}
+
 // A x: the element kernel, then Z^T. Pencil variants finish element-interior
 // DOFs in the element kernel and gather only surface DOFs; variant 0 writes
 // every local node and gathers all DOFs.
@@ -298,8 +307,7 @@ hb_status hb_apply_A_impl(const hb_mesh *m, hb_precision prec, int screen, doubl
     }
     if (prec == HB_F64X) {
         // double-float element kernel (pencil, even-odd) in its own variant's block shape
-        int v64 = m->variant[2];
-        if (dot_mode == HB_DOT_NONE && v64 == (HB_VAR_PENCIL | HB_VAR_EO) && lattice_for_Ax(m, prec)) v64 |= HB_VAR_GRID;
+        const int v64 = dot_mode == HB_DOT_NONE ? apply_variant(m, prec) : m->variant[2];
         const int ebm = hb_variant_eb_mode(v64);
         if ((ebm & 8) && !m->spos) { hb_set_error("surface positions missing for variant %d", v64); return HB_ERR_ARG; }
         const bool grid = (ebm & 16) != 0;
@@ -314,8 +322,7 @@ hb_status hb_apply_A_impl(const hb_mesh *m, hb_precision prec, int screen, doubl
         return launch_assemble_surf<double>(m, (const double *)m->yL, (const double *)x, (double *)y, m->mdiag,
                                             screen, lambda, partials ? nblk : 0, st, dot_mode, s, (ebm & 8) != 0);
     }
-    int v = m->variant[hb_variant_slot(prec)];
-    if (dot_mode == HB_DOT_NONE && v == (HB_VAR_PENCIL | HB_VAR_EO) && lattice_for_Ax(m, prec)) v |= HB_VAR_GRID;
+    const int v = dot_mode == HB_DOT_NONE ? apply_variant(m, prec) : m->variant[hb_variant_slot(prec)];
     if (v & HB_VAR_TC) {
         if (prec != HB_F64) { hb_set_error("the tensor-core element kernel is FP64 only"); return HB_ERR_ARG; }
         const bool csr = (v & HB_VAR_CSR) != 0;
@@ -389,9 +396,10 @@ hb_status hb_launch_dot_f32(const hb_mesh *m, const float *a, const float *b, in
 
 static bool valid_screen(int s) { return s == HB_SCREEN_IDENTITY || s == HB_SCREEN_MASS; }
 
-extern "C" hb_status hb_set_kernel_variant(hb_mesh *m, hb_precision prec, int variant)
+// Refuses what prec and the mesh's degree do not have; builds what the variant
+// needs.
+static hb_status prepare_variant(hb_mesh *m, hb_precision prec, int variant)
 {
-    hb_clear_error();
     if (!m) { hb_set_error("null mesh"); return HB_ERR_ARG; }
     const int slot = hb_variant_slot(prec);
     if (slot < 0) { hb_set_error("variant precision must be HB_F64, HB_F32 or HB_F64X"); return HB_ERR_ARG; }
@@ -408,7 +416,32 @@ extern "C" hb_status hb_set_kernel_variant(hb_mesh *m, hb_precision prec, int va
         hb_status st = hb_mesh_ensure_spos(m, nullptr);
         if (st != HB_OK) return st;
     }
-    m->variant[slot] = variant;
+    return HB_OK;
+}
+
+extern "C" hb_status hb_set_kernel_variant(hb_mesh *m, hb_precision prec, int variant)
+{
+    hb_clear_error();
+    const hb_status st = prepare_variant(m, prec, variant);
+    if (st != HB_OK) return st;
+    m->variant[hb_variant_slot(prec)] = m->variant_ax[hb_variant_slot(prec)] = variant;
+    return HB_OK;
+}
+
+extern "C" hb_status hb_set_apply_variant(hb_mesh *m, hb_precision prec, int variant)
+{
+    hb_clear_error();
+    const hb_status st = prepare_variant(m, prec, variant);
+    if (st != HB_OK) return st;
+    m->variant_ax[hb_variant_slot(prec)] = variant;
+    return HB_OK;
+}
+
+extern "C" hb_status hb_get_apply_variant(const hb_mesh *m, hb_precision prec, int *variant)
+{
+    if (!m || !variant) { hb_set_error("null argument"); return HB_ERR_ARG; }
+    if (hb_variant_slot(prec) < 0) { hb_set_error("variant precision must be HB_F64, HB_F32 or HB_F64X"); return HB_ERR_ARG; }
+    *variant = apply_variant(m, prec);
     return HB_OK;
 }
 
@@ -536,34 +569,46 @@ extern "C" hb_status hb_autotune(hb_mesh *m, hb_precision prec, hb_screen screen
             return sp;
         }
     }
-    const int saved = m->variant[pi];
+    const int saved = m->variant[pi], saved_ax = m->variant_ax[pi];
     int best = saved;
     float best_ms = 1e30f;
     hb_status st = HB_OK;
     // each application also reduces x.y, as every CG iteration does (p.Ap):
     // variants differ in where that work runs (element kernel or gather)
     hb_cg_state *tmp = m->state + 1;
+    // one untimed application (first launch, attribute setup), then `reps` timed ones
+    auto time = [&](int c, int dot, float &ms) {
+        m->variant[pi] = m->variant_ax[pi] = c;
+        ms = 1e30f;
+        hb_cg_state *to = dot == HB_DOT_NONE ? nullptr : tmp;
+        st = hb_apply_A_impl(m, prec, screen, lambda, x, y, to, dot, s);
+        if (st == HB_OK) e = cudaEventRecord(m->ev0, s);
+        for (int r = 0; r < reps && st == HB_OK; r++) st = hb_apply_A_impl(m, prec, screen, lambda, x, y, to, dot, s);
+        if (st == HB_OK && e == cudaSuccess) e = cudaEventRecord(m->ev1, s);
+        if (st == HB_OK && e == cudaSuccess) e = cudaEventSynchronize(m->ev1);
+        if (st == HB_OK && e == cudaSuccess) e = cudaEventElapsedTime(&ms, m->ev0, m->ev1);
+        ms /= reps;
+        return st == HB_OK && e == cudaSuccess;
+    };
     for (int c : candidates) {
         if ((c & HB_VAR_TC) && (prec != HB_F64 || !hb_tc_degree(m->N))) continue;
         if (prec == HB_F64X && !hb_valid_variant_f64x(c)) continue;
-        m->variant[pi] = c;
-        // one untimed application (first launch, attribute setup), then `reps` timed ones
-        st = hb_apply_A_impl(m, prec, screen, lambda, x, y, tmp, HB_DOT_TO_TMP, s);
-        if (st != HB_OK) break;
-        if ((e = cudaEventRecord(m->ev0, s)) != cudaSuccess) break;
-        for (int r = 0; r < reps && st == HB_OK; r++)
-            st = hb_apply_A_impl(m, prec, screen, lambda, x, y, tmp, HB_DOT_TO_TMP, s);
-        if (st != HB_OK) break;
-        if ((e = cudaEventRecord(m->ev1, s)) != cudaSuccess) break;
-        if ((e = cudaEventSynchronize(m->ev1)) != cudaSuccess) break;
-        float ms = 0.f;
-        if ((e = cudaEventElapsedTime(&ms, m->ev0, m->ev1)) != cudaSuccess) break;
-        ms /= reps;
+        float ms;
+        if (!time(c, HB_DOT_TO_TMP, ms)) break;
         if (ms_per_variant) ms_per_variant[c] = ms;
         if (ms < best_ms) {
             best_ms = ms;
             best = c;
         }
+    }
+    // A x alone on a mesh of the lattice gather's size: the winner's lattice form
+    // (the same values) if that is the faster without the dot
+    int best_ax = best;
+    constexpr int kPair = HB_VAR_PENCIL | HB_VAR_EO;
+    if (st == HB_OK && e == cudaSuccess && (best & ~(HB_VAR_ONE | HB_VAR_CSR)) == kPair && lattice_for_Ax(m, prec)) {
+        const int grid = kPair | (best & HB_VAR_ONE) | HB_VAR_GRID;
+        float rows_ms, grid_ms;
+        if (time(best, HB_DOT_NONE, rows_ms) && time(grid, HB_DOT_NONE, grid_ms) && grid_ms < rows_ms) best_ax = grid;
     }
     cudaFree(x);
     cudaFree(y);
@@ -573,9 +618,13 @@ extern "C" hb_status hb_autotune(hb_mesh *m, hb_precision prec, hb_screen screen
     }
     if (st == HB_OK) st = check_dev_err(m, s);
     m->variant[pi] = st == HB_OK ? best : saved;
+    m->variant_ax[pi] = st == HB_OK ? best_ax : saved_ax;
     if (best_variant) *best_variant = m->variant[pi];
     // the surface positions were built for the timing; keep them only if used
-    if (m->spos && !((m->variant[0] | m->variant[1] | m->variant[2]) & HB_VAR_CSR)) {
+    bool csr = false;
+    for (int q = 0; q < 3; q++)
+        csr = csr || (m->variant[q] & HB_VAR_CSR) || (m->variant_ax[q] >= 0 && (m->variant_ax[q] & HB_VAR_CSR));
+    if (m->spos && !csr) {
         cudaStreamSynchronize(s);
         hb_mesh_drop_graphs(m);
         cudaFree(m->spos);

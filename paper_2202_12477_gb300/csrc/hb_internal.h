@@ -127,6 +127,7 @@ struct hb_mesh {
     size_t device_bytes;
     cudaEvent_t ev0, ev1;
     int variant[3];     // element-kernel variant per precision (HB_F64, HB_F32, HB_F64X)
+    int variant_ax[3];  // of A x alone (no dot): a variant, or -1 until one is set or tuned (a rule on the size)
     // Jacobi preconditioner: 1 / diag(A) for the (screen, lambda) it was built for
     double *inv_diag;
     float *inv_diag32;

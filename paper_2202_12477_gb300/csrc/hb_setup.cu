@@ -604,6 +604,7 @@ extern "C" hb_status hb_mesh_create(const hb_mesh_desc *d, void *stream, hb_mesh
     m->variant[0] = HB_VAR_PENCIL | HB_VAR_EO;
     m->variant[1] = HB_VAR_PENCIL | HB_VAR_EO;
     m->variant[2] = HB_VAR_PENCIL | HB_VAR_EO;
+    m->variant_ax[0] = m->variant_ax[1] = m->variant_ax[2] = -1;
     m->N = N;
     m->n = n;
     m->E = E;

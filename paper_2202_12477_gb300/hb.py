@@ -133,6 +133,8 @@ _SIGS = [
     ("hb_tc_selftest", C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.POINTER(C.c_int)]),
     ("hb_set_kernel_variant", C.c_int, [C.c_void_p, C.c_int, C.c_int]),
     ("hb_get_kernel_variant", C.c_int, [C.c_void_p, C.c_int, C.POINTER(C.c_int)]),
+    ("hb_set_apply_variant", C.c_int, [C.c_void_p, C.c_int, C.c_int]),
+    ("hb_get_apply_variant", C.c_int, [C.c_void_p, C.c_int, C.POINTER(C.c_int)]),
     ("hb_autotune", C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_double, C.c_int, C.POINTER(C.c_int),
                               C.POINTER(C.c_double), C.c_void_p]),
     ("hb_probe", C.c_int, [C.c_int, C.c_int, C.c_size_t, C.c_int, C.POINTER(C.c_double)]),
@@ -255,6 +257,17 @@ def hb_set_kernel_variant(h, prec, variant) -> None:
 def hb_get_kernel_variant(h, prec) -> int:
     v = C.c_int(-1)
     _check(lib().hb_get_kernel_variant(h, prec, C.byref(v)))
+    return v.value
+
+
+def hb_set_apply_variant(h, prec, variant) -> None:
+    """The variant of A x alone (hb_set_kernel_variant sets it too)."""
+    _check(lib().hb_set_apply_variant(h, prec, variant))
+
+
+def hb_get_apply_variant(h, prec) -> int:
+    v = C.c_int(-1)
+    _check(lib().hb_get_apply_variant(h, prec, C.byref(v)))
     return v.value
 
 
