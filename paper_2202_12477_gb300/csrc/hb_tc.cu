@@ -167,10 +167,9 @@ extern "C" hb_status hb_tc_selftest(int mode, const float *A_host, const float *
 //
 // Exact contractions from FP16 products (an Ozaki-style split into slices):
 //   - the element's values u are put on one fixed-point grid,
-//     X = round(u / 2^E) with 2^E the unit of the element's largest exponent
-//     (|X| < 2^53: the rounding is below the last bit of the largest value),
-//     and written as seven base-256 digits, X = sum_j u_j 256^(6-j), u_0
-//     signed (|u_0| <= 32), u_1..u_6 unsigned bytes;
+//     X = round(u / 2^E) with 2^E two bits below the last of the element's
+//     largest value (|X| < 2^55), and written as seven base-256 digits,
+//     X = sum_j u_j 256^(6-j), u_0 a signed byte, u_1..u_6 unsigned ones;
 //   - D is scaled to integers D_int = round(D 2^s) (|D_int| < 2^55) and written
 //     as balanced digits b_d in [-128, 128] (seven, and an eighth below the
 //     binary point);
@@ -179,7 +178,7 @@ extern "C" hb_status hb_tc_selftest(int mode, const float *A_host, const float *
 //     without rounding. For each diagonal t = j + d <= 7 the MMA forms
 //     S_t = sum_{j+d=t} sum_m b_d[i][m] u_j[m] in its own accumulator
 //     column; D u = 2^(E-s) sum_t 256^(12-t) S_t up to the dropped diagonals
-//     t >= 8, which weigh below 2^-58 of the largest term;
+//     t >= 8, which weigh below 2^-60 of the largest term;
 //   - a digit enters the MMA as the FP16 number 256 + u_j (384 + u_0), whose
 //     bit pattern is 0x5C00 | (u_j << 2): no conversion instruction. The
 //     offsets contribute a constant per accumulator column, replaced inside the
@@ -282,19 +281,22 @@ struct tc_args {
 // |v|'s high word: the largest of several carries the largest exponent (>> 20)
 __device__ __forceinline__ unsigned abs_hi(double v) { return (unsigned)__double2hiint(v) & 0x7FFFFFFFu; }
 
-// v on the grid of unit 2^(emax - 1075): round(|v| / unit) with the sign of v
-// (|result| < 2^53; zero and subnormal v give 0). Integer instructions only:
-// 64-bit conversions run at the FP64 rate on this GPU.
+// v on the grid of unit 2^(emax - 1077): round(|v| / unit) with the sign of v
+// (|result| < 2^55; zero and subnormal v give 0). The two bits below a double's
+// last keep the values within two binades of the largest exact and cut the
+// rounding of the others to a quarter, at no cost: they fill the leading digit.
+// Integer instructions only: 64-bit conversions run at the FP64 rate on this GPU.
+constexpr int kUnit = 1077;
 __device__ __forceinline__ long long to_fixed(double v, unsigned emax)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     const unsigned e = (unsigned)(b >> 52) & 0x7FFu;
-    // 2m with the implicit bit (m the 53-bit significand), shifted out whole
+    // 8m with the implicit bit (m the 53-bit significand), shifted out whole
     // for zero and subnormals
-    const unsigned long long m2 = ((b << 1) & 0x1FFFFFFFFFFFFEull) | (1ull << 53);
+    const unsigned long long m8 = ((b << 3) & 0x7FFFFFFFFFFFF8ull) | (1ull << 55);
     const unsigned sh = e ? min(emax - e, 62u) : 62u;
-    // round(m / 2^sh), halves up: (floor(2m / 2^sh) + 1) / 2
-    const long long X = (long long)(((m2 >> sh) + 1ull) >> 1);
+    // round(4m / 2^sh), halves up: (floor(8m / 2^sh) + 1) / 2
+    const long long X = (long long)(((m8 >> sh) + 1ull) >> 1);
     return (b >> 63) ? -X : X;
 }
 
@@ -317,9 +319,10 @@ __device__ __forceinline__ double i64_to_double(long long T, int off)
     return __longlong_as_double((long long)r);
 }
 
-// floor((2^32 hi + lo) / 2^10) for |hi| < 2^41: what an int64 holds of the sum.
-// (Its unit is a sixteenth of the error that rounding the values to the
-// element's grid leaves in it.)
+// floor((2^32 hi + lo) / 2^10) for |hi| < 2^41: what an int64 holds of the sum,
+// rounded to nearest where combine has added the half. (Its unit is at most 2^-60
+// of the largest product, 1/16 of what the rounding of the values to their grid
+// leaves in the sum.)
 __device__ __forceinline__ long long halves(long long hi, long long lo)
 {
     hi += lo >> 32;
@@ -393,6 +396,8 @@ __device__ __forceinline__ void mma_done(uint64_t *bar, unsigned &phase, int war
 // the output is 2^72 hi + 2^40 lo in units of the element's grid times 2^-s.
 // A column holds S_t + 1.5 2^23 (the bias comes with the offset correction), so
 // S_t, an integer below 2^22 in magnitude, is its bits - 0x4B400000.
+// HALF: with 2^9 added, so that halves() rounds to nearest.
+template <bool HALF>
 __device__ __forceinline__ void combine(const uint32_t (&v)[16], int o, long long &hi, long long &lo)
 {
     const uint32_t *B = v + o * 8;
@@ -401,14 +406,14 @@ __device__ __forceinline__ void combine(const uint32_t (&v)[16], int o, long lon
     const int m0 = (int)(B[0] * 256u + B[1] - kBias);
     const int m1 = (int)(B[2] * 256u + B[3] - kBias);
     const int m2 = (int)(B[4] * 256u + B[5] - kBias);
-    const int m3 = (int)(B[6] * 256u + B[7] - kBias);
+    const int m3 = (int)(B[6] * 256u + B[7] - kBias + (HALF ? 512u : 0u));
     hi = (long long)m0 * 65536 + m1;
     lo = (long long)m2 * 65536 + m3;
 }
 
 // Reads the thread's KH = 4 outputs of one direction out of tensor memory (its
 // lane, columns from taddr) and hands each one's two halves to f(q, hi, lo).
-template <class C, class F>
+template <class C, bool HALF, class F>
 __device__ __forceinline__ void read_out(unsigned taddr, F &&f)
 {
     static_assert(C::KH == 4, "two loads of 16 columns");
@@ -422,7 +427,7 @@ __device__ __forceinline__ void read_out(unsigned taddr, F &&f)
 #pragma unroll
         for (int o = 0; o < 2; o++) {
             long long hi, lo;
-            combine(vv[c], o, hi, lo);
+            combine<HALF>(vv[c], o, hi, lo);
             f(2 * c + o, hi, lo);
         }
 }
@@ -558,7 +563,7 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
         }
         mma_done(bar, phase, warp, A.err, gave_up);
         // gradients in units of 2^goff: their scale meets only the exponents
-        const int goff = (int)eu - 1075 - dshift + 40 + 10;
+        const int goff = (int)eu - kUnit - dshift + 40 + 10;
         const bool ubad = eu == 0x7FFu;
         auto value = [&](long long hi, long long lo) {
             return ubad ? __longlong_as_double(0x7FF8000000000000ll) : i64_to_double<false>(halves(hi, lo), 0);
@@ -566,7 +571,7 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
         if constexpr (C::RESTAGE) stage<C, 2>(sm, el, ti, tj, k0, X);
         // ---- gradient along r into its exchange buffer; its columns are free
         // for the t chain once every thread has read them
-        read_out<C>(tl, [&](int q, long long hi, long long lo) { ExR[C::xq(el, k0 + q, ti, tj)] = value(hi, lo); });
+        read_out<C, true>(tl, [&](int q, long long hi, long long lo) { ExR[C::xq(el, k0 + q, ti, tj)] = value(hi, lo); });
         if constexpr (C::RESTAGE) hbtc::fence_async_smem();
         hbtc::fence_before_sync();
         __syncthreads();
@@ -575,11 +580,11 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
             issue<C, 2>(tmem, 0, sm, Bi);
             hbtc::mma_commit(bar);
         }
-        read_out<C>(tl + C::DCOLS,
+        read_out<C, true>(tl + C::DCOLS,
                     [&](int q, long long hi, long long lo) { ExS[C::xq(el, ti, k0 + q, tj)] = value(hi, lo); });
         mma_done(bar, phase, warp, A.err, gave_up);
         double gt[KH];
-        read_out<C>(tl, [&](int q, long long hi, long long lo) { gt[q] = value(hi, lo); });
+        read_out<C, true>(tl, [&](int q, long long hi, long long lo) { gt[q] = value(hi, lo); });
         // ---- metric (FP64): v = G grad at the thread's nodes, factors loaded here
         double vr[KH], vs[KH], vt[KH];
         unsigned evm = 0;
@@ -623,7 +628,7 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
         mma_done(bar, phase, warp, A.err, gave_up);
         if constexpr (C::RESTAGE) stage<C, 2>(sm, el, ti, tj, k0, X);
         // ---- D^T along r and s summed exactly in the exchange buffers
-        read_out<C>(tl, [&](int q, long long hi, long long lo) {
+        read_out<C, false>(tl, [&](int q, long long hi, long long lo) {
             const int xi = C::xq(el, k0 + q, ti, tj);
             Yhi[xi] = hi;
             Ylo[xi] = lo;
@@ -636,19 +641,19 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
             issue<C, 2>(tmem, 0, sm, Bi + C::BIMG);
             hbtc::mma_commit(bar);
         }
-        read_out<C>(tl + C::DCOLS, [&](int q, long long hi, long long lo) {
+        read_out<C, false>(tl + C::DCOLS, [&](int q, long long hi, long long lo) {
             const int xi = C::xq(el, ti, k0 + q, tj);
             Yhi[xi] += hi;
             Ylo[xi] += lo;
         });
         mma_done(bar, phase, warp, A.err, gave_up);
         {
-            const int yoff = (int)ev - 1075 - dshift + 40 + 10 + goff;
+            const int yoff = (int)ev - kUnit - dshift + 40 + 10 + goff;
             const bool vbad = ev == 0x7FFu;
             double *ys = A.ysurf + e * NS;
             const bool ring = ti == 0 || ti == N || tj == 0 || tj == N;
             const int r = tj == 0 ? ti : (tj == N ? n + ti : 2 * n + 2 * (tj - 1) + (ti == N ? 1 : 0));
-            read_out<C>(tl, [&](int q, long long hi, long long lo) {
+            read_out<C, true>(tl, [&](int q, long long hi, long long lo) {
                 const int k = k0 + q, xi = C::xq(el, ti, tj, k);
                 hi += Yhi[xi];
                 lo += Ylo[xi];
@@ -799,9 +804,9 @@ static void derivative_dd(int N, const double *xi, dd (&D)[16][16])
 // be most of the kernel's error) is split into eight digits: D_int = D 2^s,
 // with |D_int| < 2^55 and eight binary places (the eighth digit meets only the
 // leading digit of the values, on the last diagonal). Largest sum of magnitudes
-// an accumulator can meet (digits, offsets and the correction), without the bias:
-// 2^19.3, 2^21.0 and 2^22.0 for N = 3, 7, 15; with the bias, 1.5 2^23, below the
-// 2^24 that FP32 holds exactly. The sums S_t stay below 2^20.7.
+// an accumulator can meet (digits, offsets and the correction with the bias): 0.77,
+// 0.81 and 0.87 of the 2^24 that FP32 holds exactly, for N = 3, 7, 15. The sums S_t
+// stay below 2^20.8.
 hb_status hb_tc_upload()
 {
     using namespace tcax;
