@@ -489,11 +489,13 @@ double hb_u01(uint64_t seed, uint64_t stream, uint64_t idx);
  *                         on the tensor cores (tcgen05.mma, FP16 inputs, FP32
  *                         accumulators in tensor memory) exactly, on an
  *                         Ozaki-style split of the element's values and of D into
- *                         8-bit digits (seven, eight for D) on a per-element fixed-point grid
+ *                         8-bit digits (seven, eight for D) on a fixed-point grid
  *                         (every product and partial sum an integer below 2^24);
  *                         the exact digit sums are combined in int64 and the
- *                         metric step runs in FP64. Error per contraction about
- *                         2^-53 of the element's largest |value| times sum |D|,
+ *                         metric step runs in FP64. The grid follows every line
+ *                         at N = 3 and 15, the element at N = 7: the error of a
+ *                         contraction is about 2^-55 of the largest |value| of
+ *                         its line (N = 7: of its element) times sum |D|, below
  *                         the FP64 rounding level; an element holding a
  *                         non-finite value gives NaN. Same surface store and
  *                         gather as the pencil kernels (with CSR: the CSR-position

@@ -166,10 +166,14 @@ extern "C" hb_status hb_tc_selftest(int mode, const float *A_host, const float *
 // cores.
 //
 // Exact contractions from FP16 products (an Ozaki-style split into slices):
-//   - the element's values u are put on one fixed-point grid,
-//     X = round(u / 2^E) with 2^E two bits below the last of the element's
-//     largest value (|X| < 2^55), and written as seven base-256 digits,
-//     X = sum_j u_j 256^(6-j), u_0 a signed byte, u_1..u_6 unsigned ones;
+//   - the values u are put on a fixed-point grid, X = round(u / 2^E) with 2^E two
+//     bits below the last of the largest value (|X| < 2^55), and written as seven
+//     base-256 digits, X = sum_j u_j 256^(6-j), u_0 a signed byte, u_1..u_6
+//     unsigned ones. N = 3 and 15: a grid for every line, so a contraction is
+//     accurate to its own line, as in floating point, whatever else the element
+//     holds, and the directions are added as doubles. N = 7: a grid for the
+//     element, on which the directions' sums are added exactly; a line far below
+//     the element's largest value loses the bits between;
 //   - D is scaled to integers D_int = round(D 2^s) (|D_int| < 2^55) and written
 //     as balanced digits b_d in [-128, 128] (seven, and an eighth below the
 //     binary point);
@@ -185,9 +189,9 @@ extern "C" hb_status hb_tc_selftest(int mode, const float *A_host, const float *
 //     same MMA by 1.5 2^23 with an eighth K block: 128 in the A operand times
 //     (1.5 2^23 - constant) / 128 (split into FP16-exact parts) in the B operand;
 //   - so a column's bits are 0x4B400000 + S_t: the exact integers are combined in
-//     two int64 halves and turned into doubles by integer instructions; the
-//     gradients stay in units of the element's grid (the scale rejoins at the
-//     end, in the exponent).
+//     two int64 halves and turned into doubles by integer instructions; at N = 7
+//     the gradients stay in units of the element's grid (the scale rejoins at
+//     the end, in the exponent).
 // n = N + 1 is a power of two, so the lines of whole elements fill M-tiles of
 // 128 rows. Per M-tile and direction: one MMA chain of n / 2 K = 16 steps, A =
 // the lines' digits (128 x 8 n, K-major, K ordered (line position m, digit j)
@@ -208,11 +212,18 @@ namespace tcax {
 // three blocks of 78 registers and its own t operand, 4.42 with four; N = 15
 // 6.43 with 512 threads, 6.16 with 1024. With the accumulators biased, the
 // gradients left unscaled and one 64-bit value per sum (fewer integer
-// instructions, the busiest pipe beside FP64) 3.94, 4.25 and 5.85. (The FP64
-// pencil kernel: 8.68, 11.8 and 17.4.)
+// instructions, the busiest pipe beside FP64) 3.94, 4.25 and 5.86. A grid per line
+// at N = 3 and 15 (two more fixed-point and two more double conversions a node,
+// and the lines' maxima): 4.84 and 6.86. (The FP64 pencil kernel: 8.68, 11.8 and
+// 17.4.)
 template <int N_>
 struct shape {
     static constexpr int N = N_, n = N + 1, n2 = n * n, n3 = n2 * n;
+    // The fixed-point grid follows every line, or the element. By element N = 3 and
+    // 15 take 3.94 and 5.86 ms for 4.84 and 6.86, but one value of 1e8 among values
+    // of 1 left lines that it is not on with 8 digits, where the FP64 pencil kernel
+    // keeps 16.
+    static constexpr bool LINE = n != 8;
     static_assert(n == 4 || n == 8 || n == 16, "the lines of whole elements fill M-tiles of 128 rows");
     static constexpr int NS = 2 * n2 + 4 * N * (N - 1);  // surface nodes of an element
     static constexpr int MT = n == 8 ? 1 : 2, EPT = MT * 128 / n2;
@@ -234,7 +245,9 @@ struct shape {
     static constexpr int BIMG = n2 * 128;  // one B operand image (8 n x 8 n FP16)
     static constexpr int OFF_B = RESTAGE ? A_R + A_S : A_R + A_S + A_T;
     static constexpr int OFF_MISC = OFF_B + 2 * BIMG;
-    static constexpr int SMEM = OFF_MISC + 160;
+    // n = 16: the exponents of the 256 lines of each direction, of u and of v
+    static constexpr int OFF_LX = OFF_MISC + 160, LX = n == 16 ? 3 * 256 : 0;
+    static constexpr int SMEM = OFF_LX + 2 * LX * 4;
     // The exchange buffers (two doubles or two int64 halves per node of the
     // tile) sit in operands whose MMAs are done by then: r and s, or s alone
     static constexpr int EXS = n == 4 ? 80 : n3;  // node stride of an element
@@ -432,25 +445,79 @@ __device__ __forceinline__ void read_out(unsigned taddr, F &&f)
         }
 }
 
-// Largest v over the thread's element. n = 4: its 16 lanes.
-// n = 8: warps 0, 1, 4, 5 hold element 0, warps 2, 3, 6, 7 element 1; n = 16:
-// the block's 32 warps. Every thread calls it; it synchronises the block.
-template <class C>
+// N = 7: largest v over the thread's element (warps 0, 1, 4, 5 hold element 0,
+// warps 2, 3, 6, 7 element 1). Every thread calls it; it synchronises the block.
 __device__ __forceinline__ unsigned element_max(unsigned v, unsigned *wexp, int el)
 {
-    if constexpr (C::n == 4) {
-        for (int o = 8; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-        __syncthreads();
-        return v;
-    } else {
-        v = __reduce_max_sync(0xffffffffu, v);
-        if ((threadIdx.x & 31) == 0) wexp[threadIdx.x >> 5] = v;
-        __syncthreads();
-        if constexpr (C::n == 8)
-            return max(max(wexp[2 * el], wexp[2 * el + 1]), max(wexp[4 + 2 * el], wexp[5 + 2 * el]));
-        else
-            return __reduce_max_sync(0xffffffffu, wexp[threadIdx.x & 31]);
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) wexp[threadIdx.x >> 5] = v;
+    __syncthreads();
+    return max(max(wexp[2 * el], wexp[2 * el + 1]), max(wexp[4 + 2 * el], wexp[5 + 2 * el]));
+}
+
+// N = 3, 15: the exponents of a thread's four nodes, two 16-bit fields a word
+struct exps {
+    unsigned w[2];
+    __device__ __forceinline__ explicit exps(const double (&v)[4])
+    {
+        w[0] = (abs_hi(v[0]) >> 20) | (abs_hi(v[1]) >> 20 << 16);
+        w[1] = (abs_hi(v[2]) >> 20) | (abs_hi(v[3]) >> 20 << 16);
     }
+    __device__ __forceinline__ unsigned at(int q) const { return ((q & 2 ? w[1] : w[0]) >> (q & 1 ? 16 : 0)) & 0xFFFFu; }
+    __device__ __forceinline__ unsigned largest() const
+    {
+        const unsigned m = __vmaxu2(w[0], w[1]);
+        return max(m & 0xFFFFu, m >> 16);
+    }
+    // field by field over the lanes that differ in the bits of the masks lo, 2 lo, ..., hi
+    __device__ __forceinline__ void over_lanes(int lo, int hi)
+    {
+        for (int o = lo; o <= hi; o <<= 1)
+            for (int c = 0; c < 2; c++) w[c] = __vmaxu2(w[c], __shfl_xor_sync(0xffffffffu, w[c], o));
+    }
+};
+
+// The largest exponents along the lines: in er, es (in: of the thread's nodes, by
+// what they enter along r and s; out: of their r- and s-lines) and et (out: of its
+// t-line); row: of the three lines that are the thread's rows of the r, s and t
+// operands; bad: whether any thread of the element passes true. n = 4: an element
+// is 16 lanes, all by shuffles. n = 16: r-lines are 16 lanes; s-lines meet in the
+// exponents lx in shared memory, as do the t-lines (both zero before the call),
+// which synchronises the block.
+template <class C>
+__device__ __forceinline__ void line_max(exps &er, exps &es, const exps &t, unsigned &et, unsigned (&row)[3],
+                                         bool &bad, unsigned *lx, int line, int ti, int tj, int k0)
+{
+    et = t.largest();
+    if constexpr (C::n == 4) {
+        er.over_lanes(1, 2);
+        es.over_lanes(4, 8);
+        // row (k, j) = (tj, ti) of r: held by the lanes of tj = ti; row (k, i) = (tj, ti) of s: here
+        exps o = er;
+        for (int c = 0; c < 2; c++) o.w[c] = __shfl_sync(0xffffffffu, er.w[c], (threadIdx.x & 16) | (ti * 4));
+        row[0] = o.at(tj);
+        row[1] = es.at(tj);
+        bad = ((__ballot_sync(0xffffffffu, bad) >> (threadIdx.x & 16)) & 0xFFFFu) != 0;
+    } else {
+        er.over_lanes(1, 8);
+        es.over_lanes(16, 16);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            if (ti == 0) lx[(k0 + q) * 16 + tj] = er.at(q);
+            if ((threadIdx.x & 31) < 16) atomicMax(&lx[256 + (k0 + q) * 16 + ti], es.at(q));
+        }
+        atomicMax(&lx[512 + line], et);
+        bad = __syncthreads_or(bad) != 0;
+        unsigned v[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) v[q] = lx[256 + (k0 + q) * 16 + ti];
+        es.w[0] = v[0] | v[1] << 16;
+        es.w[1] = v[2] | v[3] << 16;
+        row[0] = lx[line];
+        row[1] = lx[256 + line];
+        et = lx[512 + line];
+    }
+    row[2] = et;
 }
 
 // Thread tid: M-tile mt, TMEM lane tid % 128: line mt 128 + lane of the tile
@@ -481,7 +548,9 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + C::OFF_MISC);
     unsigned *tptr = reinterpret_cast<unsigned *>(sm + C::OFF_MISC + 8);
     unsigned *wexp = reinterpret_cast<unsigned *>(sm + C::OFF_MISC + 16);
+    unsigned *lxu = reinterpret_cast<unsigned *>(sm + C::OFF_LX), *lxv = lxu + C::LX;
 
+    for (int q = tid; q < 2 * C::LX; q += C::THREADS) lxu[q] = 0;
     for (int q = tid; q < 2 * C::BIMG / 16; q += C::THREADS)
         reinterpret_cast<uint4 *>(Bi)[q] = reinterpret_cast<const uint4 *>(g_tc_bimg + img_off(N))[q];
     if (tid == 0) {
@@ -542,15 +611,32 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
             }
         }
-        unsigned em = 0;
-#pragma unroll
-        for (int q = 0; q < KH; q++) em = max(em, abs_hi(u[q]));
-        const unsigned eu = element_max<C>(em, wexp, el) >> 20;
         long long X[KH];
+        unsigned eu = 0, row[3];
+        if constexpr (C::LINE) {
+            exps er(u), es(u);
+            bool bad = false;  // (a non-finite line shows in its exponent)
+            line_max<C>(er, es, exps(u), eu, row, bad, lxu, line, ti, tj, k0);
 #pragma unroll
-        for (int q = 0; q < KH; q++) X[q] = eu == 0x7FFu ? 0 : to_fixed(u[q], eu);
-        stage<C, 0>(sm, el, ti, tj, k0, X);
-        stage<C, 1>(sm, el, ti, tj, k0, X);
+            for (int q = 0; q < KH; q++) X[q] = to_fixed(u[q], er.at(q));
+            stage<C, 0>(sm, el, ti, tj, k0, X);
+#pragma unroll
+            for (int q = 0; q < KH; q++) X[q] = to_fixed(u[q], es.at(q));
+            stage<C, 1>(sm, el, ti, tj, k0, X);
+#pragma unroll
+            for (int q = 0; q < KH; q++) X[q] = to_fixed(u[q], eu);
+            // (the s- and t-lines' words for v, read in the tile before)
+            for (int q = 256 + tid; q < C::LX; q += C::THREADS) lxv[q] = 0;
+        } else {
+#pragma unroll
+            for (int q = 0; q < KH; q++) eu = max(eu, abs_hi(u[q]));
+            eu = element_max(eu, wexp, el) >> 20;
+            row[0] = row[1] = row[2] = eu;
+#pragma unroll
+            for (int q = 0; q < KH; q++) X[q] = eu == 0x7FFu ? 0 : to_fixed(u[q], eu);
+            stage<C, 0>(sm, el, ti, tj, k0, X);
+            stage<C, 1>(sm, el, ti, tj, k0, X);
+        }
         if constexpr (!C::RESTAGE) stage<C, 2>(sm, el, ti, tj, k0, X);
         hbtc::fence_async_smem();
         hbtc::fence_before_sync();
@@ -562,16 +648,18 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
             hbtc::mma_commit(bar);
         }
         mma_done(bar, phase, warp, A.err, gave_up);
-        // gradients in units of 2^goff: their scale meets only the exponents
-        const int goff = (int)eu - kUnit - dshift + 40 + 10;
-        const bool ubad = eu == 0x7FFu;
-        auto value = [&](long long hi, long long lo) {
-            return ubad ? __longlong_as_double(0x7FF8000000000000ll) : i64_to_double<false>(halves(hi, lo), 0);
+        // LINE: gradients by the exponent of their line. Else in units of 2^goff:
+        // the element's scale meets only the exponents of the results.
+        const int scale = 40 + 10 - kUnit - dshift;
+        const int goff = C::LINE ? 0 : (int)eu + scale;
+        auto value = [&](int dir, long long hi, long long lo) {
+            return row[dir] == 0x7FFu ? __longlong_as_double(0x7FF8000000000000ll)
+                                      : i64_to_double<C::LINE>(halves(hi, lo), (int)row[dir] + scale);
         };
         if constexpr (C::RESTAGE) stage<C, 2>(sm, el, ti, tj, k0, X);
         // ---- gradient along r into its exchange buffer; its columns are free
         // for the t chain once every thread has read them
-        read_out<C, true>(tl, [&](int q, long long hi, long long lo) { ExR[C::xq(el, k0 + q, ti, tj)] = value(hi, lo); });
+        read_out<C, true>(tl, [&](int q, long long hi, long long lo) { ExR[C::xq(el, k0 + q, ti, tj)] = value(0, hi, lo); });
         if constexpr (C::RESTAGE) hbtc::fence_async_smem();
         hbtc::fence_before_sync();
         __syncthreads();
@@ -581,10 +669,10 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
             hbtc::mma_commit(bar);
         }
         read_out<C, true>(tl + C::DCOLS,
-                    [&](int q, long long hi, long long lo) { ExS[C::xq(el, ti, k0 + q, tj)] = value(hi, lo); });
+                          [&](int q, long long hi, long long lo) { ExS[C::xq(el, ti, k0 + q, tj)] = value(1, hi, lo); });
         mma_done(bar, phase, warp, A.err, gave_up);
         double gt[KH];
-        read_out<C, true>(tl, [&](int q, long long hi, long long lo) { gt[q] = value(hi, lo); });
+        read_out<C, true>(tl, [&](int q, long long hi, long long lo) { gt[q] = value(2, hi, lo); });
         // ---- metric (FP64): v = G grad at the thread's nodes, factors loaded here
         double vr[KH], vs[KH], vt[KH];
         unsigned evm = 0;
@@ -603,17 +691,36 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
                 evm = max(evm, max(abs_hi(vr[q]), max(abs_hi(vs[q]), abs_hi(vt[q]))));
             }
         }
-        // (element_max meets the block: every exchange read is done before
-        // the operands are staged over the exchange buffers)
-        const unsigned ev = element_max<C>(evm, wexp, el) >> 20;
+        // A non-finite value makes the whole element NaN. (The block meets here,
+        // in every form: every exchange read is done before the operands are
+        // staged over the exchange buffers.)
+        unsigned ev;
+        bool vbad = evm >> 20 == 0x7FFu;
+        if constexpr (C::LINE) {
+            exps er(vr), es(vs);
+            if constexpr (n == 4) __syncthreads();
+            line_max<C>(er, es, exps(vt), ev, row, vbad, lxv, line, ti, tj, k0);
+            for (int q = 256 + tid; q < C::LX; q += C::THREADS) lxu[q] = 0;
 #pragma unroll
-        for (int q = 0; q < KH; q++) X[q] = ev == 0x7FFu ? 0 : to_fixed(vr[q], ev);
-        stage<C, 0>(sm, el, ti, tj, k0, X);
+            for (int q = 0; q < KH; q++) X[q] = to_fixed(vr[q], er.at(q));
+            stage<C, 0>(sm, el, ti, tj, k0, X);
 #pragma unroll
-        for (int q = 0; q < KH; q++) X[q] = ev == 0x7FFu ? 0 : to_fixed(vs[q], ev);
-        stage<C, 1>(sm, el, ti, tj, k0, X);
+            for (int q = 0; q < KH; q++) X[q] = to_fixed(vs[q], es.at(q));
+            stage<C, 1>(sm, el, ti, tj, k0, X);
 #pragma unroll
-        for (int q = 0; q < KH; q++) X[q] = ev == 0x7FFu ? 0 : to_fixed(vt[q], ev);
+            for (int q = 0; q < KH; q++) X[q] = to_fixed(vt[q], ev);
+        } else {
+            ev = element_max(evm, wexp, el) >> 20;
+            vbad = ev == 0x7FFu;
+#pragma unroll
+            for (int q = 0; q < KH; q++) X[q] = vbad ? 0 : to_fixed(vr[q], ev);
+            stage<C, 0>(sm, el, ti, tj, k0, X);
+#pragma unroll
+            for (int q = 0; q < KH; q++) X[q] = vbad ? 0 : to_fixed(vs[q], ev);
+            stage<C, 1>(sm, el, ti, tj, k0, X);
+#pragma unroll
+            for (int q = 0; q < KH; q++) X[q] = vbad ? 0 : to_fixed(vt[q], ev);
+        }
         if constexpr (!C::RESTAGE) stage<C, 2>(sm, el, ti, tj, k0, X);
         hbtc::fence_async_smem();
         hbtc::fence_before_sync();
@@ -627,11 +734,16 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
         gather(g + gridDim.x);
         mma_done(bar, phase, warp, A.err, gave_up);
         if constexpr (C::RESTAGE) stage<C, 2>(sm, el, ti, tj, k0, X);
-        // ---- D^T along r and s summed exactly in the exchange buffers
-        read_out<C, false>(tl, [&](int q, long long hi, long long lo) {
+        // ---- D^T along r and s summed in the exchange buffers: the directions
+        // share a grid and are added exactly, or (LINE) as doubles
+        read_out<C, C::LINE>(tl, [&](int q, long long hi, long long lo) {
             const int xi = C::xq(el, k0 + q, ti, tj);
-            Yhi[xi] = hi;
-            Ylo[xi] = lo;
+            if constexpr (C::LINE) {
+                ExR[xi] = value(0, hi, lo);
+            } else {
+                Yhi[xi] = hi;
+                Ylo[xi] = lo;
+            }
         });
         if constexpr (C::RESTAGE) hbtc::fence_async_smem();
         hbtc::fence_before_sync();
@@ -641,23 +753,32 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
             issue<C, 2>(tmem, 0, sm, Bi + C::BIMG);
             hbtc::mma_commit(bar);
         }
-        read_out<C, false>(tl + C::DCOLS, [&](int q, long long hi, long long lo) {
+        read_out<C, C::LINE>(tl + C::DCOLS, [&](int q, long long hi, long long lo) {
             const int xi = C::xq(el, ti, k0 + q, tj);
-            Yhi[xi] += hi;
-            Ylo[xi] += lo;
+            if constexpr (C::LINE) {
+                ExR[xi] += value(1, hi, lo);
+            } else {
+                Yhi[xi] += hi;
+                Ylo[xi] += lo;
+            }
         });
         mma_done(bar, phase, warp, A.err, gave_up);
         {
-            const int yoff = (int)ev - kUnit - dshift + 40 + 10 + goff;
-            const bool vbad = ev == 0x7FFu;
+            const int yoff = (int)ev + scale + goff;
             double *ys = A.ysurf + e * NS;
             const bool ring = ti == 0 || ti == N || tj == 0 || tj == N;
             const int r = tj == 0 ? ti : (tj == N ? n + ti : 2 * n + 2 * (tj - 1) + (ti == N ? 1 : 0));
             read_out<C, true>(tl, [&](int q, long long hi, long long lo) {
                 const int k = k0 + q, xi = C::xq(el, ti, tj, k);
-                hi += Yhi[xi];
-                lo += Ylo[xi];
-                const double yc = vbad ? __longlong_as_double(0x7FF8000000000000ll) : i64_to_double<true>(halves(hi, lo), yoff);
+                double yc;
+                if constexpr (C::LINE) {
+                    yc = ExR[xi] + i64_to_double<true>(halves(hi, lo), yoff);
+                } else {
+                    hi += Yhi[xi];
+                    lo += Ylo[xi];
+                    yc = i64_to_double<true>(halves(hi, lo), yoff);
+                }
+                if (vbad) yc = __longlong_as_double(0x7FF8000000000000ll);
                 if (!active) return;
                 if (SP && (k == 0 || k == N || ring)) {
                     const int sidx = k == 0 ? a : (k == N ? n2 + a : 2 * n2 + (k - 1) * 4 * N + r);
