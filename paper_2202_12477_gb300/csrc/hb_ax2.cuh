@@ -663,9 +663,9 @@ constexpr double element_us()
            (std::is_same<T, double>::value ? 4140.0 : 10000.0);
 }
 
-// Blocks per element, E elements on 152 SMs: the power of two for which the
-// largest block's share of the element plus 1.5 us per doubling (the exchange,
-// the shorter loops) is least, while every block has an SM of its own.
+// Blocks per element, E elements: the power of two for which the largest
+// block's share of the element plus 1.5 us per doubling (the exchange, the
+// shorter loops) is least, while there are no more blocks than SMs (HB_SMS).
 // Measured, FP64 A x in us with C = 1 / 2 / 4: N = 7 and 27 elements 16.6 /
 // 12.8 / 13.2, 64 elements 17.1 / 13.3 / 14.5; N = 3, 27: 8.6 / 9.9 / 9.9;
 // N = 15, 27: 98 / 57 / 36; two blocks per SM gain nothing (N = 9, 125
@@ -675,7 +675,7 @@ inline int cluster_blocks(int64_t E)
 {
     int best = 1;
     double cost = element_us<N>();
-    for (int C = 2; C <= 4 && E * C <= 152 && C <= split<N>::half; C *= 2) {
+    for (int C = 2; C <= 4 && E * C <= HB_SMS && C <= split<N>::half; C *= 2) {
         const double c = element_us<N>() * split<N>::slabs(C) / (N + 1) + 1.5 * (C == 2 ? 1 : 2);
         if (c < cost) {
             cost = c;
@@ -707,7 +707,7 @@ inline int split_blocks(int64_t E)
     constexpr int n2 = (N + 1) * (N + 1), EB = n2 >= 256 ? 1 : 256 / n2;
     const int C = cluster_blocks<N>(E);
     if (C > 1) return C;
-    const int64_t q0 = ((E + EB - 1) / EB + 151) / 152 * EB, q = (E + 151) / 152;
+    const int64_t q0 = ((E + EB - 1) / EB + HB_SMS - 1) / HB_SMS * EB, q = (E + HB_SMS - 1) / HB_SMS;
     if (4 * q <= 3 * q0 && q <= 8) return 1;
     return !std::is_same<T, S>::value && N >= 11 ? (N == 15 ? 2 : 1) : 0;
 }

@@ -634,10 +634,10 @@ extern "C" hb_status hb_autotune(hb_mesh *m, hb_precision prec, hb_screen screen
     return st;
 }
 
-// Workspace vectors for the solvers, grown on demand (FP64 r, p, Ap; FP32 r, p,
-// Ap, d), each starting on a 256-byte boundary.
+// Workspace vectors for the solvers, grown on demand (FP64 r, p, Ap and z, which
+// is the fused CG's second p; FP32 r, p, Ap, d and z), each starting on a 256-byte
+// boundary.
 static inline int64_t cg_stride(int64_t n) { return (n + 63) / 64 * 64; }
-// Workspace vectors for the solvers, grown on demand (FP64 r, p, Ap; FP32 r, p, Ap, d).
 static hb_status cg_workspace(hb_mesh *m)
 {
     const size_t need = (size_t)cg_stride(m->n_global) * (4 * sizeof(double) + 5 * sizeof(float)) + 256;
@@ -796,7 +796,7 @@ static bool use_fused_cg(const hb_mesh *m, const hb_cg_opts *o)
     const int cap = hb_cg_fused_capacity(m->N);
     if (cap <= 0 || m->E > cap) return false;
     if (m->fused_mode == 2) return true;
-    if ((m->N >= 11 && 2 * m->E <= 152) || (m->N == 10 && 4 * m->E <= 152)) return false;
+    if ((m->N >= 11 && 2 * m->E <= HB_SMS) || (m->N == 10 && 4 * m->E <= HB_SMS)) return false;
     return m->E <= 300;
 }
 

@@ -10,6 +10,10 @@
 #include "hipbone_gb300.h"
 
 #define HB_MAX_N 15
+// SMs of a GB300: what the rules for small meshes count with (the element
+// kernel's blocks per element, the room for their partials, the fused CG's
+// range). On another count the results are the same, the choice not the fastest.
+#define HB_SMS 152
 #define HB_RED_BLOCKS 1216  // fixed grid of every reduction kernel (8 x 152 SMs)
 #define HB_RED_MAXV 4       // values one grid reduction may carry (rows of the partials buffer)
 #define HB_RED_THREADS 256
@@ -121,7 +125,7 @@ struct hb_mesh {
     unsigned *counters; // [8]
     hb_cg_state *state; // device CG states [4]: 0 outer/FP64, 1 inner/dot
     hb_cg_state *state_host;  // pinned mirror
-    void *cg_vec;       // r, p, Ap (FP64) then FP32 inner vectors
+    void *cg_vec;       // r, p, Ap, z (FP64) then FP32 inner vectors
     size_t cg_vec_bytes;
     double min_detJ;
     size_t device_bytes;

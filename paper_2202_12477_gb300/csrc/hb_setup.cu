@@ -5,8 +5,9 @@
 //   - GLL nodes by Newton's method on q(x) = (1-x^2) P_N'(x) written as
 //     N (P_{N-1}(x) - x P_N(x)), with q'(x) = -N(N+1) P_N(x);
 //   - the derivative matrix from barycentric weights, diagonal by negative sums;
-//   - the Jacobian by applying that derivative matrix to the nodal coordinates
-//     (exact, since a trilinear map is a polynomial of degree 1 <= N per axis).
+//   - the Jacobian's columns from halved edge differences of the element's eight
+//     vertices, bilinear in the other two coordinates (the trilinear map has no
+//     other terms), not by applying the derivative matrix to nodal coordinates.
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
@@ -635,9 +636,9 @@ extern "C" hb_status hb_mesh_create(const hb_mesh_desc *d, void *stream, hb_mesh
     HB_TRY_MESH(alloc((void **)&m->srow_g, sizeof(int32_t) * (m->nsr + 1)));
     HB_TRY_MESH(alloc((void **)&m->srowptr, sizeof(int32_t) * (m->nsr + 1)));
     HB_TRY_MESH(alloc((void **)&m->scols, sizeof(int32_t) * (m->nnz_s > 0 ? m->nnz_s : 1)));
-    // one partial per element-kernel block: at most two per element, or as many
-    // as there are SMs (a small mesh split over more)
-    m->n_ax_partials = 2 * E + 152;
+    // one partial per element-kernel block: at most two per element, or HB_SMS (a
+    // small mesh split over more, cluster_blocks)
+    m->n_ax_partials = 2 * E + HB_SMS;
     HB_TRY_MESH(alloc((void **)&m->ax_partials, sizeof(double) * m->n_ax_partials));
     HB_TRY_MESH(alloc((void **)&m->yL, sizeof(double) * n_local));
     HB_TRY_MESH(alloc((void **)&m->partials, sizeof(double) * HB_RED_MAXV * HB_RED_BLOCKS));
