@@ -523,7 +523,7 @@ def run_sweep(args, rank, world, local):
             for var in variants:
                 if var is not None:
                     hb.hb_set_kernel_variant(m.handle, varprec, var)
-                var = hb.hb_get_kernel_variant(m.handle, varprec)
+                var = hb.hb_get_apply_variant(m.handle, varprec)  # A x alone has its own
                 for _ in range(3):
                     m.apply_A(x, y, lam=0.1, prec=hbprec)
                 torch.cuda.synchronize()
