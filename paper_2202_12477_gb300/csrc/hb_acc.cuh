@@ -3,10 +3,10 @@
 
 namespace hbacc {
 
-// First statement of a kernel that hb_launch_after starts: waits until every
-// kernel before it on the stream is complete and its writes are visible (a
-// kernel that an ordinary launch started is so already), then lets the next
-// one's blocks start as soon as all blocks of this grid run.
+// Before the first access to memory of a kernel that hb_launch_after starts: waits
+// until every kernel before it on the stream is complete and its writes are
+// visible (a kernel that an ordinary launch started is so already), then lets the
+// next one's blocks start as soon as all blocks of this grid run.
 __device__ __forceinline__ void wait_before()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

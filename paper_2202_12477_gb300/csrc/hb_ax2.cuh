@@ -776,7 +776,7 @@ __device__ __forceinline__ void line_part(T (&in)[N + 1], int c, int C, F &&stor
 // Element e by the C blocks of this cluster, this one being block c; sm holds
 // split<N>::smem(C) bytes. load(q, g) gives node q's value of u from its DOF
 // id g >= 0, id(q) the id itself. Every thread of every block must call it.
-template <int N, class FI, class FL>
+template <int N, bool PEERS, class FI, class FL>
 __device__ __forceinline__ void pencil_split(const pencil_args &A, int64_t e, int c, int C, T *sm,
                                              hbacc::dot_acc<S> &acc, FI &&id, FL &&load)
 {
@@ -809,7 +809,7 @@ __device__ __forceinline__ void pencil_split(const pencil_args &A, int64_t e, in
             for (int f = 0; f < 6; f++) G[t][f] = __ldcs(g + f * n2);
         }
     }
-    cluster_arrive();  // (waited for before the first store to a peer)
+    if constexpr (PEERS) cluster_arrive();  // (waited for before the first store to a peer)
     __syncthreads();
     // lines: 2 ns n along r and s in the own slabs, then n^2 along t. A block
     // that owns every slab (C = 1) takes whole t-lines like the others, so no
@@ -841,7 +841,7 @@ __device__ __forceinline__ void pencil_split(const pencil_args &A, int64_t e, in
         }
     }
     __syncthreads();
-    cluster_wait();
+    if constexpr (PEERS) cluster_wait();
     auto metric = [&](int w, const S (&g)[6]) {
         const int q = w / n2, a = w - q * n2, at = a / n * rs + a % n, own = q * ss + at, full = slab(q) * ss + at;
         const T grr = to_c(g[0]), grs = to_c(g[1]), grt = to_c(g[2]), gss = to_c(g[3]), gst = to_c(g[4]),
@@ -851,7 +851,8 @@ __device__ __forceinline__ void pencil_split(const pencil_args &A, int64_t e, in
         B2[own] = fma(gst, ut, fma(gss, us, grs * ur));
         const T vt = fma(gtt, ut, fma(gst, us, grt * ur));
         B3[full] = vt;
-        for (int r = 1; r < C; r++) *peer(B3 + full, c + r < C ? c + r : c + r - C) = vt;
+        if constexpr (PEERS)
+            for (int r = 1; r < C; r++) *peer(B3 + full, c + r < C ? c + r : c + r - C) = vt;
     };
 #pragma unroll
     for (int t = 0; t < PRE; t++)
@@ -863,7 +864,7 @@ __device__ __forceinline__ void pencil_split(const pencil_args &A, int64_t e, in
         for (int q = 0; q < 6; q++) f[q] = __ldcs(g + q * n2);
         metric(w, f);
     }
-    cluster_arrive();
+    if constexpr (PEERS) cluster_arrive();
     __syncthreads();
     // D^T in place along the lines (each is read whole before it is written)
     for (int w = tid; w < whole; w += nt) {
@@ -875,7 +876,7 @@ __device__ __forceinline__ void pencil_split(const pencil_args &A, int64_t e, in
         for (int m = 0; m < n; m++) in[m] = dst[m * step];
         line_st<N, true, true>(in, [&](int m, T v) { dst[m * step] = v; });
     }
-    cluster_wait();  // the peers' v_t is here
+    if constexpr (PEERS) cluster_wait();  // the peers' v_t is here
     // the threads past the r- and s-lines first: the t-lines go to them
     for (int w = C == 1 ? n2 : (tid + nt - 2 * nl % nt) % nt; w < n2; w += nt) {
         const int at = w / n * rs + w % n;
@@ -929,22 +930,32 @@ __device__ __forceinline__ void split_refuse(const pencil_args &A, int64_t e)
 // memory, so it takes its rank and the cluster's size from the hardware, and
 // if those are not the shape asked for (a launch whose cluster attribute was
 // lost on its way), no block touches a peer: bit 2 of the error word and NaN.
-template <int N>
-__global__ void __launch_bounds__(split<N>::MAXT) ax_split_kernel(const pencil_args A, int C)
+// PEERS = false: C = 1, a block alone with its element: no peer to check for, no
+// cluster barriers (us per A x with one kernel for every C, the check in it ->
+// this: FP64 N = 5, 64 elements 11.8 -> 10.8; double-float N = 12, 20^3 850 -> 821).
+// The shape is read before the wait for the kernel before, which hides it (FP64
+// N = 9, 64 elements 21.3 without the check, 21.8 with it behind the wait, 21.4).
+template <int N, bool PEERS>
+__global__ void __launch_bounds__(split<N>::MAXT) ax_split_kernel(const pencil_args A, int blocks)
 {
+    const int C = PEERS ? blocks : 1;
+    bool lost = false;
+    if constexpr (PEERS) {
+        const int c = cluster_rank();
+        if (cluster_size() != C || c != (int)(blockIdx.x % C)) lost = true;
+    }
     hbacc::wait_before();
     if (A.run && *A.run == 0) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     hbacc::dot_acc<S> acc;
     const int64_t e = blockIdx.x / C;
-    const int c = cluster_rank();
-    if (cluster_size() != C || c != (int)(blockIdx.x % C)) {
+    if (lost) {
         split_refuse<N>(A, e);
         return;
     }
     const int32_t *__restrict__ lg = A.l2g + e * split<N>::n3;
     const S *__restrict__ x = A.x;
-    pencil_split<N>(A, e, c, C, reinterpret_cast<T *>(smem_raw), acc,
+    pencil_split<N, PEERS>(A, e, PEERS ? blockIdx.x % C : 0, C, reinterpret_cast<T *>(smem_raw), acc,
                     [&](int q) { return __ldg(lg + q); }, [&](int, int g) { return __ldg(x + g); });
     if (A.partials) {
         const double v = hbacc::block_sum(acc.value());
@@ -1057,7 +1068,7 @@ hb_status launch(const pencil_args &A, int eb_mode, cudaStream_t s, int64_t *nbl
     constexpr int n = N + 1, n2 = n * n;
     constexpr int EB1 = n2 >= 256 ? 1 : 256 / n2;
     if (A.E <= 0) return HB_OK;
-    static int attr_set[10][32] = {{0}};
+    static int attr_set[11][32] = {{0}};
     int dev = 0;
     HB_TRY_CUDA(cudaGetDevice(&dev));
     const bool sp = (eb_mode & 8) != 0;   // CSR-position surface store
@@ -1135,11 +1146,13 @@ hb_status launch(const pencil_args &A, int eb_mode, cudaStream_t s, int64_t *nbl
         if constexpr (EO) {
             const int C = which == 0 ? split_blocks<N>(A.E) : 0;
             if (C > 0) {
-                auto kern = ax_split_kernel<N>;
-                if (dev >= 0 && dev < 32 && !attr_set[9][dev]) {
+                auto kern = ax_split_kernel<N, false>;
+                if constexpr (split<N>::half > 1) kern = C > 1 ? ax_split_kernel<N, true> : kern;
+                int &set = attr_set[C > 1 ? 10 : 9][dev < 0 || dev >= 32 ? 0 : dev];
+                if (dev >= 0 && dev < 32 && !set) {
                     HB_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                      (int)split<N>::smem(1)));
-                    attr_set[9][dev] = 1;
+                    set = 1;
                 }
                 if (nblocks_out) *nblocks_out = A.E * C;
                 cudaLaunchConfig_t cfg = {};

@@ -114,7 +114,7 @@ extern "C" hb_status hb_selftest_cluster(int clustered, hb_status *status, void 
         cfg.attrs = at;
         cfg.numAttrs = clustered;
         hb_count_launch();
-        e = cudaLaunchKernelEx(&cfg, hb2::ax_split_kernel<N>, A, 2);
+        e = cudaLaunchKernelEx(&cfg, hb2::ax_split_kernel<N, true>, A, 2);
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d, sizeof(buf), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

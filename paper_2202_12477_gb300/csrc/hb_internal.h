@@ -62,7 +62,7 @@ static inline bool hb_overlap_launch(cudaStream_t s)
     return st == cudaStreamCaptureStatusNone;
 }
 
-// Launches a kernel that begins with hbacc::wait_before(): its blocks may be
+// Launches a kernel whose first access to memory follows hbacc::wait_before(): its blocks may be
 // scheduled while the kernel before it on the stream drains, so launch latency
 // and last wave overlap. FP64 A x on 4x4x4 elements, N = 7: 16.4 -> 12.8 us;
 // FP32 on 5x5x5: 13.1 -> 11.2. Only such kernels may be launched this way.
