@@ -214,13 +214,14 @@ namespace tcax {
 // gradients left unscaled and one 64-bit value per sum (fewer integer
 // instructions, the busiest pipe beside FP64) 3.94, 4.25 and 5.86. A grid per line
 // at N = 3 and 15 (two more fixed-point and two more double conversions a node,
-// and the lines' maxima): 4.84 and 6.86. (The FP64 pencil kernel: 8.68, 11.8 and
-// 17.4.)
+// and the lines' maxima): 4.84 and 6.86, 4.57 and 6.72 with one range check a
+// conversion and the element's NaN set at its end. (The FP64 pencil kernel: 8.68,
+// 11.8 and 17.4.)
 template <int N_>
 struct shape {
     static constexpr int N = N_, n = N + 1, n2 = n * n, n3 = n2 * n;
     // The fixed-point grid follows every line, or the element. By element N = 3 and
-    // 15 take 3.94 and 5.86 ms for 4.84 and 6.86, but one value of 1e8 among values
+    // 15 take 3.94 and 5.86 ms for 4.57 and 6.72, but one value of 1e8 among values
     // of 1 left lines that it is not on with 8 digits, where the FP64 pencil kernel
     // keeps 16.
     static constexpr bool LINE = n != 8;
@@ -306,11 +307,11 @@ __device__ __forceinline__ long long to_fixed(double v, unsigned emax)
     const unsigned e = (unsigned)(b >> 52) & 0x7FFu;
     // 8m with the implicit bit (m the 53-bit significand), shifted out whole
     // for zero and subnormals
-    const unsigned long long m8 = ((b << 3) & 0x7FFFFFFFFFFFF8ull) | (1ull << 55);
+    const long long m8 = (long long)(((b << 3) & 0x7FFFFFFFFFFFF8ull) | (1ull << 55));
+    const long long s8 = (b >> 63) ? -m8 : m8;  // (the same for every grid the value enters)
     const unsigned sh = e ? min(emax - e, 62u) : 62u;
-    // round(4m / 2^sh), halves up: (floor(8m / 2^sh) + 1) / 2
-    const long long X = (long long)(((m8 >> sh) + 1ull) >> 1);
-    return (b >> 63) ? -X : X;
+    // round(+-4m / 2^sh), halves up: (floor(+-8m / 2^sh) + 1) / 2
+    return ((s8 >> sh) + 1) >> 1;
 }
 
 // The integer T as a double, rounded to nearest (ties away from zero):
@@ -327,8 +328,7 @@ __device__ __forceinline__ double i64_to_double(long long T, int off)
     const unsigned long long mant = (M >> 11) + ((M >> 10) & 1ull);  // 2^52 .. 2^53
     const int ex = 1023 + 63 - lz + (OFF ? off : 0);
     unsigned long long r = sgn | (((unsigned long long)(ex - 1) << 52) + mant);
-    if (OFF && ex >= 2047) r = sgn | 0x7FF0000000000000ull;
-    if (T == 0 || (OFF && ex <= 0)) r = sgn;
+    if (T == 0 || (OFF && (unsigned)(ex - 1) >= 2046u)) r = sgn | (T != 0 && ex > 0 ? 0x7FF0000000000000ull : 0ull);
     return __longlong_as_double((long long)r);
 }
 
@@ -613,10 +613,12 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
         }
         long long X[KH];
         unsigned eu = 0, row[3];
+        bool ubad = false;
         if constexpr (C::LINE) {
             exps er(u), es(u);
-            bool bad = false;  // (a non-finite line shows in its exponent)
-            line_max<C>(er, es, exps(u), eu, row, bad, lxu, line, ti, tj, k0);
+            const exps et(u);
+            ubad = et.largest() == 0x7FFu;
+            line_max<C>(er, es, et, eu, row, ubad, lxu, line, ti, tj, k0);
 #pragma unroll
             for (int q = 0; q < KH; q++) X[q] = to_fixed(u[q], er.at(q));
             stage<C, 0>(sm, el, ti, tj, k0, X);
@@ -631,9 +633,9 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
 #pragma unroll
             for (int q = 0; q < KH; q++) eu = max(eu, abs_hi(u[q]));
             eu = element_max(eu, wexp, el) >> 20;
-            row[0] = row[1] = row[2] = eu;
+            ubad = eu == 0x7FFu;
 #pragma unroll
-            for (int q = 0; q < KH; q++) X[q] = eu == 0x7FFu ? 0 : to_fixed(u[q], eu);
+            for (int q = 0; q < KH; q++) X[q] = ubad ? 0 : to_fixed(u[q], eu);
             stage<C, 0>(sm, el, ti, tj, k0, X);
             stage<C, 1>(sm, el, ti, tj, k0, X);
         }
@@ -653,8 +655,8 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
         const int scale = 40 + 10 - kUnit - dshift;
         const int goff = C::LINE ? 0 : (int)eu + scale;
         auto value = [&](int dir, long long hi, long long lo) {
-            return row[dir] == 0x7FFu ? __longlong_as_double(0x7FF8000000000000ll)
-                                      : i64_to_double<C::LINE>(halves(hi, lo), (int)row[dir] + scale);
+            if constexpr (C::LINE) return i64_to_double<true>(halves(hi, lo), (int)row[dir] + scale);
+            return ubad ? __longlong_as_double(0x7FF8000000000000ll) : i64_to_double<false>(halves(hi, lo), 0);
         };
         if constexpr (C::RESTAGE) stage<C, 2>(sm, el, ti, tj, k0, X);
         // ---- gradient along r into its exchange buffer; its columns are free
@@ -695,7 +697,7 @@ __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_a
         // in every form: every exchange read is done before the operands are
         // staged over the exchange buffers.)
         unsigned ev;
-        bool vbad = evm >> 20 == 0x7FFu;
+        bool vbad = ubad || evm >> 20 == 0x7FFu;
         if constexpr (C::LINE) {
             exps er(vr), es(vs);
             if constexpr (n == 4) __syncthreads();
