@@ -527,8 +527,8 @@ __device__ __forceinline__ void line_max(exps &er, exps &es, const exps &t, unsi
 // (gradients to the exchange buffers, or the exact sums of D^T), start the t
 // chain into r's columns, read s out meanwhile, then t. The six metric factors
 // are prefetched into L2 at the tile's start and loaded at the metric step,
-// not held in registers. What bounds it (ncu, N = 3 / 7 / 15): the integer pipe 63 /
-// 53 / 43 %, the FP64 pipe 56 / 58 / 42 %, issue 53 / 50 / 37 % of the time; DRAM at
+// not held in registers. What bounds it (ncu, N = 3 / 7 / 15): the integer pipe 61 /
+// 53 / 41 %, the FP64 pipe 59 / 58 / 43 %, issue 52 / 50 / 36 % of the time; DRAM at
 // most a quarter of its rate.
 template <class C, bool SP>
 __global__ void __launch_bounds__(C::THREADS, C::BLOCKS) ax_tc_kernel(const tc_args A)
